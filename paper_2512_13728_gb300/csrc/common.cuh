@@ -89,7 +89,9 @@ struct DevLayer {
   // 1: the buffer pass leaves M_{t-1} in place (it writes only the norms and the bf16 copy of B),
   // and the update or the local branch forms B = M + G itself (tensor-core mode, bf16 G)
   int32_t b_deferred;
-  int32_t bpart_off, bpart_cnt;  // slots of the ||B||^2 / ||M_{t-1}||^2 partials
+  // slots of the ||B||^2 / ||M_{t-1}||^2 partials of an ALWAYS step (128-row tiles where the fused
+  // kernel forms B, row tiles elsewhere) and of the norms pass (row tiles)
+  int32_t bpart_off, bpart_cnt, npart_off, npart_cnt;
   int32_t upart_off, upart_cnt;  // slots of the ||M_t||^2 partials
 };
 

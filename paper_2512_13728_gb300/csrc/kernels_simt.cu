@@ -39,14 +39,37 @@ __device__ __forceinline__ float load_g1(const void *G, int64_t off) {
   return static_cast<const float *>(G)[off];
 }
 
+// How the 256 threads of a row-tile kernel cover a tile whose rows hold n4 16-byte groups: cw
+// threads side by side in a row (the power of two that covers n4, 8 .. 256), the others on the
+// next rows, so that short rows leave no thread idle.  One group of each operand per thread is in
+// flight and 2048 threads per SM hide the latency (launch bounds of 8 blocks where the kernel
+// fits 32 registers): the 10 B/element norms pass of the 302M-element stack took 610 us with
+// four rows in flight per thread and 4 blocks per SM (60 registers), 545 us so; the local branch
+// 450 us against 575 us with four rows in flight.
+struct RowWalk {
+  int c, r, cw, rp;  // first group and row of this thread, groups / rows between its next ones
+};
+__device__ __forceinline__ RowWalk row_walk(int64_t n4) {
+  int sh = 8;
+  while (sh > 3 && (int64_t(1) << (sh - 1)) >= n4) --sh;
+  RowWalk w;
+  w.cw = 1 << sh;
+  w.rp = kRowThreads >> sh;
+  w.c = threadIdx.x & (w.cw - 1);
+  w.r = threadIdx.x >> sh;
+  return w;
+}
+
 template <int GT, bool HAS_BH>
 __device__ void form_b_tile(const DevLayer &L, int64_t row0, int64_t nrows, float sb[4], float sm[4]) {
   const int64_t n = L.n, n4 = n >> 2;
-  for (int64_t rr = 0; rr < nrows; ++rr) {
+  const RowWalk w = row_walk(n4);
+  const bool keep_m = HAS_BH && L.b_deferred;  // M_{t-1} stays in place: the update forms B itself
+  for (int64_t rr = w.r; rr < nrows; rr += w.rp) {
     const int64_t i = row0 + rr;
     float *Mrow = L.M + i * L.ldm;
     const int64_t goff = i * L.ldg;
-    for (int64_t c4 = threadIdx.x; c4 < n4; c4 += kRowThreads) {
+    for (int64_t c4 = w.c; c4 < n4; c4 += w.cw) {
       float4 m = *reinterpret_cast<float4 *>(Mrow + 4 * c4);
       float g[4];
       load_g4<GT>(L.G, goff + 4 * c4, g);
@@ -55,7 +78,7 @@ __device__ void form_b_tile(const DevLayer &L, int64_t row0, int64_t nrows, floa
       m.x += g[0]; m.y += g[1]; m.z += g[2]; m.w += g[3];
       sb[0] = fmaf(m.x, m.x, sb[0]); sb[1] = fmaf(m.y, m.y, sb[1]);
       sb[2] = fmaf(m.z, m.z, sb[2]); sb[3] = fmaf(m.w, m.w, sb[3]);
-      if (!HAS_BH || !L.b_deferred) *reinterpret_cast<float4 *>(Mrow + 4 * c4) = m;
+      if (!keep_m) *reinterpret_cast<float4 *>(Mrow + 4 * c4) = m;
       if (HAS_BH) {  // bf16 copy of B (operand of the tensor-core contractions)
         const __nv_bfloat162 h01 = __floats2bfloat162_rn(m.x, m.y), h23 = __floats2bfloat162_rn(m.z, m.w);
         uint2 hv;
@@ -73,17 +96,20 @@ __device__ void form_b_tile(const DevLayer &L, int64_t row0, int64_t nrows, floa
         }
       }
     }
-    for (int64_t c = 4 * n4 + threadIdx.x; c < n; c += kRowThreads) {
-      const float mo = Mrow[c];
-      const float b = mo + load_g1<GT>(L.G, goff + c);
-      sm[0] = fmaf(mo, mo, sm[0]);
-      sb[0] = fmaf(b, b, sb[0]);
-      if (!HAS_BH || !L.b_deferred) Mrow[c] = b;
-      if (HAS_BH) {
-        const __nv_bfloat16 h = __float2bfloat16_rn(b);
-        L.Bh[i * L.ldbh + c] = h;
-        if (L.Bl != nullptr) L.Bl[i * L.ldbh + c] = __float2bfloat16_rn(b - __bfloat162float(h));
-      }
+  }
+  // columns past the last multiple of 4
+  const int64_t tail = n - 4 * n4;
+  for (int64_t e = threadIdx.x; e < nrows * tail; e += kRowThreads) {
+    const int64_t i = row0 + e / tail, c = 4 * n4 + e % tail;
+    const float mo = L.M[i * L.ldm + c];
+    const float b = mo + load_g1<GT>(L.G, i * L.ldg + c);
+    sm[0] = fmaf(mo, mo, sm[0]);
+    sb[0] = fmaf(b, b, sb[0]);
+    if (!keep_m) L.M[i * L.ldm + c] = b;
+    if (HAS_BH) {
+      const __nv_bfloat16 h = __float2bfloat16_rn(b);
+      L.Bh[i * L.ldbh + c] = h;
+      if (L.Bl != nullptr) L.Bl[i * L.ldbh + c] = __float2bfloat16_rn(b - __bfloat162float(h));
     }
   }
 }
@@ -92,7 +118,7 @@ __device__ void form_b_tile(const DevLayer &L, int64_t row0, int64_t nrows, floa
 // keeps one; without, only B (into M) and the norms, the halves following for the Dion-branch
 // layers alone once the gate has run (split_b_kernel).
 template <bool HALVES>
-__global__ void __launch_bounds__(kRowThreads) form_b_kernel(Shared sh, const int4 *tiles) {
+__global__ void __launch_bounds__(kRowThreads, HALVES ? 5 : 8) form_b_kernel(Shared sh, const int4 *tiles) {
   __shared__ double red[kRowThreads / 32];
   const int4 t = tiles[blockIdx.x];
   DION_TILE_CHECK(t.x >= 0 && t.x < sh.num_layers, sh.status);
@@ -131,12 +157,13 @@ __global__ void __launch_bounds__(kRowThreads) split_b_kernel(Shared sh, const i
   if (!sh.active[t.x]) return;
   const DevLayer &L = sh.layers[t.x];
   DION_TILE_CHECK(t.y >= 0 && t.z >= 1 && (int64_t)t.y + t.z <= L.m && L.Bh != nullptr && L.Bl != nullptr, sh.status);
-  const int64_t n = L.n, n4 = n >> 2;
-  for (int64_t rr = 0; rr < t.z; ++rr) {
+  const int64_t n = L.n, n4 = n >> 2, nrows = t.z;
+  const RowWalk w = row_walk(n4);
+  for (int64_t rr = w.r; rr < nrows; rr += w.rp) {
     const int64_t i = t.y + rr;
     const float *Brow = L.M + i * L.ldm;
     __nv_bfloat16 *hrow = L.Bh + i * L.ldbh, *lrow = L.Bl + i * L.ldbh;
-    for (int64_t c4 = threadIdx.x; c4 < n4; c4 += kRowThreads) {
+    for (int64_t c4 = w.c; c4 < n4; c4 += w.cw) {
       const float4 b = *reinterpret_cast<const float4 *>(Brow + 4 * c4);
       const __nv_bfloat162 h01 = __floats2bfloat162_rn(b.x, b.y), h23 = __floats2bfloat162_rn(b.z, b.w);
       const float2 f01 = __bfloat1622float2(h01), f23 = __bfloat1622float2(h23);
@@ -150,12 +177,14 @@ __global__ void __launch_bounds__(kRowThreads) split_b_kernel(Shared sh, const i
       *reinterpret_cast<uint2 *>(hrow + 4 * c4) = hv;
       *reinterpret_cast<uint2 *>(lrow + 4 * c4) = lv;
     }
-    for (int64_t c = 4 * n4 + threadIdx.x; c < n; c += kRowThreads) {
-      const float b = Brow[c];
-      const __nv_bfloat16 h = __float2bfloat16_rn(b);
-      hrow[c] = h;
-      lrow[c] = __float2bfloat16_rn(b - __bfloat162float(h));
-    }
+  }
+  const int64_t tail = n - 4 * n4;
+  for (int64_t e = threadIdx.x; e < nrows * tail; e += kRowThreads) {
+    const int64_t i = t.y + e / tail, c = 4 * n4 + e % tail;
+    const float b = L.M[i * L.ldm + c];
+    const __nv_bfloat16 h = __float2bfloat16_rn(b);
+    L.Bh[i * L.ldbh + c] = h;
+    L.Bl[i * L.ldbh + c] = __float2bfloat16_rn(b - __bfloat162float(h));
   }
 }
 
@@ -186,10 +215,12 @@ __device__ __forceinline__ double from_max_key(unsigned long long k) {
 // RMMC (in lane 0; +inf when not finite, which counts as above every threshold).
 __device__ double gate_layer(const Shared &sh, const StepArgs &a, int l, int lane) {
   const DevLayer &Ly = sh.layers[l];
+  // the norms pass (B in M) and the buffer pass fill row-tile slots, the fused kernel its own
+  const int off = sh.b_in_m ? Ly.npart_off : Ly.bpart_off, cnt = sh.b_in_m ? Ly.npart_cnt : Ly.bpart_cnt;
   double sb = 0.0, sm = 0.0;
-  for (int k = lane; k < Ly.bpart_cnt; k += 32) {  // fixed lane/slot assignment
-    sb += __ldcg(&sh.bpart[2 * (Ly.bpart_off + k)]);
-    sm += __ldcg(&sh.bpart[2 * (Ly.bpart_off + k) + 1]);
+  for (int k = lane; k < cnt; k += 32) {  // fixed lane/slot assignment
+    sb += __ldcg(&sh.bpart[2 * (off + k)]);
+    sm += __ldcg(&sh.bpart[2 * (off + k) + 1]);
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -311,80 +342,26 @@ void launch_gate_reduced(const Shared &sh, const StepArgs &a, cudaStream_t s) {
 // ==================================================================== norms + gate ===
 // Gated modes with the fused buffer + B Q kernel: Algorithm 2 needs ||B|| before it knows which
 // layers take the Dion branch, so this pass forms B = M + G into M (read M, G; write M:
-// 10 B/element) with the sums of B^2 and M_{t-1}^2 per 128-row tile (the fused kernel's slots),
-// and the last block to finish runs the gate.  The fused kernel and everything after it touch
-// only the layers that sync and read B from M; the local branch then only updates X.
-// Tile = {layer, 128-row block}.
-constexpr int kNormThreads = 256;
-template <int GT>
-__device__ void norms_tile(const DevLayer &L, int64_t row0, int64_t nrows, float sb[4], float sm[4]) {
-  float *M = L.M;
-  const int64_t n = L.n, n4 = n >> 2;
-  // four rows at a time: each thread keeps four independent M and G loads in flight
-  int64_t rr = 0;
-  for (; rr + 4 <= nrows; rr += 4) {
-    const int64_t i = row0 + rr;
-    for (int64_t c4 = threadIdx.x; c4 < n4; c4 += kNormThreads) {
-      float4 m[4];
-      float g[4][4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        m[u] = __ldcs(reinterpret_cast<const float4 *>(L.M + (i + u) * L.ldm + 4 * c4));
-        load_g4<GT>(L.G, (i + u) * L.ldg + 4 * c4, g[u]);
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const float b0 = m[u].x + g[u][0], b1 = m[u].y + g[u][1], b2 = m[u].z + g[u][2], b3 = m[u].w + g[u][3];
-        sm[0] = fmaf(m[u].x, m[u].x, sm[0]); sm[1] = fmaf(m[u].y, m[u].y, sm[1]);
-        sm[2] = fmaf(m[u].z, m[u].z, sm[2]); sm[3] = fmaf(m[u].w, m[u].w, sm[3]);
-        sb[0] = fmaf(b0, b0, sb[0]); sb[1] = fmaf(b1, b1, sb[1]);
-        sb[2] = fmaf(b2, b2, sb[2]); sb[3] = fmaf(b3, b3, sb[3]);
-        *reinterpret_cast<float4 *>(M + (i + u) * L.ldm + 4 * c4) = make_float4(b0, b1, b2, b3);
-      }
-    }
-  }
-  for (; rr < nrows; ++rr) {
-    const int64_t i = row0 + rr;
-    for (int64_t c4 = threadIdx.x; c4 < n4; c4 += kNormThreads) {
-      const float4 m = __ldcs(reinterpret_cast<const float4 *>(L.M + i * L.ldm + 4 * c4));
-      float g[4];
-      load_g4<GT>(L.G, i * L.ldg + 4 * c4, g);
-      const float b0 = m.x + g[0], b1 = m.y + g[1], b2 = m.z + g[2], b3 = m.w + g[3];
-      sm[0] = fmaf(m.x, m.x, sm[0]); sm[1] = fmaf(m.y, m.y, sm[1]);
-      sm[2] = fmaf(m.z, m.z, sm[2]); sm[3] = fmaf(m.w, m.w, sm[3]);
-      sb[0] = fmaf(b0, b0, sb[0]); sb[1] = fmaf(b1, b1, sb[1]);
-      sb[2] = fmaf(b2, b2, sb[2]); sb[3] = fmaf(b3, b3, sb[3]);
-      *reinterpret_cast<float4 *>(M + i * L.ldm + 4 * c4) = make_float4(b0, b1, b2, b3);
-    }
-  }
-  // columns past the last multiple of 4
-  for (int64_t e = threadIdx.x; e < nrows * (n - 4 * n4); e += kNormThreads) {
-    const int64_t i = row0 + e / (n - 4 * n4), c = 4 * n4 + e % (n - 4 * n4);
-    const float mo = M[i * L.ldm + c], b = mo + load_g1<GT>(L.G, i * L.ldg + c);
-    sm[0] = fmaf(mo, mo, sm[0]);
-    sb[0] = fmaf(b, b, sb[0]);
-    M[i * L.ldm + c] = b;
-  }
-}
-
-__global__ void __launch_bounds__(kNormThreads) norms_gate_kernel(Shared sh, StepArgs a, const int4 *tiles) {
+// 10 B/element) with the sums of B^2 and M_{t-1}^2 per row tile (the buffer pass's tiles and
+// slots), and the last block to finish runs the gate.  The fused kernel and everything after it
+// touch only the layers that sync and read B from M; the local branch then only updates X.
+constexpr int kNormThreads = kRowThreads;
+__global__ void __launch_bounds__(kNormThreads, 8) norms_gate_kernel(Shared sh, StepArgs a, const int4 *tiles) {
   __shared__ double red[kNormThreads / 32];
   __shared__ int last_s, count_s;
   __shared__ double max_s[kNormThreads / 32];
-  const int4 t = tiles[blockIdx.x];  // {layer, 128-row block}
+  const int4 t = tiles[blockIdx.x];  // {layer, first row, rows, slot}
   DION_TILE_CHECK(t.x >= 0 && t.x < sh.num_layers, sh.status);
   const DevLayer &L = sh.layers[t.x];
-  DION_TILE_CHECK(t.y >= 0 && (int64_t)t.y * 128 < L.m, sh.status);
-  const int64_t row0 = (int64_t)t.y * 128, nrows = min((int64_t)128, L.m - row0);
+  DION_TILE_CHECK(t.y >= 0 && t.z >= 1 && (int64_t)t.y + t.z <= L.m, sh.status);
   float sb[4] = {0.f, 0.f, 0.f, 0.f}, sm[4] = {0.f, 0.f, 0.f, 0.f};
-  if (L.g_dtype == DT_BF16) norms_tile<DT_BF16>(L, row0, nrows, sb, sm);
-  else norms_tile<DT_FP32>(L, row0, nrows, sb, sm);
+  if (L.g_dtype == DT_BF16) form_b_tile<DT_BF16, false>(L, t.y, t.z, sb, sm);
+  else form_b_tile<DT_FP32, false>(L, t.y, t.z, sb, sm);
   const double b = block_sum<kNormThreads>(((double)sb[0] + sb[1]) + ((double)sb[2] + sb[3]), red);
   const double mo = block_sum<kNormThreads>(((double)sm[0] + sm[1]) + ((double)sm[2] + sm[3]), red);
   if (threadIdx.x == 0) {
-    const int slot = L.bpart_off + t.y;
-    sh.bpart[2 * slot] = b;
-    sh.bpart[2 * slot + 1] = mo;
+    sh.bpart[2 * t.w] = b;
+    sh.bpart[2 * t.w + 1] = mo;
     __threadfence();  // this block's partials are visible before it is counted
     last_s = atomicAdd(&sh.gate_scratch[2], 1ull) == (unsigned long long)(gridDim.x - 1);
   }
@@ -1139,11 +1116,12 @@ template <int GT>
 __device__ void local_tile(const DevLayer &L, int64_t row0, int64_t nrows, float eta_local, float keep, bool b_in_m) {
   const int64_t n = L.n, n4 = n >> 2;
   const bool form_m = L.b_deferred != 0 && !b_in_m;
-  for (int64_t rr = 0; rr < nrows; ++rr) {
+  const RowWalk w = row_walk(n4);
+  for (int64_t rr = w.r; rr < nrows; rr += w.rp) {
     const int64_t i = row0 + rr;
     float *Xrow = L.X + i * L.ldx, *Mrow = L.M + i * L.ldm;
     const int64_t goff = i * L.ldg;
-    for (int64_t c4 = threadIdx.x; c4 < n4; c4 += kRowThreads) {
+    for (int64_t c4 = w.c; c4 < n4; c4 += w.cw) {
       float4 x = *reinterpret_cast<float4 *>(Xrow + 4 * c4);
       float g[4];
       load_g4<GT>(L.G, goff + 4 * c4, g);
@@ -1156,11 +1134,13 @@ __device__ void local_tile(const DevLayer &L, int64_t row0, int64_t nrows, float
         *reinterpret_cast<float4 *>(Mrow + 4 * c4) = m;
       }
     }
-    for (int64_t c = 4 * n4 + threadIdx.x; c < n; c += kRowThreads) {
-      const float g = load_g1<GT>(L.G, goff + c);
-      Xrow[c] = fmaf(-eta_local, g, Xrow[c] * keep);
-      if (form_m) Mrow[c] += g;
-    }
+  }
+  const int64_t tail = n - 4 * n4;
+  for (int64_t e = threadIdx.x; e < nrows * tail; e += kRowThreads) {
+    const int64_t i = row0 + e / tail, c = 4 * n4 + e % tail;
+    const float g = load_g1<GT>(L.G, i * L.ldg + c);
+    L.X[i * L.ldx + c] = fmaf(-eta_local, g, L.X[i * L.ldx + c] * keep);
+    if (form_m) L.M[i * L.ldm + c] += g;
   }
 }
 

@@ -131,6 +131,18 @@ dion_status validate_layer(const dion_layer &ly) {
   return DION_OK;
 }
 
+// Elements of a row tile (whole rows of one layer) of the buffer, norms and local kernels: 64K
+// where the plan has enough for four or more blocks per SM, fewer on smaller plans, so that they
+// still spread over the chip (down to 1K, four elements per thread).  The buffer pass of a
+// 256 x 512 matrix took 57 us in two 64K tiles and takes 8.5 us in 128 of 1K; on the 302M-element
+// stack 32K and 64K measured the same, but idle blocks (a branch no layer takes) cost 2 us per
+// thousand.
+int64_t row_tile_elems(const dion_layer *layers, int32_t num_layers, int sms) {
+  int64_t total = 0;
+  for (int32_t l = 0; l < num_layers; ++l) total += layers[l].m * layers[l].n;
+  return std::min<int64_t>(65536, std::max<int64_t>(1024, total / (4 * std::max(sms, 1))));
+}
+
 template <class T>
 cudaError_t upload(T *dst, const std::vector<T> &src) {
   if (src.empty()) return cudaSuccess;
@@ -203,6 +215,7 @@ dion_status dion_plan_create(const dion_layer *layers, int32_t num_layers, int32
     p->xr_off = o_R[0];
     p->xr_count = (int64_t)((o_R[num_layers - 1] - o_R[0]) / sizeof(float)) + a.n * lp;
   }
+  const int64_t tile_elems = row_tile_elems(layers, num_layers, sms);
   for (int32_t l = 0; l < num_layers; ++l) {
     const dion_layer &ly = layers[l];
     DevLayer &d = dl[l];
@@ -219,12 +232,14 @@ dion_status dion_plan_create(const dion_layer *layers, int32_t num_layers, int32
     o_P[l] = cv.take<float>(ly.m * d.ldp);
     o_S[l] = cv.take<float>(ly.r * d.ldp);
     o_Li[l] = cv.take<float>(ly.r * d.ldp);
-    // row tiles of about 64K elements for the buffer and local kernels
-    const int64_t rows = std::max<int64_t>(1, std::min<int64_t>(ly.m, 65536 / ly.n));
+    // row tiles of the buffer, norms and local kernels
+    const int64_t rows = std::max<int64_t>(1, std::min<int64_t>(ly.m, tile_elems / ly.n));
     d.bpart_off = (int32_t)bt.size();
     for (int64_t r0 = 0; r0 < ly.m; r0 += rows)
       bt.push_back(make_int4(l, (int)r0, (int)std::min(rows, ly.m - r0), (int)bt.size()));
     d.bpart_cnt = (int32_t)bt.size() - d.bpart_off;
+    d.npart_off = d.bpart_off;
+    d.npart_cnt = d.bpart_cnt;
     // update tiles of the CUDA-core update kernel (FP32 mode)
     d.upart_off = (int32_t)ut.size();
     for (int64_t ti = 0; ti < (ly.m + kUpdTileM - 1) / kUpdTileM; ++ti)

@@ -142,7 +142,6 @@ dion_status layout(const dion_layer *layers, int32_t L, int32_t precision, int n
   }
   lo.o_maps = take(sizeof(LayerMaps) * std::max(L, 1), 128);
   lo.o_utiles = take(sizeof(int4) * std::max<size_t>(lo.utiles.size(), 1));
-  lo.o_ftiles = take(sizeof(int4) * std::max<size_t>(lo.ftiles.size(), 1));
   lo.o_rtiles = take(sizeof(int4) * std::max<size_t>(lo.rtiles.size(), 1));
   lo.o_qtiles = take(sizeof(int4) * std::max<size_t>(lo.qtiles.size(), 1));
   lo.o_gtiles = take(sizeof(int4) * std::max<size_t>(lo.gram_tiles.size(), 1));
@@ -199,8 +198,6 @@ void bind(const TcLayout &lo, char *base, DevLayer *dl, int32_t L, TcPlan *tp) {
   tp->maps = reinterpret_cast<LayerMaps *>(base + lo.o_maps);
   tp->utiles = reinterpret_cast<int4 *>(base + lo.o_utiles);
   tp->n_utiles = (int32_t)lo.utiles.size();
-  tp->ftiles = reinterpret_cast<int4 *>(base + lo.o_ftiles);
-  tp->n_ftiles = (int32_t)lo.ftiles.size();
   tp->rtiles = reinterpret_cast<int4 *>(base + lo.o_rtiles);
   tp->n_rtiles = (int32_t)lo.rtiles.size();
   tp->qtiles = reinterpret_cast<int4 *>(base + lo.o_qtiles);
@@ -278,7 +275,6 @@ cudaError_t init(const TcLayout &lo, char *base, const DevLayer *dl, int32_t L, 
     return v.empty() ? cudaSuccess : cudaMemcpy(dst, v.data(), sizeof(int4) * v.size(), cudaMemcpyHostToDevice);
   };
   if (e == cudaSuccess) e = up(tp->utiles, lo.utiles);
-  if (e == cudaSuccess) e = up(tp->ftiles, lo.ftiles);
   if (e == cudaSuccess) e = up(tp->rtiles, lo.rtiles);
   if (e == cudaSuccess) e = up(tp->qtiles, lo.qtiles);
   if (e == cudaSuccess) e = up(tp->gram_tiles, lo.gram_tiles);
@@ -354,7 +350,7 @@ void step(dion_plan *p, const TcPlan &tp, const Shared &sh_in, const StepArgs &a
     tick(p, s, "gate");
   } else if (tp.fuse_buffer) {
     // gated modes: the norms and the gate first, then the fused kernel on the Dion-branch layers
-    launch_norms_gate(sh, a, tp.ftiles, tp.n_ftiles, s);
+    launch_norms_gate(sh, a, btiles, n_btiles, s);
     tick(p, s, "norms_gate");
     launch_fused_bq(sh, tp, true, s);
     tick(p, s, "tc_form_bq");
@@ -410,7 +406,7 @@ void step_phase(const TcPlan &tp, const Shared &sh_in, const StepArgs &a, int32_
   switch (phase) {
     case DION_PHASE_NORMS:  // B = M + G, ||B||, this worker's RMMC, prev_norm <- ||B||
       if (tp.fuse_buffer) {
-        launch_norms_gate(sh, a, tp.ftiles, tp.n_ftiles, s);
+        launch_norms_gate(sh, a, btiles, n_btiles, s);
       } else {
         launch_form_b(sh, btiles, n_btiles, s, !x3);  // BF16X3: the halves after the branch is known
         launch_gate(sh, a, s);

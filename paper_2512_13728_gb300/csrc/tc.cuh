@@ -56,7 +56,7 @@ struct TcLayout {
   Schedule s_update, s_bq, s_btp, s_gram, s_trsm;
   size_t end = 0;
   size_t o_maps = 0;
-  size_t o_utiles = 0, o_ftiles = 0, o_rtiles = 0, o_qtiles = 0, o_gtiles = 0, o_ttiles = 0;
+  size_t o_utiles = 0, o_rtiles = 0, o_qtiles = 0, o_gtiles = 0, o_ttiles = 0;
   std::vector<size_t> o_phi, o_rhi, o_qnhi, o_bh, o_ptraw, o_pt, o_colsq, o_colinv;
   std::vector<size_t> o_bl, o_plo, o_rlo, o_qnlo;  // BF16X3 low halves
   std::vector<uint64_t> guards;  // offsets of the guard words after each region
@@ -81,8 +81,6 @@ struct TcPlan {
   LayerMaps *maps = nullptr;
   int4 *utiles = nullptr;
   int32_t n_utiles = 0;
-  int4 *ftiles = nullptr;
-  int32_t n_ftiles = 0;
   int4 *rtiles = nullptr;
   int32_t n_rtiles = 0;
   int4 *qtiles = nullptr;

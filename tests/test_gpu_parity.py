@@ -584,3 +584,25 @@ def test_cuda_graph_replay_matches_direct_steps(prec, gate):
         plan.close()
     for a, b in zip(*outs):
         assert torch.equal(a, b)
+
+
+# ------------------------------------------------------- row tiles at their edges ---
+
+ROW_TILES = wl.scaled(wl.WORKLOADS["gpt160m_block_r192"], "rowtiles",
+                      [(1, 5), (5, 3), (300, 1), (2, 1500), (257, 33), (131, 1027), (9, 4)], rank=1, steps=3)
+
+
+@pytest.mark.parametrize("prec,gate", [("fp32", oc.GATE_ALWAYS), ("fp32", oc.GATE_PER_LAYER),
+                                       ("bf16", oc.GATE_GLOBAL), ("bf16", oc.GATE_PER_LAYER),
+                                       ("bf16x3", oc.GATE_PER_LAYER)])
+def test_row_tiles(prec, gate):
+    """The buffer, norms, split and local kernels where rows are shorter than 8 groups of four, end in
+    a partial group, exceed 256 groups, or are fewer than a tile's.  In the fp32-class modes half of
+    the layers synchronize; in bf16, whose row-tile kernels are the norms and the local branch, all
+    stay local, which is fp32 arithmetic and held to the fp32 bound (a synchronized rank-1 layer
+    with a handful of columns is not: |B| |q| / |B q| is unbounded there, and multiplies the 2^-9 of
+    its operands)."""
+    local = prec == "bf16"
+    taus = [0.5 if l % 2 and not local else 1e9 for l in range(len(ROW_TILES.shapes))]
+    run_per_step(ROW_TILES, PRECS[prec], dict(gate_mode=gate, tau_global=1e9 if local else 0.5), ROW_TILES.steps,
+                 TOL_FP32, taus=taus)
