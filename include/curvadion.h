@@ -221,7 +221,9 @@ dion_status dion_get_device_status(dion_plan *plan, int32_t clear, int32_t *code
  * Errors: INVALID_ARG (NULL plan), CUDA. */
 dion_status dion_plan_refresh(dion_plan *plan, void *stream);
 
-/* Number of kernel launches one dion_step enqueues for this plan. */
+/* Number of kernel launches that the plan's last dion_step enqueued (before the first step, and
+ * for a plan that only steps with DION_GATE_ALWAYS: those of such a step).  The gated modes launch
+ * the norms pass and the local branch besides. */
 int32_t dion_step_launch_count(const dion_plan *plan);
 
 /* Per-launch timing with CUDA events (measurement support; not part of the paper's method).

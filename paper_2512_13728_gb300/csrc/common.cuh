@@ -122,8 +122,8 @@ struct Shared {
   double *norm_b;        // [L]
   int32_t *status;       // [1] first device error
   uint8_t *orth_shifted; // [L] 1 = a Cholesky pass of this step needed the shift (third pass runs)
-  // [kScratchSlots]: the gate's running max of RMMC (ordered key), its finished-block count, the
-  // norms pass's finished-block count, (written by the gate) the number of layers that take the
+  // [kScratchSlots]: the gate's running max of RMMC (ordered key), its finished-block count, a
+  // spare slot, (written by the gate) the number of layers that take the
   // Dion branch this step, which lets the later persistent kernels return at once when it is 0,
   // and (reset by the gate, counted by the Cholesky kernels) the layers that took the shifted
   // retry, which lets the third CholeskyQR pass return at once when it is 0
@@ -176,7 +176,7 @@ __device__ __forceinline__ double block_sum(double v, double *red /* >= THREADS/
 
 // ---------------------------------------------------------------- launch wrappers ---
 // CUDA-core (fp32) kernels, kernels_simt.cu
-void launch_form_b(const Shared &sh, const int4 *tiles, int32_t ntiles, cudaStream_t s, bool halves = true);
+void launch_form_b(const Shared &sh, const int4 *tiles, int32_t ntiles, cudaStream_t s, bool halves);
 void launch_split_b(const Shared &sh, const int4 *tiles, int32_t ntiles, bool needed, cudaStream_t s);
 void launch_gate(const Shared &sh, const StepArgs &a, cudaStream_t s);
 // the branch from RMMC values already in a.rmmc (reduced over data-parallel workers)
@@ -194,7 +194,6 @@ void launch_colnorm(const Shared &sh, const int4 *tiles, int32_t ntiles, float e
                     cudaStream_t s);
 void launch_update(const Shared &sh, const int4 *tiles, int32_t ntiles, float mu, float eta, float keep,
                    cudaStream_t s);
-void launch_norms_gate(const Shared &sh, const StepArgs &a, const int4 *tiles, int32_t ntiles, cudaStream_t s);
 void launch_local(const Shared &sh, const int4 *tiles, int32_t ntiles, float eta_local, float keep,
                   cudaStream_t s);
 void launch_finalize(const Shared &sh, const StepArgs &a, cudaStream_t s);

@@ -44,7 +44,7 @@ __device__ __forceinline__ float load_g1(const void *G, int64_t off) {
 // next rows, so that short rows leave no thread idle.  One group of each operand per thread is in
 // flight and 2048 threads per SM hide the latency (launch bounds of 8 blocks where the kernel
 // fits 32 registers): the 10 B/element norms pass of the 302M-element stack took 610 us with
-// four rows in flight per thread and 4 blocks per SM (60 registers), 545 us so; the local branch
+// four rows in flight per thread and 4 blocks per SM (60 registers), 463 us so; the local branch
 // 450 us against 575 us with four rows in flight.
 struct RowWalk {
   int c, r, cw, rp;  // first group and row of this thread, groups / rows between its next ones
@@ -116,10 +116,12 @@ __device__ void form_b_tile(const DevLayer &L, int64_t row0, int64_t nrows, floa
 
 // HALVES: also write the layer's bf16 copy of B (or, in BF16X3, its two halves) where the plan
 // keeps one; without, only B (into M) and the norms, the halves following for the Dion-branch
-// layers alone once the gate has run (split_b_kernel).
+// layers alone once the gate has run (split_b_kernel), or from the fused buffer + B Q kernel: in
+// the gated modes with bf16 G this is the norms pass (read M, G; write M: 10 B/element on every
+// layer), after which everything touches only the layers that sync and reads B from M.
 template <bool HALVES>
 __global__ void __launch_bounds__(kRowThreads, HALVES ? 5 : 8) form_b_kernel(Shared sh, const int4 *tiles) {
-  __shared__ double red[kRowThreads / 32];
+  __shared__ double red[2 * (kRowThreads / 32)];
   const int4 t = tiles[blockIdx.x];
   DION_TILE_CHECK(t.x >= 0 && t.x < sh.num_layers, sh.status);
   const DevLayer &L = sh.layers[t.x];
@@ -132,11 +134,23 @@ __global__ void __launch_bounds__(kRowThreads, HALVES ? 5 : 8) form_b_kernel(Sha
     if (L.g_dtype == DT_BF16) form_b_tile<DT_BF16, false>(L, t.y, t.z, sb, sm);
     else form_b_tile<DT_FP32, false>(L, t.y, t.z, sb, sm);
   }
-  const double b = block_sum<kRowThreads>(((double)sb[0] + sb[1]) + ((double)sb[2] + sb[3]), red);
-  const double mo = block_sum<kRowThreads>(((double)sm[0] + sm[1]) + ((double)sm[2] + sm[3]), red);
-  if (threadIdx.x == 0) {
-    sh.bpart[2 * t.w] = b;
-    sh.bpart[2 * t.w + 1] = mo;
+  // both sums in one fixed-order reduction (a barrier, after which all warps but the first leave)
+  double b = ((double)sb[0] + sb[1]) + ((double)sb[2] + sb[3]), mo = ((double)sm[0] + sm[1]) + ((double)sm[2] + sm[3]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    b += __shfl_xor_sync(0xffffffffu, b, o);
+    mo += __shfl_xor_sync(0xffffffffu, mo, o);
+  }
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (lane == 0) {
+    red[warp] = b;
+    red[kRowThreads / 32 + warp] = mo;
+  }
+  __syncthreads();
+  if (threadIdx.x < 2) {
+    double v = 0.0;
+    for (int w = 0; w < kRowThreads / 32; ++w) v += red[threadIdx.x * (kRowThreads / 32) + w];
+    sh.bpart[2 * t.w + threadIdx.x] = v;
   }
 }
 
@@ -337,58 +351,6 @@ __global__ void __launch_bounds__(kGateRedThreads) gate_reduced_kernel(Shared sh
 
 void launch_gate_reduced(const Shared &sh, const StepArgs &a, cudaStream_t s) {
   gate_reduced_kernel<<<1, kGateRedThreads, 0, s>>>(sh, a);
-}
-
-// ==================================================================== norms + gate ===
-// Gated modes with the fused buffer + B Q kernel: Algorithm 2 needs ||B|| before it knows which
-// layers take the Dion branch, so this pass forms B = M + G into M (read M, G; write M:
-// 10 B/element) with the sums of B^2 and M_{t-1}^2 per row tile (the buffer pass's tiles and
-// slots), and the last block to finish runs the gate.  The fused kernel and everything after it
-// touch only the layers that sync and read B from M; the local branch then only updates X.
-constexpr int kNormThreads = kRowThreads;
-__global__ void __launch_bounds__(kNormThreads, 8) norms_gate_kernel(Shared sh, StepArgs a, const int4 *tiles) {
-  __shared__ double red[kNormThreads / 32];
-  __shared__ int last_s, count_s;
-  __shared__ double max_s[kNormThreads / 32];
-  const int4 t = tiles[blockIdx.x];  // {layer, first row, rows, slot}
-  DION_TILE_CHECK(t.x >= 0 && t.x < sh.num_layers, sh.status);
-  const DevLayer &L = sh.layers[t.x];
-  DION_TILE_CHECK(t.y >= 0 && t.z >= 1 && (int64_t)t.y + t.z <= L.m, sh.status);
-  float sb[4] = {0.f, 0.f, 0.f, 0.f}, sm[4] = {0.f, 0.f, 0.f, 0.f};
-  if (L.g_dtype == DT_BF16) form_b_tile<DT_BF16, false>(L, t.y, t.z, sb, sm);
-  else form_b_tile<DT_FP32, false>(L, t.y, t.z, sb, sm);
-  const double b = block_sum<kNormThreads>(((double)sb[0] + sb[1]) + ((double)sb[2] + sb[3]), red);
-  const double mo = block_sum<kNormThreads>(((double)sm[0] + sm[1]) + ((double)sm[2] + sm[3]), red);
-  if (threadIdx.x == 0) {
-    sh.bpart[2 * t.w] = b;
-    sh.bpart[2 * t.w + 1] = mo;
-    __threadfence();  // this block's partials are visible before it is counted
-    last_s = atomicAdd(&sh.gate_scratch[2], 1ull) == (unsigned long long)(gridDim.x - 1);
-  }
-  __syncthreads();
-  if (!last_s) return;
-  __threadfence();
-  // the last block: Algorithm 2 for every layer, one warp per layer, and the maximum of RMMC
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  double mx = -1.0;
-  for (int l = warp; l < sh.num_layers; l += kNormThreads / 32) mx = fmax(mx, gate_layer(sh, a, l, lane));
-  if (lane == 0) max_s[warp] = mx;
-  __syncthreads();
-  __shared__ int gflag_s;
-  if (threadIdx.x == 0) {
-    double g = -1.0;
-    for (int w = 0; w < kNormThreads / 32; ++w) g = fmax(g, max_s[w]);
-    const int gf = (sh.num_layers > 0 && above(g, a.tau_global)) ? 1 : 0;
-    a.gflag[0] = (uint8_t)gf;
-    gflag_s = gf;
-    sh.gate_scratch[2] = 0ull;  // for the next step (kernel boundary orders it)
-  }
-  __syncthreads();
-  gate_finish(sh, a, gflag_s, &count_s);
-}
-
-void launch_norms_gate(const Shared &sh, const StepArgs &a, const int4 *tiles, int32_t ntiles, cudaStream_t s) {
-  if (ntiles > 0) norms_gate_kernel<<<ntiles, kNormThreads, 0, s>>>(sh, a, tiles);
 }
 
 // ==================================================================== grouped GEMM ===

@@ -33,7 +33,7 @@ struct dion_plan {
   int32_t n_gtiles[kSets] = {};
   size_t chol_smem = 0;
   tc::TcPlan tcp{};  // tensor-core path (BF16 / BF16X3)
-  int32_t launches_per_step = 0;
+  int32_t launches_per_step = 0;  // of the last step (before the first: of an ALWAYS step)
   // data-parallel phases (dion_step_phase): the exchange ranges (offsets into ws, fp32 counts)
   // and the phase the next call must run
   size_t xp_off = 0, xr_off = 0;
@@ -63,25 +63,27 @@ struct dion_plan {
 };
 
 namespace cd {
-// Called by the step sequences: records the event that closes launch `cursor` when timing is on.
+constexpr int32_t kMaxLaunches = 24;  // launches of the longest step
+// Called by the step sequences: counts the launch and, when timing is on, records the event that
+// closes it.
 void tick(dion_plan *p, cudaStream_t s, const char *name) {
-  if (p->timing_steps <= 0 || p->recorded >= p->timing_steps) return;
-  const int32_t per = p->launches_per_step + 1;
-  if (p->cursor < p->launches_per_step) {
-    if ((int32_t)p->names.size() < p->launches_per_step) p->names.resize(p->launches_per_step, "");
+  if (p->timing_steps > 0 && p->recorded < p->timing_steps && p->cursor < kMaxLaunches) {
+    if ((int32_t)p->names.size() < kMaxLaunches) p->names.resize(kMaxLaunches, "");
     p->names[p->cursor] = name;
-    cudaEventRecord(p->ev[(size_t)p->recorded * per + p->cursor + 1], s);
+    cudaEventRecord(p->ev[(size_t)p->recorded * (kMaxLaunches + 1) + p->cursor + 1], s);
   }
   ++p->cursor;
 }
 void tick_begin(dion_plan *p, cudaStream_t s) {
   p->cursor = 0;
   if (p->timing_steps <= 0 || p->recorded >= p->timing_steps) return;
-  cudaEventRecord(p->ev[(size_t)p->recorded * (p->launches_per_step + 1)], s);
+  cudaEventRecord(p->ev[(size_t)p->recorded * (kMaxLaunches + 1)], s);
 }
 void tick_end(dion_plan *p) {
-  if (p->timing_steps <= 0 || p->recorded >= p->timing_steps) return;
-  ++p->recorded;
+  // steps are averaged launch by launch: a gate mode with another sequence starts again
+  if (p->cursor != p->launches_per_step && p->recorded > 0) p->recorded = -1;
+  p->launches_per_step = p->cursor;
+  if (p->timing_steps > 0 && p->recorded < p->timing_steps) ++p->recorded;
 }
 }  // namespace cd
 
@@ -396,7 +398,7 @@ dion_status dion_plan_create(const dion_layer *layers, int32_t num_layers, int32
     delete p;
     return DION_ERR_CUDA;
   }
-  p->launches_per_step = (precision == DION_PREC_FP32) ? 17 : tc::launches_per_step(p->tcp);
+  p->launches_per_step = (precision == DION_PREC_FP32) ? 16 : tc::launches_per_step(p->tcp);
 #ifdef DION_DEBUG_CHECKS
   p->launches_per_step += 1;  // the guard check at the end of every step
 #endif
@@ -444,7 +446,7 @@ void enqueue_step(dion_plan *p, const Shared &sh, const tc::TcPlan &tcp, const d
   const StepArgs a = make_args(hp, prev_norm, rmmc_out, rmmc_eq1_out, sync_flags_out, global_flag_out);
   tick_begin(p, s);
   if (p->precision == DION_PREC_FP32) {
-    launch_form_b(sh, p->btiles, p->n_btiles, s);
+    launch_form_b(sh, p->btiles, p->n_btiles, s, false);
     tick(p, s, "form_b");
     launch_gate(sh, a, s);
     tick(p, s, "gate");
@@ -467,8 +469,10 @@ void enqueue_step(dion_plan *p, const Shared &sh, const tc::TcPlan &tcp, const d
     tick(p, s, "colnorm");
     launch_update(sh, p->utiles, p->n_utiles, a.mu, a.eta, a.keep_sync, s);  // M, X
     tick(p, s, "update");
-    launch_local(sh, p->btiles, p->n_btiles, a.eta_local, a.keep_local, s);  // local branch
-    tick(p, s, "local");
+    if (a.gate_mode != GATE_ALWAYS) {
+      launch_local(sh, p->btiles, p->n_btiles, a.eta_local, a.keep_local, s);  // local branch
+      tick(p, s, "local");
+    }
     launch_finalize(sh, a, s);                                      // Equation 1
     tick(p, s, "finalize");
   } else {
@@ -492,7 +496,7 @@ void enqueue_phase(dion_plan *p, const StepArgs &a, int32_t phase, cudaStream_t 
   }
   switch (phase) {
     case DION_PHASE_NORMS:  // B = M + G, ||B||, this worker's RMMC, prev_norm <- ||B||
-      launch_form_b(sh, p->btiles, p->n_btiles, s);
+      launch_form_b(sh, p->btiles, p->n_btiles, s, false);
       launch_gate(sh, a, s);
       break;
     case DION_PHASE_POWER:  // the branch from the reduced RMMC, then P = B Q on the Dion layers
@@ -764,7 +768,7 @@ dion_status dion_timing_enable(dion_plan *p, int32_t max_steps) {
   if (cudaDeviceSynchronize() != cudaSuccess) return DION_ERR_CUDA;
   free_events(p);
   if (max_steps == 0) return DION_OK;
-  const size_t count = (size_t)max_steps * (p->launches_per_step + 1);
+  const size_t count = (size_t)max_steps * (kMaxLaunches + 1);
   p->ev.resize(count);
   for (size_t i = 0; i < count; ++i) {
     if (cudaEventCreate(&p->ev[i]) != cudaSuccess) {
@@ -781,8 +785,8 @@ dion_status dion_timing_enable(dion_plan *p, int32_t max_steps) {
 dion_status dion_timing_read(dion_plan *p, int32_t cap, float *ms_out, const char **names_out, int32_t *count_out,
                              int32_t *steps_out) {
   if (!p || !count_out || !steps_out || (cap > 0 && (!ms_out || !names_out))) return DION_ERR_INVALID_ARG;
-  const int32_t per = p->launches_per_step + 1;
-  const int32_t n = std::min(cap, p->launches_per_step);
+  const int32_t per = kMaxLaunches + 1;
+  const int32_t n = std::min(std::min(cap, p->launches_per_step), kMaxLaunches);
   for (int32_t i = 0; i < n; ++i) {
     double tot = 0.0;
     for (int32_t st = 0; st < p->recorded; ++st) {

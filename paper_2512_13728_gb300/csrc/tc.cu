@@ -331,7 +331,7 @@ cudaError_t init(const TcLayout &lo, char *base, const DevLayer *dl, int32_t L, 
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   tp->num_sms = sms;
-  tp->launches = tp->fuse_buffer ? 17 : x3 ? 19 : 18;  // BF16X3: the split of B after the gate
+  tp->launches = tp->fuse_buffer ? 16 : x3 ? 18 : 17;  // of an ALWAYS step; BF16X3: the split of B
   return e;
 }
 
@@ -350,8 +350,10 @@ void step(dion_plan *p, const TcPlan &tp, const Shared &sh_in, const StepArgs &a
     tick(p, s, "gate");
   } else if (tp.fuse_buffer) {
     // gated modes: the norms and the gate first, then the fused kernel on the Dion-branch layers
-    launch_norms_gate(sh, a, btiles, n_btiles, s);
+    launch_form_b(sh, btiles, n_btiles, s, false);
     tick(p, s, "norms_gate");
+    launch_gate(sh, a, s);
+    tick(p, s, "gate");
     launch_fused_bq(sh, tp, true, s);
     tick(p, s, "tc_form_bq");
   } else {
@@ -390,8 +392,10 @@ void step(dion_plan *p, const TcPlan &tp, const Shared &sh_in, const StepArgs &a
   tick(p, s, "colnorm_scale");
   launch_update(sh, tp, a.mu, a.eta, a.keep_sync, s);  // M_t, X_t (error feedback, update)
   tick(p, s, "tc_update");
-  launch_local(sh, btiles, n_btiles, a.eta_local, a.keep_local, s);
-  tick(p, s, "local");
+  if (a.gate_mode != GATE_ALWAYS) {
+    launch_local(sh, btiles, n_btiles, a.eta_local, a.keep_local, s);
+    tick(p, s, "local");
+  }
   launch_finalize(sh, a, s);
   tick(p, s, "finalize");
 }
@@ -405,12 +409,9 @@ void step_phase(const TcPlan &tp, const Shared &sh_in, const StepArgs &a, int32_
   const bool x3 = tp.precision == DION_PREC_BF16X3;
   switch (phase) {
     case DION_PHASE_NORMS:  // B = M + G, ||B||, this worker's RMMC, prev_norm <- ||B||
-      if (tp.fuse_buffer) {
-        launch_norms_gate(sh, a, btiles, n_btiles, s);
-      } else {
-        launch_form_b(sh, btiles, n_btiles, s, !x3);  // BF16X3: the halves after the branch is known
-        launch_gate(sh, a, s);
-      }
+      // the bf16 copy of B: with bf16 G from the fused kernel, in BF16X3 after the branch is known
+      launch_form_b(sh, btiles, n_btiles, s, !tp.fuse_buffer && !x3);
+      launch_gate(sh, a, s);
       break;
     case DION_PHASE_POWER:  // the branch from the reduced RMMC, then P = B Q on the Dion layers
       launch_gate_reduced(sh, a, s);
