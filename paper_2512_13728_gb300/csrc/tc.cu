@@ -79,6 +79,10 @@ dion_status layout(const dion_layer *layers, int32_t L, int32_t precision, int n
   lo.o_plo.assign(L, 0);
   lo.o_rlo.assign(L, 0);
   lo.o_qnlo.assign(L, 0);
+  // entries of a row tile of Q: 16K, fewer where the plan has less than four such tiles per SM
+  int64_t nr = 0;
+  for (int32_t l = 0; l < L; ++l) nr += layers[l].n * layers[l].r;
+  const int64_t qelems = std::min<int64_t>(16384, std::max<int64_t>(1024, nr / (4 * std::max(num_sms, 1))));
   for (int32_t l = 0; l < L; ++l) {
     const dion_layer &ly = layers[l];
     const int64_t ldp = (ly.r + 7) / 8 * 8, ldbh = (ly.n + 7) / 8 * 8;
@@ -103,7 +107,7 @@ dion_status layout(const dion_layer *layers, int32_t L, int32_t precision, int n
     for (int64_t mb = 0; mb < (ly.m + 127) / 128; ++mb)
       for (int64_t nb = 0; nb < (ly.n + 127) / 128; ++nb)
         lo.utiles.push_back(make_int4(l, (int)mb, (int)nb, (int)lo.utiles.size()));
-    const int64_t qrow = std::max<int64_t>(1, std::min<int64_t>(ly.n, 16384 / ly.r));
+    const int64_t qrow = std::max<int64_t>(1, std::min<int64_t>(ly.n, qelems / ly.r));
     for (int64_t r0 = 0; r0 < ly.n; r0 += qrow)
       lo.qtiles.push_back(make_int4(l, (int)r0, (int)std::min(qrow, ly.n - r0), 0));
     for (int64_t mb = 0; mb < (ly.m + 127) / 128; ++mb) lo.ftiles.push_back(make_int4(l, (int)mb, 0, 0));

@@ -860,57 +860,57 @@ __global__ void __launch_bounds__(256) colnorm_reduce_kernel(Shared sh, const in
   }
 }
 
-// Q_t = R diag(colinv) (fp32, caller's buffer) and its bf16 copy; tiles of rows of R.  One
-// warp per row, 16-byte loads of R (rows padded to a multiple of 8 floats), the scale factors
-// of the lane's columns kept in registers; the caller's Q is written only inside its r columns.
+// Q_t = R diag(colinv) (fp32, caller's buffer) and its bf16 copy; tiles of rows of R.  A thread
+// owns one 16-byte group of columns (its scale factors in registers) of every rp-th row of the
+// tile: cw threads (the power of two that covers the r / 4 groups) side by side in a row, so that
+// small ranks leave few lanes idle (a warp per row left 20 of 32 idle at r = 48: 35 us on the
+// 160M stack, 14 us now; 6.5 us against 31 us for one 512 x 16 R, spread over the
+// chip by smaller tiles).  Bound by HBM at large ranks (10 B per entry).  The caller's Q is
+// written only inside its r columns; rows of R and of the bf16 copies are padded to 8.
 constexpr int kScaleThreads = 256;
-__global__ void __launch_bounds__(kScaleThreads) colnorm_scale_kernel(Shared sh, const int4 *tiles) {
+__global__ void __launch_bounds__(kScaleThreads, 8) colnorm_scale_kernel(Shared sh, const int4 *tiles) {
   const int4 t = tiles[blockIdx.x];  // {layer, first row, rows, 0}
   DION_TILE_CHECK(t.x >= 0 && t.x < sh.num_layers && t.y >= 0 && t.z >= 1 &&
                       (int64_t)t.y + t.z <= sh.layers[t.x].n, sh.status);
   if (!sh.active[t.x]) return;
   const DevLayer &L = sh.layers[t.x];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int r = (int)L.r, r4 = (r + 3) / 4;  // r <= 512: at most 4 chunks per lane
-  float4 cs[4];
+  const int r = (int)L.r, r4 = (r + 3) / 4;  // r <= 512: at most 128 groups
+  int lg = 7;
+  while (lg > 0 && (1 << (lg - 1)) >= r4) --lg;
+  const int c4 = threadIdx.x & ((1 << lg) - 1), rp = kScaleThreads >> lg;
+  if (c4 >= r4) return;
+  const int c = 4 * c4;
+  const bool whole = c + 4 <= r;
+  const float4 cs = make_float4(L.colinv[c], c + 1 < r ? L.colinv[c + 1] : 0.f, c + 2 < r ? L.colinv[c + 2] : 0.f,
+                                c + 3 < r ? L.colinv[c + 3] : 0.f);
+  const int64_t ldp = L.ldp, ldq = L.ldq;
+  const float *R = L.R + c;
+  float *Q = L.Q + c;
+  __nv_bfloat16 *hi = L.Qn_hi + c, *lo = L.Qn_lo == nullptr ? nullptr : L.Qn_lo + c;
+  for (int64_t i = t.y + (threadIdx.x >> lg); i < (int64_t)t.y + t.z; i += rp) {
+    const float4 rv = *reinterpret_cast<const float4 *>(R + i * ldp);
+    const float4 q = make_float4(rv.x * cs.x, rv.y * cs.y, rv.z * cs.z, rv.w * cs.w);
+    const __nv_bfloat162 h01 = __floats2bfloat162_rn(q.x, q.y), h23 = __floats2bfloat162_rn(q.z, q.w);
+    uint2 hv;
+    hv.x = *reinterpret_cast<const uint32_t *>(&h01);
+    hv.y = *reinterpret_cast<const uint32_t *>(&h23);
+    *reinterpret_cast<uint2 *>(hi + i * ldp) = hv;
+    if (lo != nullptr) {  // BF16X3: q - bf16(q), rounded to bf16
+      const float2 f01 = __bfloat1622float2(h01), f23 = __bfloat1622float2(h23);
+      const __nv_bfloat162 l01 = __floats2bfloat162_rn(q.x - f01.x, q.y - f01.y);
+      const __nv_bfloat162 l23 = __floats2bfloat162_rn(q.z - f23.x, q.w - f23.y);
+      uint2 lv;
+      lv.x = *reinterpret_cast<const uint32_t *>(&l01);
+      lv.y = *reinterpret_cast<const uint32_t *>(&l23);
+      *reinterpret_cast<uint2 *>(lo + i * ldp) = lv;
+    }
+    if (whole) {
+      *reinterpret_cast<float4 *>(Q + i * ldq) = q;
+    } else {
+      const float qq[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const int c = 4 * (lane + 32 * k);
-    cs[k] = make_float4(c < r ? L.colinv[c] : 0.f, c + 1 < r ? L.colinv[c + 1] : 0.f,
-                        c + 2 < r ? L.colinv[c + 2] : 0.f, c + 3 < r ? L.colinv[c + 3] : 0.f);
-  }
-  for (int64_t i = t.y + warp; i < (int64_t)t.y + t.z; i += kScaleThreads / 32) {
-    const float *Rrow = L.R + i * L.ldp;
-    float4 rv[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-      if (lane + 32 * k < r4) rv[k] = *reinterpret_cast<const float4 *>(Rrow + 4 * (lane + 32 * k));
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int c4 = lane + 32 * k;
-      if (c4 >= r4) continue;
-      const float4 q = make_float4(rv[k].x * cs[k].x, rv[k].y * cs[k].y, rv[k].z * cs[k].z, rv[k].w * cs[k].w);
-      const __nv_bfloat162 h01 = __floats2bfloat162_rn(q.x, q.y), h23 = __floats2bfloat162_rn(q.z, q.w);
-      uint2 hv;
-      hv.x = *reinterpret_cast<const uint32_t *>(&h01);
-      hv.y = *reinterpret_cast<const uint32_t *>(&h23);
-      *reinterpret_cast<uint2 *>(L.Qn_hi + i * L.ldp + 4 * c4) = hv;  // workspace rows: padded
-      if (L.Qn_lo != nullptr) {  // BF16X3: q - bf16(q), rounded to bf16
-        const float2 f01 = __bfloat1622float2(h01), f23 = __bfloat1622float2(h23);
-        const __nv_bfloat162 l01 = __floats2bfloat162_rn(q.x - f01.x, q.y - f01.y);
-        const __nv_bfloat162 l23 = __floats2bfloat162_rn(q.z - f23.x, q.w - f23.y);
-        uint2 lv;
-        lv.x = *reinterpret_cast<const uint32_t *>(&l01);
-        lv.y = *reinterpret_cast<const uint32_t *>(&l23);
-        *reinterpret_cast<uint2 *>(L.Qn_lo + i * L.ldp + 4 * c4) = lv;
-      }
-      float *Qrow = L.Q + i * L.ldq + 4 * c4;
-      if (4 * c4 + 4 <= r) {
-        *reinterpret_cast<float4 *>(Qrow) = q;
-      } else {
-        const float qq[4] = {q.x, q.y, q.z, q.w};
-        for (int e = 0; e < r - 4 * c4; ++e) Qrow[e] = qq[e];
-      }
+      for (int e = 0; e < 3; ++e)
+        if (c + e < r) Q[i * ldq + e] = qq[e];
     }
   }
 }

@@ -606,3 +606,11 @@ def test_row_tiles(prec, gate):
     taus = [0.5 if l % 2 and not local else 1e9 for l in range(len(ROW_TILES.shapes))]
     run_per_step(ROW_TILES, PRECS[prec], dict(gate_mode=gate, tau_global=1e9 if local else 0.5), ROW_TILES.steps,
                  TOL_FP32, taus=taus)
+
+
+@pytest.mark.parametrize("rank", [2, 5, 8, 31, 65, 130, 253])
+def test_column_scaling_ranks(rank):
+    """ColumnNormalize's row tiles where a row of R has one group of four columns, a partial last
+    group, or a number of groups that is or is not a power of two (split operands: 1e-4)."""
+    w = wl.scaled(wl.WORKLOADS["gpt160m_block_r192"], "scale", [(300, 270), (270, 261), (256, 520)], rank=rank, steps=2)
+    run_per_step(w, PRECS["bf16x3"], dict(gate_mode=oc.GATE_ALWAYS), w.steps, TOL_FP32)
