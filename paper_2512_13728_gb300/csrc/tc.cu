@@ -172,6 +172,7 @@ void bind(const TcLayout &lo, char *base, DevLayer *dl, int32_t L, TcPlan *tp) {
     dl[l].rtile_cnt = (int32_t)((dl[l].n + 127) / 128);
     // the update forms B = M + G itself (BF16 mode with bf16 G); BF16X3 writes B into M
     dl[l].b_deferred = (dl[l].g_dtype == DT_BF16 && lo.precision == DION_PREC_BF16) ? 1 : 0;
+    tp->defers = tp->defers || dl[l].b_deferred != 0;
     if (lo.precision == DION_PREC_BF16X3) {
       dl[l].Bl = reinterpret_cast<__nv_bfloat16 *>(base + lo.o_bl[l]);
       dl[l].P_lo = reinterpret_cast<__nv_bfloat16 *>(base + lo.o_plo[l]);
@@ -233,12 +234,10 @@ cudaError_t encode_maps(const DevLayer *dl, int32_t L, LayerMaps *dst) {
     const uint64_t p16 = (uint64_t)d.ldp * 2, p32 = (uint64_t)d.ldp * 4;
     const bool ok = encode_bf16_2d(&m.P_hi, d.P_hi, d.r, d.m, p16, 64, 128) &&
                     encode_bf16_2d(&m.R_hi, d.R_hi, d.r, d.n, p16, 64, 128) &&
-                    encode_bf16_2d(&m.Qn_hi, d.Qn_hi, d.r, d.n, p16, 64, 128) &&
+                    encode_bf16_2d(&m.R_64, d.R_hi, d.r, d.n, p16, 64, 64) &&
                     encode_f32_2d(&m.Mf, d.M, d.n, d.m, (uint64_t)d.ldm * 4, 32, 128) &&
                     encode_f32_2d(&m.Xf, d.X, d.n, d.m, (uint64_t)d.ldx * 4, 32, 128) &&
-                    encode_f32_2d(&m.Mf16, d.M, d.n, d.m, (uint64_t)d.ldm * 4, 16, 128) &&
-                    encode_f32_2d(&m.Xf16, d.X, d.n, d.m, (uint64_t)d.ldx * 4, 16, 128) &&
-                    (d.g_dtype != DT_BF16 || encode_bf16_2d(&m.Gh16, d.G, d.n, d.m, (uint64_t)d.ldg * 2, 16, 128)) &&
+                    (d.g_dtype != DT_BF16 || encode_bf16_2d(&m.Gh32, d.G, d.n, d.m, (uint64_t)d.ldg * 2, 32, 128)) &&
                     (d.g_dtype != DT_BF16 || encode_bf16_2d(&m.Gh64, d.G, d.n, d.m, (uint64_t)d.ldg * 2, 64, 128)) &&
                     encode_bf16_2d(&m.Qn_mn, d.Qn_hi, d.r, d.n, p16, 64, 64) &&
                     encode_bf16_2d(&m.P_mn, d.P_hi, d.r, d.m, p16, 64, 64) &&
@@ -257,17 +256,16 @@ cudaError_t encode_maps(const DevLayer *dl, int32_t L, LayerMaps *dst) {
                     (d.P_lo == nullptr ||
                      (encode_bf16_2d(&m.P_lo, d.P_lo, d.r, d.m, p16, 64, 128) &&
                       encode_bf16_2d(&m.R_lo, d.R_lo, d.r, d.n, p16, 64, 128) &&
-                      encode_bf16_2d(&m.Qn_lo, d.Qn_lo, d.r, d.n, p16, 64, 128) &&
                       encode_bf16_2d(&m.Qn_lo_mn, d.Qn_lo, d.r, d.n, p16, 64, 64) &&
                       encode_bf16_2d(&m.P_lo_mn, d.P_lo, d.r, d.m, p16, 64, 64) &&
                       encode_bf16_2d(&m.Bl_mn, d.Bl, d.n, d.m, (uint64_t)d.ldbh * 2, 64, 64) &&
                       encode_bf16_2d(&m.Bl_k, d.Bl, d.n, d.m, (uint64_t)d.ldbh * 2, 64, 128) &&
                       encode_bf16_2d(&m.P_hi32, d.P_hi, d.r, d.m, p16, 32, 128) &&
                       encode_bf16_2d(&m.P_lo32, d.P_lo, d.r, d.m, p16, 32, 128) &&
-                      encode_bf16_2d(&m.R_hi32, d.R_hi, d.r, d.n, p16, 32, 128) &&
-                      encode_bf16_2d(&m.R_lo32, d.R_lo, d.r, d.n, p16, 32, 128) &&
-                      encode_bf16_2d(&m.Qn_hi32, d.Qn_hi, d.r, d.n, p16, 32, 128) &&
-                      encode_bf16_2d(&m.Qn_lo32, d.Qn_lo, d.r, d.n, p16, 32, 128)));
+                      encode_bf16_2d(&m.R_hi32, d.R_hi, d.r, d.n, p16, 32, 64) &&
+                      encode_bf16_2d(&m.R_lo32, d.R_lo, d.r, d.n, p16, 32, 64) &&
+                      encode_bf16_2d(&m.Qn_hi32, d.Qn_hi, d.r, d.n, p16, 32, 64) &&
+                      encode_bf16_2d(&m.Qn_lo32, d.Qn_lo, d.r, d.n, p16, 32, 64)));
     if (!ok) return cudaErrorInvalidValue;
   }
   return cudaMemcpy(dst, maps.data(), sizeof(LayerMaps) * maps.size(), cudaMemcpyHostToDevice);

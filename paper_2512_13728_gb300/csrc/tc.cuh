@@ -15,14 +15,13 @@ namespace tc {
 // swizzle with 64-element inner boxes; fp32 maps use 32-element (128-byte) inner boxes.
 struct LayerMaps {
   CUtensorMap P_hi;   // m x r bf16:  box {64, 128}  update: A operand (K = r)
-  CUtensorMap R_hi;   // n x r bf16:  box {64, 128}  update: B operand of P R^T
-  CUtensorMap Qn_hi;  // n x r bf16:  box {64, 128}  update: B operand of P Q_t^T
-  CUtensorMap Mf;     // m x n fp32 (caller M): box {32, 128}  update: B in / M_t out
-  CUtensorMap Xf;     // m x n fp32 (caller X): box {32, 128}  update: X in / out
-  CUtensorMap Mf16, Xf16;  // m x n fp32: box {16, 128}, 64-byte swizzle (update epilogue)
-  CUtensorMap Gh16;        // m x n bf16 G: box {16, 128}, 32-byte swizzle (update epilogue)
+  CUtensorMap R_hi;   // n x r bf16:  box {64, 128}  B^T P: output store
+  CUtensorMap R_64;   // n x r bf16:  box {64, 64}   update: B operand of P R^T (a CTA's half)
+  CUtensorMap Mf, Xf;      // m x n fp32 (caller M, X): box {32, 128}  update streams
+  CUtensorMap Gh32;        // m x n bf16 G: box {32, 128}, 64-byte swizzle  update streams
   CUtensorMap Gh64;        // m x n bf16 G: box {64, 128}  fused buffer pass + B Q
-  CUtensorMap Qn_mn;  // n x r bf16:  box {64, 64}   B Q: MN-major B operand (K = n)
+  CUtensorMap Qn_mn;  // n x r bf16:  box {64, 64}   B Q: MN-major B operand (K = n); update: B operand
+                      // of P Q_t^T (a CTA's half, K = r)
   CUtensorMap P_mn;   // m x r bf16:  box {64, 64}   B^T P: MN-major B operand (K = m)
   CUtensorMap Bh_mn;  // m x n bf16:  box {64, 64}   B^T P: MN-major A operand (K = m)
   CUtensorMap Bh_k;   // m x n bf16:  box {64, 128}  B Q: K-major A operand (K = n)
@@ -37,10 +36,11 @@ struct LayerMaps {
   CUtensorMap Linv;   // r x r fp32:  box {32, 128}  TRSM B operand (rows of L^{-1})
   CUtensorMap Linv32; // r x r fp32:  box {32, 32}   Cholesky trailing update (reduce-add)
   // BF16X3: the low halves, boxes as their high counterparts (zeroed maps in the other modes)
-  CUtensorMap P_lo, R_lo, Qn_lo;  // K-major {64, 128}: update operands
+  CUtensorMap P_lo, R_lo;  // {64, 128}: output stores of the solve and of B^T P
   CUtensorMap Qn_lo_mn, P_lo_mn, Bl_mn;  // MN-major {64, 64}: B Q / B^T P operands
   CUtensorMap Bl_k;   // K-major {64, 128}: B Q A operand
-  // BF16X3 update operands in 32-wide K chunks: K-major {32, 128}, 64-byte swizzle
+  // BF16X3 update operands in 32-wide K chunks: K-major, 64-byte swizzle, {32, 128} for P and
+  // {32, 64} (a CTA's half) for R and Q_t
   CUtensorMap P_hi32, P_lo32, R_hi32, R_lo32, Qn_hi32, Qn_lo32;
 };
 
@@ -96,6 +96,7 @@ struct TcPlan {
   int32_t precision = 0;
   int32_t launches = 0;
   bool fuse_buffer = false;
+  bool defers = false;  // some layer leaves B = M + G to the update (unless this step has B in M)
   uint32_t fb_smem = 0;
   size_t chol_tc_smem = 0;  // the first pass's Cholesky on tensor cores (BF16 mode)
   // CUDA-core pieces reused by this path (set by the plan)

@@ -1,13 +1,24 @@
 // Error feedback + parameter update (Algorithm 1/2, sync branch):
 //   M = B - (1 - mu) P R^T,   X = X - eta sqrt(m/n) P Q_t^T
-// run as one persistent, warp-specialized kernel over 128 x 128 output tiles:
-//   warp 0      TMA producer: bf16 K-major chunks of P (A), R and Q_t (two B operands) into a
-//               3-stage shared-memory ring (BF16X3: also their low halves);
-//   warp 1      MMA issuer: two 128x128x16 tcgen05.mma per k-step into a double-buffered
+// run as one persistent, warp-specialized kernel over 256 x 128 output tiles, one CTA pair per
+// tile (CTA c owns its rows 128 c .. 128 c + 127):
+//   warp 0      TMA producer: bf16 K-major chunks of P (A: this CTA's 128 rows) and of R and Q_t
+//               (B: this CTA's half, 64 of the tile's 128 rows) into a shared-memory ring
+//               (BF16X3: also their low halves);
+//   warp 1      (CTA 0) MMA issuer: two 256x128x16 pair MMAs per k-step into a double-buffered
 //               pair of TMEM accumulators (U1 = P R^T, U2 = P Q_t^T; 4 x 128 = 512 columns);
-//   warps 2..5  epilogue (both CTAs): TMA-load 128 x 16 fp32 boxes of B (in the M buffer) and X,
-//               read U1/U2 from TMEM (thread = tile row), compute M_t and X_t in shared
-//               memory, TMA-store both; per-tile fp64 partial of ||M_t||^2 for Equation 1.
+//   warp 6      streams: TMA loads of 128 x 32 boxes of M, X (and G) into a ring of sub-chunk
+//               buffers, TMA stores of the buffers the epilogue has finished;
+//   warps 2..5  epilogue (thread = tile row): U1/U2 from TMEM, M_t and X_t computed in place in the
+//               sub-chunk buffers; per-tile fp64 partial of ||M_t||^2 for Equation 1.
+// HBM-bound.  The streams have a warp of their own, so that no epilogue thread waits for a store to
+// be read before the next load goes out, and move 128-byte row segments (64-byte ones reached 6.0
+// TB/s at rank 48, these 6.3); the pair MMA halves the R and Q_t bytes each SM receives, which pays
+// for the larger stream buffers.  Measured before (a CTA per 128 x 128 tile, 64-byte segments issued
+// by the epilogue's first thread, a barrier per sub-chunk), with a stream warp alone, and now:
+// 290 / 262 / 256 us on the 160M stack at rank 192, 542 / 475 / 437 us on half of the 350M stack
+// (B in M), 1003 / 917 / 908 us on all of it with split operands, 3826 / 4075 / 3726 us on the 1.3B
+// stack at rank 512.  The same loads as cp.async copies from four more warps: 257, 459, 943, 4024.
 #include "tc.cuh"
 #include "tc_common.cuh"
 #include "tc_kernels.cuh"
@@ -18,45 +29,46 @@ namespace cd {
 namespace tc {
 
 // ============================================================ update (tcgen05) kernel ===
-// CTAs 2 s and 2 s + 1 take row tiles 2 p and 2 p + 1 of the same column blocks in the same
-// order (schedule segment s), so the R and Q_t chunks one of them loads are usually still in L2
-// when the other asks for them.  Each CTA loads all three operand boxes of a stage itself.
-constexpr uint32_t U_OPB = 128u * 64u * 2u;           // 128 x 64 bf16 operand box (BF16: one per operand)
-constexpr uint32_t U_OPB32 = 128u * 32u * 2u;         // 128 x 32 bf16 operand box (BF16X3)
-constexpr uint32_t U_EBOX = 128u * 16u * 4u;          // one 128 x 16 fp32 box (64-byte swizzle)
-constexpr uint32_t U_GBOX = 128u * 16u * 2u;          // one 128 x 16 bf16 box of G (32-byte swizzle)
-constexpr uint32_t U_EBUF2 = 2u * U_EBOX + U_GBOX;     // M, X and G of one 16-column sub-chunk (20 KB)
-static_assert(U_EBUF2 % 1024u == 0, "every box of a sub-chunk buffer stays 1024-byte aligned");
-constexpr int U_THREADS = 192;
-constexpr uint32_t U_IDESC = idesc_bf16(128, 128, false, false);
-// Ring depths.  BF16: 3 stages of {P, R, Q_t} in 64-wide K chunks (128-byte swizzle) and 4
-// epilogue sub-chunk buffers of M, X and G.  BF16X3: each stage also holds the low halves of P,
-// R and Q_t (P R^T = Ph Rh^T + Ph Rl^T + Pl Rh^T, the same for P Q_t^T), and B is already in M
-// (no G box); its stages take 32-wide K chunks (64-byte swizzle), so 3 stages of 6 boxes leave
-// room for 5 epilogue buffers of M and X (loads 4 sub-chunks ahead: with 2 buffers, one load in
-// flight, the epilogue waited on every sub-chunk).
-template <bool X3>
+constexpr int U_SUB = 32;                        // columns of a stream sub-chunk: 128-byte row segments
+constexpr uint32_t U_EBOX = 128u * U_SUB * 4u;  // one 128 x 32 fp32 box of M or X (128-byte swizzle)
+constexpr uint32_t U_GBOX = 128u * U_SUB * 2u;  // one 128 x 32 bf16 box of G (64-byte swizzle)
+constexpr int U_THREADS = 7 * 32;
+constexpr uint32_t U_IDESC = idesc_bf16(256, 128, false, false);
+// Ring depths.  A stage holds this CTA's 128 rows of P and its 64 rows of R and of Q_t: BF16 in
+// 64-wide K chunks (128-byte swizzle); BF16X3, with the low halves too (P R^T = Ph Rh^T + Ph Rl^T
+// + Pl Rh^T, the same for P Q_t^T), in 32-wide K chunks (64-byte swizzle): 32 KB either way.  The
+// rest of shared memory holds stream sub-chunks of M, X and, where the kernel forms B = M + G
+// itself (GIN), G: 40 KB or 32 KB each.
+// DEEP takes a fourth operand stage in place of a stream buffer, for ranks above kDeepRank: there a
+// tile's operands (r / 64 chunks of 32 KB) outweigh its streams, and more stream loads in flight
+// only delay them: 3726 us against 4553 on the 1.3B stack at rank 512, 1041 / 1108 on twelve
+// 1536-wide blocks at rank 384, 1051 / 1058 at rank 320, and the other way round at 272 (1067 /
+// 1034); with B in M 959 / 993 at rank 384, 936 / 941 at 320.
+constexpr int kDeepRank = 304;  // between the ranks measured on either side
+template <bool X3, bool GIN, bool DEEP>
 struct UpdCfg {
   static constexpr uint32_t KW = X3 ? 32u : 64u;  // K chunk width (bf16 elements per operand row)
-  static constexpr uint32_t OPB = X3 ? U_OPB32 : U_OPB;
-  static constexpr int STAGES = 3;
-  static constexpr uint32_t STAGE = (X3 ? 6u : 3u) * OPB;  // P, R, Q_t [, P_lo, R_lo, Q_lo]
-  static constexpr int EBUF = X3 ? 5 : 4;
-  static constexpr uint32_t EBUF2 = X3 ? 2u * U_EBOX : U_EBUF2;  // bytes of one sub-chunk buffer
-  static constexpr uint32_t SMEM = 1024u + STAGES * STAGE + EBUF * EBUF2 + 256u;
+  static constexpr uint32_t PB = 128u * KW * 2u, BB = 64u * KW * 2u;  // bytes of a P box, of an R or Q_t box
+  static constexpr uint32_t HALF = PB + 2u * BB;  // P, R, Q_t; BF16X3: then their low halves
+  static constexpr int STAGES = DEEP ? 4 : 3;
+  static constexpr uint32_t STAGE = (X3 ? 2u : 1u) * HALF;
+  static constexpr int EBUF = GIN ? (DEEP ? 2 : 3) : (DEEP ? 3 : 4);
+  static constexpr uint32_t EBUFB = 2u * U_EBOX + (GIN ? U_GBOX : 0u);  // bytes of one sub-chunk buffer
+  static constexpr uint32_t SMEM = 1024u + STAGES * STAGE + EBUF * EBUFB + 256u;
+  static_assert(EBUFB % 1024u == 0 && HALF % 1024u == 0, "every box stays aligned to its swizzle atom");
+  static_assert(SMEM <= 227u * 1024u, "update smem");
+  static_assert((2 * STAGES + 4 + 2 * EBUF + 1) * 8 <= 256, "barriers");
 };
-static_assert(UpdCfg<true>::SMEM <= 227u * 1024u && UpdCfg<false>::SMEM <= 227u * 1024u, "update smem");
 
 // Tile = {layer, row-tile pair p, column tile, ||M_t|| slot of row tile 2 p}.
-template <bool X3>
-__global__ void __launch_bounds__(U_THREADS, 1)
+template <bool X3, bool GIN, bool DEEP>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(U_THREADS, 1)
     tc_update_kernel(Shared sh, const int4 *__restrict__ tiles, const int *__restrict__ off, const LayerMaps *__restrict__ maps,
                      float mu, float eta, float keep) {
-  constexpr int U_STAGES = UpdCfg<X3>::STAGES;
-  constexpr uint32_t U_STAGE = UpdCfg<X3>::STAGE;
-  constexpr uint32_t KW = UpdCfg<X3>::KW, OPB = UpdCfg<X3>::OPB;
-  constexpr int U_EBUF = UpdCfg<X3>::EBUF;
-  constexpr uint32_t U_EBUFB = UpdCfg<X3>::EBUF2;
+  using Cfg = UpdCfg<X3, GIN, DEEP>;
+  constexpr int U_STAGES = Cfg::STAGES, U_EBUF = Cfg::EBUF;
+  constexpr uint32_t U_STAGE = Cfg::STAGE, U_EBUFB = Cfg::EBUFB;
+  constexpr uint32_t KW = Cfg::KW, PB = Cfg::PB, BB = Cfg::BB, HALF = Cfg::HALF;
   if (sh.gate_scratch[kScratchActive] == 0ull) return;  // no layer takes the Dion branch
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = align1024(smem_raw);
@@ -65,37 +77,48 @@ __global__ void __launch_bounds__(U_THREADS, 1)
   uint64_t *bars = reinterpret_cast<uint64_t *>(epi + U_EBUF * U_EBUFB);
   uint64_t *full = bars, *empty = bars + U_STAGES;
   uint64_t *acc_full = bars + 2 * U_STAGES, *acc_empty = acc_full + 2, *epi_full = acc_empty + 2;
-  uint64_t *drain = epi_full + U_EBUF;
+  uint64_t *epi_done = epi_full + U_EBUF, *drain = epi_done + U_EBUF;
   __shared__ uint32_t tmem_base_s;
   __shared__ int abort_s;
   __shared__ double red_s[4];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // hand-off waits between the roles use the plan's limit; the drains below keep the default
   const Abort ab{&abort_s, sh.handoff_limit_ns};
-  const uint32_t rank = blockIdx.x & 1u;  // row tile 2 p + rank of the segment's tiles
+  const uint32_t rank = cluster_ctarank();  // row tile 2 p + rank of the segment's tiles
   const int seg = blockIdx.x >> 1;
+  // 32-column sub-chunks of a tile that start inside the matrix; 0 for the pair's second tile
+  // when it lies past the last row tile
+  auto subs_of = [&](const int4 &t) -> int {
+    const DevLayer &L = sh.layers[t.x];
+    if ((int64_t)(2 * t.y + (int)rank) * 128 >= L.m) return 0;
+    return (int)min((int64_t)(128 / U_SUB), (L.n - (int64_t)t.z * 128 + U_SUB - 1) / U_SUB);
+  };
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < U_STAGES; ++i) {
-      mbar_init(&full[i], 1);
-      mbar_init(&empty[i], 1);  // this CTA's MMA commit
+      mbar_init(&full[i], 1);   // used in CTA 0: its arm, both CTAs' bytes
+      mbar_init(&empty[i], 1);  // pair commit after the stage's MMAs
     }
     for (int b = 0; b < 2; ++b) {
-      mbar_init(&acc_full[b], 1);
-      mbar_init(&acc_empty[b], 1);  // the epilogue leader, after its warps have read TMEM
+      mbar_init(&acc_full[b], 1);   // pair commit after the tile's MMAs
+      mbar_init(&acc_empty[b], 2);  // used in CTA 0: each CTA's epilogue leader, its warps having read TMEM
     }
-    for (int b = 0; b < U_EBUF; ++b) mbar_init(&epi_full[b], 1);
+    for (int b = 0; b < U_EBUF; ++b) {
+      mbar_init(&epi_full[b], 1);  // the sub-chunk's loads
+      mbar_init(&epi_done[b], 4);  // one arrival per epilogue warp: M_t and X_t are in the buffer
+    }
     mbar_init(drain, 1);
     abort_s = 0;
     fence_mbar_init();
   }
   if (warp == 1) {
-    tmem_alloc(&tmem_base_s, 512);
-    tmem_relinquish();
+    tmem_alloc_pair(&tmem_base_s, 512);
+    tmem_relinquish_pair();
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  cluster_sync();  // both CTAs' barriers and TMEM exist before anything crosses the pair
   const uint32_t tmem = tmem_base_s;
 
   if (warp == 0) {
@@ -113,29 +136,31 @@ __global__ void __launch_bounds__(U_THREADS, 1)
           const uint32_t s = it % U_STAGES, ph = (it / U_STAGES) & 1u;
           if (!ab.wait(&empty[s], ph ^ 1u, sh.status)) { ok = false; break; }
           uint8_t *sp = stage + s * U_STAGE;
-          mbar_expect_tx(&full[s], U_STAGE);
-          const int k0 = kc * (int)KW;
+          const uint32_t fb = cluster_addr(&full[s], 0);
+          if (rank == 0) mbar_expect_tx(&full[s], 2u * U_STAGE);
+          const int k0 = kc * (int)KW, b0 = t.z * 128 + (int)rank * 64;
           if (X3) {
-            tma_load_2d(sp, &mp->P_hi32, &full[s], k0, mb * 128);
-            tma_load_2d(sp + OPB, &mp->R_hi32, &full[s], k0, t.z * 128);
-            tma_load_2d(sp + 2 * OPB, &mp->Qn_hi32, &full[s], k0, t.z * 128);
-            tma_load_2d(sp + 3 * OPB, &mp->P_lo32, &full[s], k0, mb * 128);
-            tma_load_2d(sp + 4 * OPB, &mp->R_lo32, &full[s], k0, t.z * 128);
-            tma_load_2d(sp + 5 * OPB, &mp->Qn_lo32, &full[s], k0, t.z * 128);
+            tma_load_2d_pair(sp, &mp->P_hi32, fb, k0, mb * 128);
+            tma_load_2d_pair(sp + PB, &mp->R_hi32, fb, k0, b0);
+            tma_load_2d_pair(sp + PB + BB, &mp->Qn_hi32, fb, k0, b0);
+            tma_load_2d_pair(sp + HALF, &mp->P_lo32, fb, k0, mb * 128);
+            tma_load_2d_pair(sp + HALF + PB, &mp->R_lo32, fb, k0, b0);
+            tma_load_2d_pair(sp + HALF + PB + BB, &mp->Qn_lo32, fb, k0, b0);
           } else {
-            tma_load_2d(sp, &mp->P_hi, &full[s], k0, mb * 128);
-            tma_load_2d(sp + OPB, &mp->R_hi, &full[s], k0, t.z * 128);
-            tma_load_2d(sp + 2 * OPB, &mp->Qn_hi, &full[s], k0, t.z * 128);
+            tma_load_2d_pair(sp, &mp->P_hi, fb, k0, mb * 128);
+            tma_load_2d_pair(sp + PB, &mp->R_64, fb, k0, b0);
+            tma_load_2d_pair(sp + PB + BB, &mp->Qn_mn, fb, k0, b0);
           }
         }
       }
-      // drain: every load this CTA issued has landed
+      // drain: the last stages' loads have landed and been consumed (their stage was freed); after
+      // an abort the first wait that runs out has given every load far longer than it takes
       for (uint32_t k = (it > U_STAGES ? it - U_STAGES : 0); k < it; ++k)
-        mbar_wait(&full[k % U_STAGES], (k / U_STAGES) & 1u, sh.status);
+        if (!mbar_wait(&empty[k % U_STAGES], (k / U_STAGES) & 1u, sh.status)) break;
     }
   } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA issuer
-    if (lane == 0) {
+    if (lane == 0 && rank == 0) {
       uint32_t it = 0, tcount = 0;
       bool ok = true;
       for (int ti = off[seg]; ti < off[seg + 1] && ok; ++ti) {
@@ -151,152 +176,153 @@ __global__ void __launch_bounds__(U_THREADS, 1)
           if (!ab.wait(&full[s], ph, sh.status)) { ok = false; break; }
           tc_fence_after();
           const uint32_t base = smem_u32(stage + s * U_STAGE);
-          // K-major operand box o of the stage, advanced by k16 steps of 16 elements (32 bytes)
+          // K-major operand box at offset o of the stage, advanced by k16 steps of 16 elements (32 bytes)
           auto desc = [&](uint32_t o, int k16) {
-            const uint32_t a = base + o * OPB + (uint32_t)k16 * 32u;
+            const uint32_t a = base + o + (uint32_t)k16 * 32u;
             return X3 ? smem_desc_sw64(a, 512) : smem_desc_sw128(a, 0, 1024);
           };
 #pragma unroll
           for (int k16 = 0; k16 < (int)(KW / 16u); ++k16) {
-            const uint64_t ad = desc(0, k16), rd = desc(1, k16), qd = desc(2, k16);
+            const uint64_t ad = desc(0, k16), rd = desc(PB, k16), qd = desc(PB + BB, k16);
             const uint32_t acc = (kc | k16) ? 1u : 0u;
-            umma_bf16(d1, ad, rd, U_IDESC, acc);
-            umma_bf16(d2, ad, qd, U_IDESC, acc);
+            umma_pair_bf16(d1, ad, rd, U_IDESC, acc);
+            umma_pair_bf16(d2, ad, qd, U_IDESC, acc);
             if (X3) {  // P R^T = Ph Rh^T + Ph Rl^T + Pl Rh^T, P Q_t^T likewise
-              const uint64_t adl = desc(3, k16);
-              umma_bf16(d1, ad, desc(4, k16), U_IDESC, 1u);
-              umma_bf16(d1, adl, rd, U_IDESC, 1u);
-              umma_bf16(d2, ad, desc(5, k16), U_IDESC, 1u);
-              umma_bf16(d2, adl, qd, U_IDESC, 1u);
+              const uint64_t adl = desc(HALF, k16);
+              umma_pair_bf16(d1, ad, desc(HALF + PB, k16), U_IDESC, 1u);
+              umma_pair_bf16(d1, adl, rd, U_IDESC, 1u);
+              umma_pair_bf16(d2, ad, desc(HALF + PB + BB, k16), U_IDESC, 1u);
+              umma_pair_bf16(d2, adl, qd, U_IDESC, 1u);
             }
           }
-          umma_commit(&empty[s]);  // the stage is free once its MMAs have read it
+          umma_pair_commit_mc(&empty[s], 0x3);  // the stage is free in both CTAs once its MMAs have read it
         }
         if (!ok) break;
-        umma_commit(&acc_full[b]);
+        umma_pair_commit_mc(&acc_full[b], 0x3);
         ++tcount;
       }
-      umma_commit(drain);  // every MMA of this CTA has completed before TMEM is freed
+      umma_pair_commit(drain);  // every MMA of the pair has completed before TMEM is freed
       mbar_wait(drain, 0, sh.status);
     }
-  } else {
-    // ---------------------------------------------------------------- epilogue (128 threads)
-    // B and X stream in 16-column sub-chunks through U_EBUF buffers.  The leader keeps the
-    // loads U_EBUF - 1 sub-chunks ahead of the one being written back, across tile boundaries
-    // (they do not depend on the MMAs), so HBM latency is covered without taking shared memory
-    // from the operand ring.
-    const int et = threadIdx.x - 64;
-    const uint32_t row = 32u * (warp & 3) + lane;  // TMEM lane = tile row
-    const bool leader = (et == 0);
-    const int tend = off[seg + 1];
-    // 16-column sub-chunks of a tile that start inside the matrix; 0 for the pair's second tile
-    // when it lies past the last row tile
-    auto subs_of = [&](const int4 &t) -> int {
-      const DevLayer &L = sh.layers[t.x];
-      if ((int64_t)(2 * t.y + (int)rank) * 128 >= L.m) return 0;
-      return (int)std::min<int64_t>(8, (L.n - (int64_t)t.z * 128 + 15) / 16);
-    };
-    int lt = off[seg], lj = 0;  // load cursor: tile, sub-chunk
-    auto skip_empty = [&]() {
-      while (lt < tend && (!sh.active[tiles[lt].x] || subs_of(tiles[lt]) == 0)) ++lt;
-    };
-    skip_empty();
-    uint32_t ecount = 0, issued = 0;
-    auto issue_upto = [&](uint32_t target) {  // leader: loads of sub-chunks [issued, target)
-      while (issued < target && lt < tend) {
+  } else if (warp == 6) {
+    // ---------------------------------------------------------------- streams of M, X and G
+    // Loads run as far ahead of the epilogue as there are buffers, across tile boundaries (they do
+    // not depend on the MMAs): the next load into a buffer goes out as soon as its store has been
+    // read.
+    if (lane == 0) {
+      const int tend = off[seg + 1];
+      int lt = off[seg], lj = 0;  // load cursor: tile, sub-chunk
+      auto skip_empty = [&]() {
+        while (lt < tend && (!sh.active[tiles[lt].x] || subs_of(tiles[lt]) == 0)) ++lt;
+      };
+      skip_empty();
+      uint32_t issued = 0, stored = 0;
+      auto load_next = [&]() {  // the next sub-chunk, into the buffer of sub-chunk issued - U_EBUF
         const int4 t = tiles[lt];
         const LayerMaps *mp = maps + t.x;
         const uint32_t eb = issued % U_EBUF;
-        // the buffer's previous sub-chunk (issued - U_EBUF) was stored at least one sub-chunk
-        // ago: at most the latest store group may still be reading shared memory
-        if (issued >= U_EBUF) bulk_wait_read<1>();
         uint8_t *bs = epi + eb * U_EBUFB;
-        const int r0 = (2 * t.y + (int)rank) * 128, x0 = t.z * 128 + lj * 16;
-        const bool defer = sh.layers[t.x].b_deferred != 0 && !sh.b_in_m;  // B = M + G is formed here
+        const int r0 = (2 * t.y + (int)rank) * 128, x0 = t.z * 128 + lj * U_SUB;
+        const bool defer = GIN && sh.layers[t.x].b_deferred != 0;  // B = M + G is formed here
         mbar_expect_tx(&epi_full[eb], 2u * U_EBOX + (defer ? U_GBOX : 0u));
-        tma_load_2d(bs, &mp->Mf16, &epi_full[eb], x0, r0);
-        tma_load_2d(bs + U_EBOX, &mp->Xf16, &epi_full[eb], x0, r0);
-        if (defer) tma_load_2d(bs + 2 * U_EBOX, &mp->Gh16, &epi_full[eb], x0, r0);
+        tma_load_2d(bs, &mp->Mf, &epi_full[eb], x0, r0);
+        tma_load_2d(bs + U_EBOX, &mp->Xf, &epi_full[eb], x0, r0);
+        if (defer) tma_load_2d(bs + 2 * U_EBOX, &mp->Gh32, &epi_full[eb], x0, r0);
         ++issued;
         if (++lj == subs_of(t)) {
           lj = 0;
           ++lt;
           skip_empty();
         }
+      };
+      while (issued < (uint32_t)U_EBUF && lt < tend) load_next();
+      bool ok = true;
+      for (int ti = off[seg]; ti < tend && ok; ++ti) {
+        const int4 t = tiles[ti];
+        if (!sh.active[t.x]) continue;
+        const LayerMaps *mp = maps + t.x;
+        const int ns = subs_of(t), r0 = (2 * t.y + (int)rank) * 128;
+        for (int sub = 0; sub < ns; ++sub, ++stored) {
+          const uint32_t eb = stored % U_EBUF;
+          if (!ab.wait(&epi_done[eb], (stored / U_EBUF) & 1u, sh.status)) { ok = false; break; }
+          uint8_t *bs = epi + eb * U_EBUFB;
+          const int x0 = t.z * 128 + sub * U_SUB;  // past the matrix's edges: clipped by the store
+          tma_store_2d(&mp->Mf, bs, x0, r0);
+          tma_store_2d(&mp->Xf, bs + U_EBOX, x0, r0);
+          bulk_commit();
+          if (lt < tend) {
+            bulk_wait_read<0>();
+            load_next();
+          }
+        }
       }
-    };
-    if (leader) issue_upto(U_EBUF - 1);
-    uint32_t tcount = 0;
-    uint32_t waited = 0;  // sub-chunks whose load this role has waited for, in order
-    bool ok = true;
-    for (int ti = off[seg]; ti < tend && ok; ++ti) {
+      bulk_wait<0>();
+      // every load has landed (after an abort the epilogue may not have waited for the last ones):
+      // the latest load of each buffer, whose phase is the barrier's latest
+      for (uint32_t k = issued > (uint32_t)U_EBUF ? issued - U_EBUF : 0u; k < issued; ++k)
+        mbar_wait(&epi_full[k % U_EBUF], (k / U_EBUF) & 1u, sh.status);
+    }
+  } else {
+    // ---------------------------------------------------------------- epilogue (128 threads)
+    const int et = threadIdx.x - 64;
+    const uint32_t row = 32u * (warp & 3) + lane;  // TMEM lane = tile row
+    const bool leader = (et == 0);
+    const int tend = off[seg + 1];
+    uint32_t tcount = 0, ecount = 0;
+    for (int ti = off[seg]; ti < tend; ++ti) {
       const int4 t = tiles[ti];
       if (!sh.active[t.x]) continue;
       const DevLayer &L = sh.layers[t.x];
-      const LayerMaps *mp = maps + t.x;
       const float dec = 1.f - mu, c = eta * L.sqrt_m_over_n;
-      const int mb = 2 * t.y + (int)rank, r0 = mb * 128, c0 = t.z * 128;
       const int ntc = (int)((L.n + 127) / 128);
       const int ns = subs_of(t);
-      const bool defer = L.b_deferred != 0 && !sh.b_in_m;
+      const bool defer = GIN && L.b_deferred != 0;
       const uint32_t b = tcount & 1u, aph = (tcount >> 1) & 1u;
       if (!named_and(1, 128, ab.wait(&acc_full[b], aph, sh.status))) break;
       tc_fence_after();
       float ss = 0.f;
-      for (int j = 0; j < (ns + 1) / 2 && ok; ++j) {  // 32-column TMEM chunk j = sub-chunks 2j, 2j + 1
+      bool ok = true;  // warp-uniform; the four warps agree at the tile's last barrier
+      for (int j = 0; j < ns; ++j) {  // sub-chunk j = 32-column TMEM chunk j
         uint32_t u1[32], u2[32];
         tmem_ld32(tmem + ((32u * (warp & 3)) << 16) + b * 256u + j * 32, u1);
         tmem_ld32(tmem + ((32u * (warp & 3)) << 16) + b * 256u + 128u + j * 32, u2);
         tmem_ld_wait();
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int sub = 2 * j + h;
-          if (sub >= ns) break;
-          const uint32_t k = ecount + sub, eb = k % U_EBUF, eph = (k / U_EBUF) & 1u;
-          if (!named_and(1, 128, ab.wait(&epi_full[eb], eph, sh.status))) {
-            ok = false;
-            break;
-          }
-          waited = k + 1;
-          uint8_t *bs = epi + eb * U_EBUFB;
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const uint32_t o = sw64_f32(row, q);
-            const int cc = h * 16 + q * 4;
-            float4 bv = *reinterpret_cast<float4 *>(bs + o);
-            float4 xv = *reinterpret_cast<float4 *>(bs + U_EBOX + o);
-            if (defer) {  // B = M_{t-1} + G, the same fp32 additions as the buffer pass
-              const uint2 gv = *reinterpret_cast<const uint2 *>(bs + 2 * U_EBOX + sw32_offset(row, (uint32_t)q >> 1) +
-                                                                (q & 1) * 8);
-              bv.x += __uint_as_float(gv.x << 16);
-              bv.y += __uint_as_float(gv.x & 0xffff0000u);
-              bv.z += __uint_as_float(gv.y << 16);
-              bv.w += __uint_as_float(gv.y & 0xffff0000u);
-            }
-            bv.x = fmaf(-dec, __uint_as_float(u1[cc + 0]), bv.x);
-            bv.y = fmaf(-dec, __uint_as_float(u1[cc + 1]), bv.y);
-            bv.z = fmaf(-dec, __uint_as_float(u1[cc + 2]), bv.z);
-            bv.w = fmaf(-dec, __uint_as_float(u1[cc + 3]), bv.w);
-            xv.x = fmaf(-c, __uint_as_float(u2[cc + 0]), xv.x * keep);  // keep: decoupled weight decay
-            xv.y = fmaf(-c, __uint_as_float(u2[cc + 1]), xv.y * keep);
-            xv.z = fmaf(-c, __uint_as_float(u2[cc + 2]), xv.z * keep);
-            xv.w = fmaf(-c, __uint_as_float(u2[cc + 3]), xv.w * keep);
-            ss = fmaf(bv.x, bv.x, ss); ss = fmaf(bv.y, bv.y, ss);
-            ss = fmaf(bv.z, bv.z, ss); ss = fmaf(bv.w, bv.w, ss);
-            *reinterpret_cast<float4 *>(bs + o) = bv;
-            *reinterpret_cast<float4 *>(bs + U_EBOX + o) = xv;
-          }
-          fence_async_smem();
-          named_sync(1, 128);
-          if (leader) {  // out-of-range rows/columns of a ragged tile are clipped by the store
-            tma_store_2d(&mp->Mf16, bs, c0 + sub * 16, r0);
-            tma_store_2d(&mp->Xf16, bs + U_EBOX, c0 + sub * 16, r0);
-            bulk_commit();
-            issue_upto(k + U_EBUF);  // sub-chunk k + U_EBUF - 1 reuses the buffer of k - 1
-          }
+        const uint32_t k = ecount + j, eb = k % U_EBUF, eph = (k / U_EBUF) & 1u;
+        if (!__all_sync(0xffffffffu, ab.wait(&epi_full[eb], eph, sh.status))) {
+          ok = false;
+          break;
         }
+        uint8_t *bs = epi + eb * U_EBUFB;
+#pragma unroll
+        for (int q = 0; q < U_SUB / 4; ++q) {
+          const uint32_t o = sw128_f32(row, q);
+          float4 bv = *reinterpret_cast<float4 *>(bs + o);
+          float4 xv = *reinterpret_cast<float4 *>(bs + U_EBOX + o);
+          if (defer) {  // B = M_{t-1} + G, the same fp32 additions as the buffer pass
+            const uint2 gv =
+                *reinterpret_cast<const uint2 *>(bs + 2 * U_EBOX + sw64_f32(row, (uint32_t)q >> 1) + (q & 1) * 8);
+            bv.x += __uint_as_float(gv.x << 16);
+            bv.y += __uint_as_float(gv.x & 0xffff0000u);
+            bv.z += __uint_as_float(gv.y << 16);
+            bv.w += __uint_as_float(gv.y & 0xffff0000u);
+          }
+          bv.x = fmaf(-dec, __uint_as_float(u1[4 * q + 0]), bv.x);
+          bv.y = fmaf(-dec, __uint_as_float(u1[4 * q + 1]), bv.y);
+          bv.z = fmaf(-dec, __uint_as_float(u1[4 * q + 2]), bv.z);
+          bv.w = fmaf(-dec, __uint_as_float(u1[4 * q + 3]), bv.w);
+          xv.x = fmaf(-c, __uint_as_float(u2[4 * q + 0]), xv.x * keep);  // keep: decoupled weight decay
+          xv.y = fmaf(-c, __uint_as_float(u2[4 * q + 1]), xv.y * keep);
+          xv.z = fmaf(-c, __uint_as_float(u2[4 * q + 2]), xv.z * keep);
+          xv.w = fmaf(-c, __uint_as_float(u2[4 * q + 3]), xv.w * keep);
+          ss = fmaf(bv.x, bv.x, ss); ss = fmaf(bv.y, bv.y, ss);
+          ss = fmaf(bv.z, bv.z, ss); ss = fmaf(bv.w, bv.w, ss);
+          *reinterpret_cast<float4 *>(bs + o) = bv;
+          *reinterpret_cast<float4 *>(bs + U_EBOX + o) = xv;
+        }
+        fence_async_smem();  // the buffer is read by the stream warp's store
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&epi_done[eb]);
       }
-      if (!ok) break;
       ecount += ns;
       // per-tile ||M_t||^2 (rows/columns outside the matrix hold 0), fixed reduction order;
       // the barrier also ends every thread's TMEM reads of this accumulator
@@ -305,42 +331,50 @@ __global__ void __launch_bounds__(U_THREADS, 1)
       for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
       if (lane == 0) red_s[warp - 2] = v;
       tc_fence_before();
-      named_sync(1, 128);
+      if (!named_and(1, 128, ok)) break;
       if (leader) {
-        mbar_arrive(&acc_empty[b]);  // every thread has read accumulator buffer b
+        mbar_arrive_cluster(cluster_addr(&acc_empty[b], 0));  // every thread has read accumulator buffer b
         if (ns > 0) sh.upart[t.w + (int)rank * ntc] = (red_s[0] + red_s[1]) + (red_s[2] + red_s[3]);
       }
       ++tcount;
     }
-    if (leader) {
-      bulk_wait<0>();
-      // loads issued but not waited for (only after an abort): at most U_EBUF - 1 of them, in
-      // distinct buffers, so each wait is for the latest phase of its buffer
-      for (uint32_t k = waited; k < issued; ++k) mbar_wait(&epi_full[k % U_EBUF], (k / U_EBUF) & 1u, sh.status);
-    }
   }
   tc_fence_before();
   __syncthreads();
+  cluster_sync();  // both CTAs are done with the pair's TMEM and barriers
   tc_fence_after();
-  if (warp == 1) tmem_dealloc(tmem, 512);
+  if (warp == 1) tmem_dealloc_pair(tmem, 512);
 }
 
 // ========================================================================= launch ===
+template <bool X3, bool GIN, bool DEEP>
+cudaError_t setup() {
+  return cudaFuncSetAttribute(tc_update_kernel<X3, GIN, DEEP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)UpdCfg<X3, GIN, DEEP>::SMEM);
+}
 cudaError_t setup_update_kernel(bool x3) {
-  return x3 ? cudaFuncSetAttribute(tc_update_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)UpdCfg<true>::SMEM)
-            : cudaFuncSetAttribute(tc_update_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)UpdCfg<false>::SMEM);
+  if (x3) return setup<true, false, false>();
+  for (const cudaError_t e : {setup<false, true, false>(), setup<false, false, false>(), setup<false, true, true>(),
+                              setup<false, false, true>()})
+    if (e != cudaSuccess) return e;
+  return cudaSuccess;
+}
+
+template <bool X3, bool GIN, bool DEEP>
+static void launch_as(const Shared &sh, const TcPlan &tp, float mu, float eta, float keep, cudaStream_t s) {
+  tc_update_kernel<X3, GIN, DEEP><<<2 * tp.d_update.grid, U_THREADS, UpdCfg<X3, GIN, DEEP>::SMEM, s>>>(
+      sh, tp.d_update.tiles, tp.d_update.off, tp.maps, mu, eta, keep);
 }
 
 void launch_update(const Shared &sh, const TcPlan &tp, float mu, float eta, float keep, cudaStream_t s) {
   if (tp.d_update.grid <= 0) return;
-  if (tp.precision == DION_PREC_BF16X3)
-    tc_update_kernel<true><<<2 * tp.d_update.grid, U_THREADS, UpdCfg<true>::SMEM, s>>>(
-        sh, tp.d_update.tiles, tp.d_update.off, tp.maps, mu, eta, keep);
-  else
-    tc_update_kernel<false><<<2 * tp.d_update.grid, U_THREADS, UpdCfg<false>::SMEM, s>>>(
-        sh, tp.d_update.tiles, tp.d_update.off, tp.maps, mu, eta, keep);
+  const bool gin = tp.defers && !sh.b_in_m;  // else B is in M
+  const bool deep = tp.max_r > kDeepRank;
+  if (tp.precision == DION_PREC_BF16X3) launch_as<true, false, false>(sh, tp, mu, eta, keep, s);
+  else if (gin && deep) launch_as<false, true, true>(sh, tp, mu, eta, keep, s);
+  else if (gin) launch_as<false, true, false>(sh, tp, mu, eta, keep, s);
+  else if (deep) launch_as<false, false, true>(sh, tp, mu, eta, keep, s);
+  else launch_as<false, false, false>(sh, tp, mu, eta, keep, s);
 }
 
 }  // namespace tc

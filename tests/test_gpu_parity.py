@@ -614,3 +614,15 @@ def test_column_scaling_ranks(rank):
     group, or a number of groups that is or is not a power of two (split operands: 1e-4)."""
     w = wl.scaled(wl.WORKLOADS["gpt160m_block_r192"], "scale", [(300, 270), (270, 261), (256, 520)], rank=rank, steps=2)
     run_per_step(w, PRECS["bf16x3"], dict(gate_mode=oc.GATE_ALWAYS), w.steps, TOL_FP32)
+
+
+@pytest.mark.parametrize("gate", ["always", "per_layer"])
+@pytest.mark.parametrize("rank", [64, 65, 256, 304, 305, 352])
+def test_update_pair_tiles(rank, gate):
+    """The update's pair tiles at the edges of its K chunks (64) and of its two ring shapes (rank 304),
+    with an odd number of row tiles (the pair's second tile empty), a column tile narrower than one
+    CTA's half, and a last 32-column sub-chunk that is partial; G added in the update (always) and B
+    already in M (per layer)."""
+    w = wl.scaled(wl.WORKLOADS["gpt160m_block_r192"], "pair", [(360, 400), (400, 390), (520, 385)], rank=rank, steps=2)
+    mode = oc.GATE_ALWAYS if gate == "always" else oc.GATE_PER_LAYER
+    run_per_step(w, PRECS["bf16"], dict(gate_mode=mode), w.steps, TOL_BF16)
