@@ -61,19 +61,134 @@ __device__ __forceinline__ void trinv32_row(float (&x)[CB], const float *D, cons
   }
 }
 
-// v <- T v for a lower-triangular 32 x 32 T (row-major, stride CB), in place from the bottom.
-template <int C>
+// v <- T v for a lower-triangular 32 x 32 T (row-major, row pitch LD), in place from the bottom.
+template <int C, int LD = CB>
 __device__ __forceinline__ void trmv32(float (&v)[CB], const float *T) {
   if constexpr (C >= 0) {
     float a0 = 0.f, a1 = 0.f;
 #pragma unroll
     for (int c2 = 0; c2 <= C; c2 += 2) {
-      a0 = fmaf(T[C * CB + c2], v[c2], a0);
-      if (c2 + 1 <= C) a1 = fmaf(T[C * CB + c2 + 1], v[c2 + 1], a1);
+      a0 = fmaf(T[C * LD + c2], v[c2], a0);
+      if (c2 + 1 <= C) a1 = fmaf(T[C * LD + c2 + 1], v[c2 + 1], a1);
     }
     v[C] = a0 + a1;
-    trmv32<C - 1>(v, T);
+    trmv32<C - 1, LD>(v, T);
   }
+}
+
+// Cholesky factor and inverse of a 32 x 32 block by two warps.  The first (diag_factor) eliminates
+// the columns, lane = row; the second (diag_invert) carries the inverse along one eight-column
+// segment behind, lane = column.  Both are loops over the columns of a segment, in registers that
+// move down one place per column (v[0] is the current column), so that the code stays small (fully
+// unrolled columns cost 20K cycles of instruction fetches the first time through) and the work
+// shrinks with the segments.  Bound by the elimination's chain from column to column; about 5K
+// cycles against 12.6K for chol32_col and trinv32_row in one warp.
+struct DiagScratch {
+  // current column, unscaled, from the pivot down; [CB]: the next diagonal entry ([CB + 1]: dump for
+  // the lanes that do not hold it, which spares the loop a divergent branch)
+  float col[2][CB + 4];
+  float t[CB][CB];  // t[J][i - J] = a_iJ / pivot_J below the pivot, else 0
+  float rs[CB];     // 1 / sqrt(pivot_J)
+};
+template <int ID>
+__device__ __forceinline__ void diag_arrive() { asm volatile("bar.arrive %0, 64;" ::"n"(ID) : "memory"); }
+template <int ID>
+__device__ __forceinline__ void diag_sync() { asm volatile("bar.sync %0, 64;" ::"n"(ID) : "memory"); }
+
+struct DiagState {
+  float piv, rs, next;  // this column's pivot, its reciprocal square root, the next diagonal entry
+  float4 a;             // the column's first four entries from the pivot down
+};
+__device__ __forceinline__ void diag_column(DiagScratch &sc, DiagState &ds, int J, int lane, float v0, float v1) {
+  float *col = sc.col[J & 1];
+  col[(lane - J) & 31] = lane >= J ? v0 : 0.f;
+  col[lane == J + 1 ? CB : CB + 1] = v1;
+  __syncwarp();
+  ds.a = *reinterpret_cast<const float4 *>(col);
+  ds.next = col[CB];
+}
+// Columns 32 - N .. 39 - N: v[0 .. N) hold this lane's row from column 32 - N on.  Every lane also
+// works out the next pivot (the arithmetic of the lane that holds it), and the next column is on its
+// way through shared memory before this one's multiply-adds, which run under both latencies.
+template <int N>
+__device__ __forceinline__ void diag_factor_segment(float (&v)[CB], DiagState &ds, DiagScratch &sc, int lane) {
+#pragma unroll 1
+  for (int J = CB - N; J < CB - N + 8; ++J) {
+    const float *col = sc.col[J & 1];
+    const float4 a = ds.a;
+    const float inv = ds.rs * ds.rs;
+    const float t = lane > J ? v[0] * inv : 0.f;
+    const float v0 = fmaf(-t, a.y, v[1]), v1 = fmaf(-t, a.z, v[2]), v2 = fmaf(-t, a.w, v[3]);
+    sc.rs[J] = ds.rs;
+    ds.piv = fmaf(-(a.y * inv), a.y, ds.next);
+    ds.rs = rsqrtf(ds.piv);
+    diag_column(sc, ds, J + 1, lane, v0, v1);
+    sc.t[J][(lane - J) & 31] = t;
+    v[0] = v0;
+    v[1] = v1;
+    v[2] = v2;
+#pragma unroll
+    for (int q = 1; q < N / 4; ++q) {
+      const float4 b = *reinterpret_cast<const float4 *>(col + 4 * q);
+      v[4 * q - 1] = fmaf(-t, b.x, v[4 * q]);
+      v[4 * q] = fmaf(-t, b.y, v[4 * q + 1]);
+      v[4 * q + 1] = fmaf(-t, b.z, v[4 * q + 2]);
+      v[4 * q + 2] = fmaf(-t, b.w, v[4 * q + 3]);
+    }
+  }
+}
+// v: this lane's row of the block (entries right of the diagonal are not used).  Returns whether
+// every pivot was positive and finite.  ID .. ID + 3: named barriers shared with diag_invert.
+template <int ID>
+__device__ __forceinline__ bool diag_factor(float (&v)[CB], DiagScratch &sc, int lane) {
+  DiagState ds;
+  ds.piv = __shfl_sync(0xffffffffu, v[0], 0);
+  ds.rs = rsqrtf(ds.piv);
+  diag_column(sc, ds, 0, lane, v[0], v[1]);
+  diag_factor_segment<32>(v, ds, sc, lane);
+  diag_arrive<ID>();
+  diag_factor_segment<24>(v, ds, sc, lane);
+  diag_arrive<ID + 1>();
+  diag_factor_segment<16>(v, ds, sc, lane);
+  diag_arrive<ID + 2>();
+  diag_factor_segment<8>(v, ds, sc, lane);
+  diag_arrive<ID + 3>();
+  __syncwarp();
+  const float mine = sc.rs[lane];  // a pivot that is not positive and finite leaves NaN, inf or 0
+  return __all_sync(0xffffffffu, mine > 0.f && mine < INFINITY);
+}
+
+// Rows 32 - N .. 39 - N of the inverse: x[0 .. N) hold this lane's column from row 32 - N on.
+template <int N, int LD>
+__device__ __forceinline__ void diag_invert_segment(float (&x)[CB], const DiagScratch &sc, float *DI, int lane) {
+#pragma unroll 1
+  for (int J = CB - N; J < CB - N + 8; ++J) {
+    const float cur = x[0];
+    DI[J * LD + lane] = cur * sc.rs[J];
+#pragma unroll
+    for (int q = 0; q < N / 4; ++q) {
+      const float4 b = *reinterpret_cast<const float4 *>(sc.t[J] + 4 * q);
+      if (q > 0) x[4 * q - 1] = fmaf(-b.x, cur, x[4 * q]);
+      x[4 * q] = fmaf(-b.y, cur, x[4 * q + 1]);
+      x[4 * q + 1] = fmaf(-b.z, cur, x[4 * q + 2]);
+      x[4 * q + 2] = fmaf(-b.w, cur, x[4 * q + 3]);
+    }
+  }
+}
+// DI <- the inverse of the factor, row-major with row pitch LD.
+template <int ID, int LD>
+__device__ __forceinline__ void diag_invert(const DiagScratch &sc, float *DI, int lane) {
+  float x[CB];
+#pragma unroll
+  for (int c = 0; c < CB; ++c) x[c] = (c == lane) ? 1.f : 0.f;
+  diag_sync<ID>();
+  diag_invert_segment<32, LD>(x, sc, DI, lane);
+  diag_sync<ID + 1>();
+  diag_invert_segment<24, LD>(x, sc, DI, lane);
+  diag_sync<ID + 2>();
+  diag_invert_segment<16, LD>(x, sc, DI, lane);
+  diag_sync<ID + 3>();
+  diag_invert_segment<8, LD>(x, sc, DI, lane);
 }
 
 }  // namespace cd

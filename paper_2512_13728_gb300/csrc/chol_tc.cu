@@ -1,5 +1,5 @@
-// Cholesky factor and inverse of the first CholeskyQR pass (DION_PREC_BF16) with the rank-32
-// trailing update on tcgen05 tensor cores and TMA reduce-adds.
+// Cholesky factor and inverse of the first CholeskyQR pass for ranks above 256 (chol_tmem.cu takes
+// the others) with the rank-32 trailing update on tcgen05 tensor cores and TMA reduce-adds.
 //
 // Same right-looking sweep as chol_inv_kernel (kernels_simt.cu): one CTA of 16 warps per layer
 // builds L^{-1} in place in the L^{-1} buffer W, over 32-wide block columns k (k0 = 32 k).  W
@@ -258,6 +258,7 @@ __global__ void __launch_bounds__(kThreads, 1) chol_inv_tc_kernel(Shared sh, con
   if (!sh.active[l]) return;
   const DevLayer &Ly = sh.layers[l];
   const int r = (int)Ly.r;
+  if (r <= kCholTmemRank) return;  // chol_inv_tmem_kernel's
   const int64_t ls = Ly.ldp;
   const float *S = Ly.S;
   float *Li = Ly.Linv;

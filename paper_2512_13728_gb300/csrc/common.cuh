@@ -186,7 +186,12 @@ void launch_gemm(const Shared &sh, const GemmProblem *probs, const int4 *tiles, 
 cudaError_t prepare_chol_inv(int32_t max_r, size_t *smem_out);
 // near_identity: Frobenius bound on S - I below which passes 1 and 2 use the first-order factor
 void launch_chol_inv(const Shared &sh, size_t smem, int32_t pass, float near_identity, cudaStream_t s);
-// the first CholeskyQR pass with the trailing update on tensor cores (chol_tc.cu, BF16 mode)
+// the first CholeskyQR pass in the tensor-core modes: layers of rank up to kCholTmemRank with the
+// working matrix in tensor memory (chol_tmem.cu), the others with the trailing update on tensor
+// cores (chol_tc.cu); each kernel skips the other's layers
+constexpr int kCholTmemRank = 256;
+cudaError_t prepare_chol_inv_tmem(size_t *smem_out);
+void launch_chol_inv_tmem(const Shared &sh, size_t smem, cudaStream_t s);
 cudaError_t prepare_chol_inv_tc(int32_t max_r, size_t *smem_out);
 namespace tc { struct LayerMaps; }
 void launch_chol_inv_tc(const Shared &sh, const tc::LayerMaps *maps, size_t smem, cudaStream_t s);

@@ -328,7 +328,10 @@ cudaError_t init(const TcLayout &lo, char *base, const DevLayer *dl, int32_t L, 
   if (tp->fuse_buffer && tp->fb_smem > 227u * 1024u) return cudaErrorInvalidValue;
   if (e == cudaSuccess && tp->fuse_buffer) e = setup_fused_bq_kernel(tp->fb_smem);
   if (e == cudaSuccess) e = setup_orth_kernels(tp->o_smem, x3);
+  tp->min_r = lo.max_r;
+  for (int32_t l = 0; l < L; ++l) tp->min_r = std::min<int32_t>(tp->min_r, (int32_t)dl[l].r);
   if (e == cudaSuccess) e = prepare_chol_inv_tc(lo.max_r, &tp->chol_tc_smem);
+  if (e == cudaSuccess) e = prepare_chol_inv_tmem(&tp->chol_tmem_smem);
   int dev = 0, sms = 0;
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -340,6 +343,18 @@ cudaError_t init(const TcLayout &lo, char *base, const DevLayer *dl, int32_t L, 
 int32_t launches_per_step(const TcPlan &tp) { return tp.launches; }
 
 void refresh(const TcPlan &tp, const Shared &sh, cudaStream_t s) { launch_qn_refresh(sh, tp, s); }
+
+// The first pass's Cholesky: one kernel per rank range that the plan has (p: its timing hooks).
+static void launch_chol_first(dion_plan *p, const Shared &sh, const TcPlan &tp, cudaStream_t s) {
+  if (tp.min_r <= kCholTmemRank) {
+    launch_chol_inv_tmem(sh, tp.chol_tmem_smem, s);
+    if (p) tick(p, s, "chol_inv0");
+  }
+  if (tp.max_r > kCholTmemRank) {
+    launch_chol_inv_tc(sh, tp.maps, tp.chol_tc_smem, s);
+    if (p) tick(p, s, "chol_inv0");
+  }
+}
 
 void step(dion_plan *p, const TcPlan &tp, const Shared &sh_in, const StepArgs &a, const int4 *btiles,
           int32_t n_btiles, const int4 *ctiles, int32_t n_ctiles, size_t chol_smem, cudaStream_t s) {
@@ -373,16 +388,19 @@ void step(dion_plan *p, const TcPlan &tp, const Shared &sh_in, const StepArgs &a
     launch_form_bq(sh, tp, s);  // P = B Q_{t-1} on the layers that take the Dion branch
     tick(p, s, "tc_bq");
   }
-  static const char *kChol[3] = {"chol_inv0", "chol_inv1", "chol_inv2"};
+  static const char *kChol[3] = {"", "chol_inv1", "chol_inv2"};
   static const char *kGram[3] = {"tc_gram0", "tc_gram1", "tc_gram2"};
   static const char *kTrsm[3] = {"tc_trsm0", "tc_trsm1", "tc_trsm2"};
   const bool x3 = tp.precision == DION_PREC_BF16X3;
   for (int pass = 0; pass < 3; ++pass) {  // CholeskyQR2; the third pass only after a shifted retry
     launch_orth(sh, tp, true, pass, s);  // S = X^T X
     tick(p, s, kGram[pass]);
-    if (pass == 0) launch_chol_inv_tc(sh, tp.maps, tp.chol_tc_smem, s);  // trailing update on tensor cores (3xTF32)
-    else launch_chol_inv(sh, chol_smem, pass, x3 ? 1e-3f : 6e-2f, s);  // passes 1-2: usually the first-order factor
-    tick(p, s, kChol[pass]);
+    if (pass == 0) {
+      launch_chol_first(p, sh, tp, s);  // trailing update on tensor cores (3xTF32)
+    } else {
+      launch_chol_inv(sh, chol_smem, pass, x3 ? 1e-3f : 6e-2f, s);  // usually the first-order factor
+      tick(p, s, kChol[pass]);
+    }
     launch_orth(sh, tp, false, pass, s);  // X L^{-T} and its transpose, or its bf16 copy (halves) at the end
     tick(p, s, kTrsm[pass]);
   }
@@ -425,7 +443,7 @@ void step_phase(const TcPlan &tp, const Shared &sh_in, const StepArgs &a, int32_
       launch_transpose_praw(sh, tp, s);  // the first Gram reads P_raw^T
       for (int pass = 0; pass < 3; ++pass) {
         launch_orth(sh, tp, true, pass, s);
-        if (pass == 0) launch_chol_inv_tc(sh, tp.maps, tp.chol_tc_smem, s);
+        if (pass == 0) launch_chol_first(nullptr, sh, tp, s);
         else launch_chol_inv(sh, chol_smem, pass, x3 ? 1e-3f : 6e-2f, s);
         launch_orth(sh, tp, false, pass, s);
       }

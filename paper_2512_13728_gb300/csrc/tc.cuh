@@ -98,7 +98,8 @@ struct TcPlan {
   bool fuse_buffer = false;
   bool defers = false;  // some layer leaves B = M + G to the update (unless this step has B in M)
   uint32_t fb_smem = 0;
-  size_t chol_tc_smem = 0;  // the first pass's Cholesky on tensor cores (BF16 mode)
+  size_t chol_tc_smem = 0, chol_tmem_smem = 0;  // the first pass's Cholesky on tensor cores
+  int32_t min_r = 0;
   // CUDA-core pieces reused by this path (set by the plan)
   const GemmProblem *const *probs = nullptr;
   const int4 *const *gtiles = nullptr;

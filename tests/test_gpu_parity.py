@@ -626,3 +626,19 @@ def test_update_pair_tiles(rank, gate):
     w = wl.scaled(wl.WORKLOADS["gpt160m_block_r192"], "pair", [(360, 400), (400, 390), (520, 385)], rank=rank, steps=2)
     mode = oc.GATE_ALWAYS if gate == "always" else oc.GATE_PER_LAYER
     run_per_step(w, PRECS["bf16"], dict(gate_mode=mode), w.steps, TOL_BF16)
+
+
+@pytest.mark.parametrize("prec,tol", [("bf16", TOL_BF16), ("bf16x3", TOL_FP32)])
+@pytest.mark.parametrize("rank", [1, 15, 32, 33, 96, 127, 128, 129, 161, 224, 240, 256])
+def test_cholesky_ranks(rank, prec, tol):
+    """The first pass's Cholesky at the edges of its 32-wide blocks, of its 16-column MMA widths and
+    of its 128-row TMEM blocks."""
+    w = wl.scaled(wl.WORKLOADS["gpt160m_block_r192"], "chol", [(520, 300), (300, 520)], rank=rank, steps=2)
+    run_per_step(w, PRECS[prec], dict(gate_mode=oc.GATE_ALWAYS), w.steps, tol)
+
+
+def test_cholesky_mixed_ranks():
+    """A plan whose layers' ranks lie on both sides of 256 (one kernel each)."""
+    w = wl.scaled(wl.WORKLOADS["gpt160m_block_r192"], "cholmix", [(520, 300), (300, 200), (400, 700), (200, 64)],
+                  rank=300, steps=2)
+    run_per_step(w, PRECS["bf16"], dict(gate_mode=oc.GATE_ALWAYS), w.steps, TOL_BF16)
