@@ -2,6 +2,7 @@
 // FFMA sweep; chol_tc.cu: sweep with the trailing update on tensor cores).
 #pragma once
 
+#include <cstdint>
 #include <cuda_runtime.h>
 
 namespace cd {
@@ -189,6 +190,53 @@ __device__ __forceinline__ void diag_invert(const DiagScratch &sc, float *DI, in
   diag_invert_segment<16, LD>(x, sc, DI, lane);
   diag_sync<ID + 3>();
   diag_invert_segment<8, LD>(x, sc, DI, lane);
+}
+
+// Row i and 16-byte column group j4 (4 j4 <= i) of flat group p of a lower triangle whose rows
+// 4 b .. 4 b + 3 hold b + 1 groups each, 2 b (b + 1) groups before them (p < 2^24: the fp32
+// estimate of b is off by at most one, corrected in integers; 32-bit division).
+__device__ __forceinline__ void lower_group(int64_t p, int &i, int &j4) {
+  const uint32_t pu = (uint32_t)p;
+  uint32_t b = (uint32_t)((sqrtf(2.f * (float)pu + 1.f) - 1.f) * 0.5f);
+  while (2u * (b + 1u) * (b + 2u) <= pu) ++b;
+  while (b > 0u && 2u * b * (b + 1u) > pu) --b;
+  const uint32_t off = pu - 2u * b * (b + 1u), q = off / (b + 1u);
+  i = (int)(4u * b + q);
+  j4 = (int)(off - q * (b + 1u));
+}
+
+// S (lower triangle) += its other `parts` - 1 partial sums, `stride` floats apart, in order, by a
+// block of THREADS threads; visible to the whole block on return.
+template <int THREADS>
+__device__ __forceinline__ void sum_gram_parts(float *S, int r, int64_t ls, int parts, int64_t stride) {
+  if (parts <= 1) return;
+  const int nb4 = r / 4, groups = 2 * nb4 * (nb4 + 1) + (r % 4) * (nb4 + 1);
+  constexpr int U = 4;  // groups in flight per thread and part
+  for (int g0 = threadIdx.x; g0 < groups; g0 += THREADS * U) {
+    float4 a[U];
+    float *p[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      int i = 0, j4 = 0;
+      if (g0 + u * THREADS < groups) lower_group(g0 + u * THREADS, i, j4);
+      p[u] = S + (int64_t)i * ls + 4 * j4;
+      a[u] = *reinterpret_cast<const float4 *>(p[u]);
+    }
+#pragma unroll 2
+    for (int q = 1; q < parts; ++q) {
+      float4 b[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) b[u] = *reinterpret_cast<const float4 *>(p[u] + q * stride);
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        a[u].x += b[u].x; a[u].y += b[u].y; a[u].z += b[u].z; a[u].w += b[u].w;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (g0 + u * THREADS < groups) *reinterpret_cast<float4 *>(p[u]) = a[u];
+  }
+  __syncthreads();
 }
 
 }  // namespace cd

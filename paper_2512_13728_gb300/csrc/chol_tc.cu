@@ -109,7 +109,7 @@ __device__ __forceinline__ void issue_unit(const TcState &ts, uint32_t g, int a0
 
 // 0: factored; 1: a pivot was not positive and finite (uniform over the block); 2: a wait for
 // the tensor cores gave up.
-__device__ int chol_inverse_tc(const float *__restrict__ S, float *__restrict__ W, int r, int64_t ls, float shift,
+__device__ int chol_inverse_tc(const float *S, float *__restrict__ W, int r, int64_t ls, float shift,
                                float *D, float *DI, float *rd, int *bad, TcState &ts, int32_t *status) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, q = tid - 32;
   // W <- lower triangle of S + shift I (coalesced; the upper triangle is never read before each
@@ -280,6 +280,7 @@ __global__ void __launch_bounds__(kThreads, 1) chol_inv_tc_kernel(Shared sh, con
   __shared__ double red[kThreads / 32];
   __shared__ double trace_s;
   const int tid = threadIdx.x;
+  sum_gram_parts<kThreads>(Ly.S, r, ls, Ly.s_parts, Ly.s_stride);
   if (tid == 0) {
     for (int i = 0; i < 3; ++i) mbar_init(&ts.bars[i], 1);
     fence_mbar_init();

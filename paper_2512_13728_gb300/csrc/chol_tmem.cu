@@ -114,22 +114,25 @@ __device__ __forceinline__ void issue(const State &st, int b, int n0, int nn, bo
 
 // 0: factored; 1: a pivot was not positive and finite (uniform over the block); 2: a wait for the
 // tensor cores gave up.
-__device__ int sweep(const float *__restrict__ S, float *__restrict__ W, int r, int64_t ls, float shift, State &st,
+__device__ int sweep(const float *S, const float *S2, float *__restrict__ W, int r, int64_t ls, float shift, State &st,
                      int32_t *status) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int rw = warp & 7, row = 32 * rw + lane;  // the rows whose TMEM lanes this warp can reach
   const uint32_t lanes = (uint32_t)(32 * (warp & 3)) << 16;
   const int nblk = (r + CB - 1) / CB;
-  // W <- lower triangle of S + shift I; zeros past r.  Warps rw and rw + 8 share the 32-column
+  // W <- lower triangle of S (+ S2) + shift I; zeros past r.  Warps rw and rw + 8 share the 32-column
   // chunks of rows 32 rw ..; the columns right of the diagonal chunk are never read.
   for (int c = warp >> 3; c <= rw && rw < yt_rows(r) / 32; c += 2) {
     float v[32];
 #pragma unroll
     for (int g = 0; g < 8; ++g) {
       const int j = 32 * c + 4 * g;
-      float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (row < r && j < r) x = *reinterpret_cast<const float4 *>(S + (int64_t)row * ls + j);  // pitch: a multiple of 8
-      v[4 * g] = x.x; v[4 * g + 1] = x.y; v[4 * g + 2] = x.z; v[4 * g + 3] = x.w;
+      float4 x = make_float4(0.f, 0.f, 0.f, 0.f), y = x;
+      if (row < r && j < r) {  // pitch: a multiple of 8
+        x = *reinterpret_cast<const float4 *>(S + (int64_t)row * ls + j);
+        if (S2 != nullptr) y = *reinterpret_cast<const float4 *>(S2 + (int64_t)row * ls + j);
+      }
+      v[4 * g] = x.x + y.x; v[4 * g + 1] = x.y + y.y; v[4 * g + 2] = x.z + y.z; v[4 * g + 3] = x.w + y.w;
     }
 #pragma unroll
     for (int e = 0; e < 32; ++e) {
@@ -257,6 +260,10 @@ __global__ void __launch_bounds__(kThreads, 1) chol_inv_tmem_kernel(Shared sh) {
   st.bad = &bad;
   st.gave_up = &gave_up;
   const uint32_t cols = r <= 128 ? 128u : 512u;
+  // two partial sums are added on their way into TMEM; more, in a pass of their own (its coalesced
+  // reads keep more in flight: eight parts at r = 192 cost 8 us, added on the way 20)
+  const float *S2 = Ly.s_parts == 2 ? S + Ly.s_stride : nullptr;
+  if (Ly.s_parts > 2) sum_gram_parts<kThreads>(Ly.S, r, ls, Ly.s_parts, Ly.s_stride);
   if (tid == 0) {
     for (int i = 0; i < 3; ++i) mbar_init(&bars_s[i], 1);
     gave_up = 0;
@@ -281,11 +288,12 @@ __global__ void __launch_bounds__(kThreads, 1) chol_inv_tmem_kernel(Shared sh) {
   float shift = 0.f;
 #pragma unroll 1
   for (;;) {
-    res = sweep(S, Li, r, ls, shift, st, sh.status);
+    res = sweep(S, S2, Li, r, ls, shift, st, sh.status);
     if (res != 1 || shifted) break;
     // a retry from S + s I (shifted CholeskyQR, as in chol_inv_kernel)
     double tr = 0.0;
-    for (int i = tid; i < r; i += kThreads) tr += (double)S[(int64_t)i * ls + i];
+    for (int i = tid; i < r; i += kThreads)
+      tr += (double)S[(int64_t)i * ls + i] + (S2 != nullptr ? (double)S2[(int64_t)i * ls + i] : 0.0);
     tr = block_sum<kThreads>(tr, red);
     if (tid == 0) trace_s = tr;
     __syncthreads();

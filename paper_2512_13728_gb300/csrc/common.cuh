@@ -70,7 +70,11 @@ struct DevLayer {
   float *P_raw;  // m x r (ld ldp)  P = B Q before orthogonalization
   float *P;      // m x r (ld ldp)  orthonormal P
   float *R;      // n x r (ld ldp)  R = B^T P
-  float *S;      // r x r (ld ldp)  Gram X^T X; lower triangle becomes the Cholesky factor L
+  // r x r (ld ldp)  Gram X^T X (lower triangle); in the tensor-core modes s_parts partial sums over
+  // row ranges of X, s_stride floats apart, which the Cholesky kernels add up into the first
+  float *S;
+  int32_t s_parts;
+  int64_t s_stride;
   float *Linv;   // r x r (ld ldp)  L^{-1} (lower triangular, zeros above the diagonal)
   // tensor-core operand copies (bf16, rows of pitch ldp unless stated); null in FP32 mode
   __nv_bfloat16 *P_hi;   // m x r : P

@@ -504,19 +504,6 @@ void launch_gemm(const Shared &sh, const GemmProblem *probs, const int4 *tiles, 
 constexpr int kCholThreads = 512;
 constexpr int kFoBatch = 8;  // 16-byte groups each thread has in flight in the first-order factor
 
-// Row i and 16-byte column group j4 (4 j4 <= i) of flat group p of a lower triangle whose rows
-// 4 b .. 4 b + 3 hold b + 1 groups each, 2 b (b + 1) groups before them (p < 2^24: the fp32
-// estimate of b is off by at most one, corrected in integers; 32-bit division).
-__device__ __forceinline__ void lower_group(int64_t p, int &i, int &j4) {
-  const uint32_t pu = (uint32_t)p;
-  uint32_t b = (uint32_t)((sqrtf(2.f * (float)pu + 1.f) - 1.f) * 0.5f);
-  while (2u * (b + 1u) * (b + 2u) <= pu) ++b;
-  while (b > 0u && 2u * b * (b + 1u) > pu) --b;
-  const uint32_t off = pu - 2u * b * (b + 1u), q = off / (b + 1u);
-  i = (int)(4u * b + q);
-  j4 = (int)(off - q * (b + 1u));
-}
-
 // Column c of Y lives at ysw(c): bit 2 flips when bit 5 is set, so the two 16-byte halves of
 // an 8-column group swap in every other 32-column stretch.  Eight consecutive groups read by
 // one quarter-warp then fall on distinct banks.
@@ -531,7 +518,7 @@ __device__ __forceinline__ void load8y(const float *row, int c0, float w[8]) {  
 // over the block, on a pivot that is not positive and finite.  Shared memory: D (CB x CBP),
 // DI (CB x CB), rd (CB reciprocal pivots), Y (CB x ldy, ldy >= r rounded up to 8, columns
 // >= r zero).
-__device__ bool chol_inverse(const float *__restrict__ S, float *__restrict__ W, int r, int64_t ls, float shift,
+__device__ bool chol_inverse(const float *S, float *__restrict__ W, int r, int64_t ls, float shift,
                              float *D, float *DI, float *rd, float *Y, int ldy, int *bad) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, q = tid - 32;
   for (int k0 = 0; k0 < r; k0 += CB) {
@@ -651,7 +638,7 @@ __device__ bool chol_inverse(const float *__restrict__ S, float *__restrict__ W,
 // reduce-scatter over the lanes) and, off the diagonal, its column sums into its own partial
 // vector; the partials are then summed in warp order, so the estimate is deterministic.
 // Shared memory: Y (at least 18 rows of ldy floats).  Called by the whole block.
-__device__ __noinline__ float power_norm_sym(const float *__restrict__ S, int r, int64_t ls, float *Y, int ldy) {
+__device__ __noinline__ float power_norm_sym(const float *S, int r, int64_t ls, float *Y, int ldy) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   __shared__ float wn[kCholThreads / 32];
   __shared__ float lam_s;
@@ -738,6 +725,7 @@ __global__ void __launch_bounds__(kCholThreads, 1) chol_inv_kernel(Shared sh, in
   const int64_t ls = Ly.ldp;  // leading dimension of S and L^{-1} (a multiple of 8)
   const float *S = Ly.S;
   float *Li = Ly.Linv;
+  sum_gram_parts<kCholThreads>(Ly.S, r, ls, Ly.s_parts, Ly.s_stride);
   extern __shared__ __align__(16) float smem[];
   float *D = smem;                 // CB x CBP
   float *rd = D + CB * CBP;        // CB

@@ -217,6 +217,8 @@ dion_status dion_plan_create(const dion_layer *layers, int32_t num_layers, int32
     p->xr_off = o_R[0];
     p->xr_count = (int64_t)((o_R[num_layers - 1] - o_R[0]) / sizeof(float)) + a.n * lp;
   }
+  const std::vector<int32_t> s_parts = precision == DION_PREC_FP32 ? std::vector<int32_t>(num_layers, 1)
+                                                                   : tc::gram_parts(layers, num_layers, sms);
   const int64_t tile_elems = row_tile_elems(layers, num_layers, sms);
   for (int32_t l = 0; l < num_layers; ++l) {
     const dion_layer &ly = layers[l];
@@ -232,7 +234,10 @@ dion_status dion_plan_create(const dion_layer *layers, int32_t num_layers, int32
     d.ldp = (int32_t)((ly.r + 7) / 8 * 8);
     p->max_r = std::max<int32_t>(p->max_r, (int32_t)ly.r);
     o_P[l] = cv.take<float>(ly.m * d.ldp);
-    o_S[l] = cv.take<float>(ly.r * d.ldp);
+    // parts start at multiples of the Gram's 128-row output tiles, whose rows past r hold zeros
+    d.s_parts = s_parts[l];
+    d.s_stride = (ly.r + 127) / 128 * 128 * d.ldp;
+    o_S[l] = cv.take<float>((d.s_parts - 1) * d.s_stride + ly.r * d.ldp);
     o_Li[l] = cv.take<float>(ly.r * d.ldp);
     // row tiles of the buffer, norms and local kernels
     const int64_t rows = std::max<int64_t>(1, std::min<int64_t>(ly.m, tile_elems / ly.n));

@@ -6,6 +6,7 @@
 #include "tc_kernels.cuh"
 
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 
 namespace cd {
@@ -39,6 +40,7 @@ Schedule lpt(const std::vector<int4> &tiles, const std::vector<double> &cost, in
     load[best] += cost[i];
     per[best].push_back(i);
   }
+  sc.makespan = *std::max_element(load.begin(), load.end());
   sc.off.push_back(0);
   for (int c = 0; c < sc.grid; ++c) {
     for (int i : per[c]) sc.tiles.push_back(tiles[i]);
@@ -47,6 +49,43 @@ Schedule lpt(const std::vector<int4> &tiles, const std::vector<double> &cost, in
   return sc;
 }
 }  // namespace
+
+// The Gram sums over the m rows of X in 32-row chunks, one pair tile per layer (two at r > 256), and
+// a long layer's tile, or a plan with few tiles, would leave most CTA pairs idle: layers are split
+// into row ranges of at most T chunks.  T (the longest layer's chunks over 1 .. 8) is the one with
+// the smallest estimate, in chunk times (0.45 us): the longest-processing-time makespan of the
+// tiles, each with 4 chunk times for its start and end, plus 3.3 (r / 256)^2 for each further
+// partial sum that a Cholesky CTA has to read.  A pass, unsplit / split: 47 / 16 us on the 160M
+// block (18 of 76 pairs busy with the ranges, 6 without), 50 / 35 us on its stack at rank 192, 47 / 26
+// at rank 48, 231 / 175 us on the 350M stack with split operands; the 1.3B stack stays unsplit.
+std::vector<int32_t> gram_parts(const dion_layer *layers, int32_t L, int num_sms) {
+  int64_t longest = 1;
+  for (int32_t l = 0; l < L; ++l) longest = std::max<int64_t>(longest, (layers[l].m + 31) / 32);
+  std::vector<int32_t> best(L, 1), parts(L, 1);
+  double best_cost = INFINITY;
+  for (int n = 1; n <= 8; ++n) {
+    const int64_t T = std::max<int64_t>(1, (longest + n - 1) / n);
+    std::vector<int4> tiles;
+    std::vector<double> cost;
+    double sums = 0.0;
+    for (int32_t l = 0; l < L; ++l) {
+      const int64_t chunks = (layers[l].m + 31) / 32, q = (chunks + T - 1) / T, per = (chunks + q - 1) / q;
+      parts[l] = (int32_t)((chunks + per - 1) / per);  // none empty
+      const double rr = (double)layers[l].r / 256.0;
+      sums = std::max(sums, (parts[l] - 1) * 3.3 * rr * rr);
+      for (int32_t i = 0; i < parts[l] * (layers[l].r > 256 ? 2 : 1); ++i) {
+        tiles.push_back(make_int4(l, 0, 0, 0));
+        cost.push_back((double)per + 4.0);
+      }
+    }
+    const double c = lpt(tiles, cost, std::max(num_sms / 2, 1)).makespan + sums;
+    if (c < best_cost) {
+      best_cost = c;
+      best = parts;
+    }
+  }
+  return best;
+}
 
 dion_status layout(const dion_layer *layers, int32_t L, int32_t precision, int num_sms, size_t start,
                    TcLayout *out) {
@@ -57,6 +96,7 @@ dion_status layout(const dion_layer *layers, int32_t L, int32_t precision, int n
     if (layers[l].r > 256) return DION_ERR_UNSUPPORTED;
   TcLayout &lo = *out;
   lo.precision = precision;
+  const std::vector<int32_t> parts = gram_parts(layers, L, num_sms);
   size_t off = start;
   auto take = [&](size_t bytes, size_t align = 256) {  // a region and its guard words
     off = (off + align - 1) / align * align;
@@ -102,7 +142,13 @@ dion_status layout(const dion_layer *layers, int32_t L, int32_t precision, int n
     lo.o_pt[l] = take(ly.r * ldmt * 4);
     lo.o_colsq[l] = take((size_t)((ly.n + 127) / 128) * ldp * 8);
     lo.o_colinv[l] = take(ldp * 4);
-    for (int64_t rb = 0; rb < (ly.r + 127) / 128; ++rb) lo.gram_tiles.push_back(make_int4(l, (int)rb, 0, 0));
+    {  // {layer, pair tile | part << 8, first 32-row chunk, chunks}
+      const int64_t chunks = (ly.m + 31) / 32, per = (chunks + parts[l] - 1) / parts[l];
+      for (int32_t q = 0; q < parts[l]; ++q)
+        for (int p = 0; p < (ly.r > 256 ? 2 : 1); ++p)
+          lo.gram_tiles.push_back(make_int4(l, p | (q << 8), (int)(q * per),
+                                            (int)std::min<int64_t>(per, chunks - q * per)));
+    }
     for (int64_t mb = 0; mb < (ly.m + 127) / 128; ++mb) lo.trsm_tiles.push_back(make_int4(l, (int)mb, 0, 0));
     for (int64_t mb = 0; mb < (ly.m + 127) / 128; ++mb)
       for (int64_t nb = 0; nb < (ly.n + 127) / 128; ++nb)
@@ -138,7 +184,7 @@ dion_status layout(const dion_layer *layers, int32_t L, int32_t precision, int n
   lo.s_btp = pair_sched(pairs_of(lo.rtiles), [&](const int4 &t) { return (double)layers[t.x].m + 2.0 * layers[t.x].r; });
   // equal cost for every tile of a layer (at r > 256 both load two boxes per chunk), so that
   // they run side by side and stream the layer's X^T from DRAM about once
-  lo.s_gram = pair_sched(pairs_of(lo.gram_tiles), [&](const int4 &t) { return (double)layers[t.x].m * layers[t.x].r; });
+  lo.s_gram = pair_sched(lo.gram_tiles, [&](const int4 &t) { return (double)t.w + 4.0; });
   lo.s_trsm = pair_sched(pairs_of(lo.trsm_tiles), [&](const int4 &t) { return 3.0 * layers[t.x].r + 64.0; });
   for (Schedule *sc : {&lo.s_update, &lo.s_bq, &lo.s_btp, &lo.s_gram, &lo.s_trsm}) {
     sc->o_tiles = take(sizeof(int4) * std::max<size_t>(sc->tiles.size(), 1));
@@ -148,7 +194,6 @@ dion_status layout(const dion_layer *layers, int32_t L, int32_t precision, int n
   lo.o_utiles = take(sizeof(int4) * std::max<size_t>(lo.utiles.size(), 1));
   lo.o_rtiles = take(sizeof(int4) * std::max<size_t>(lo.rtiles.size(), 1));
   lo.o_qtiles = take(sizeof(int4) * std::max<size_t>(lo.qtiles.size(), 1));
-  lo.o_gtiles = take(sizeof(int4) * std::max<size_t>(lo.gram_tiles.size(), 1));
   lo.o_ttiles = take(sizeof(int4) * std::max<size_t>(lo.trsm_tiles.size(), 1));
   lo.fuse_buffer = L > 0 && !x3;  // BF16X3 forms B and its two bf16 halves in the buffer pass
   for (int32_t l = 0; l < L; ++l) lo.fuse_buffer = lo.fuse_buffer && layers[l].g_dtype == DION_DTYPE_BF16;
@@ -207,8 +252,6 @@ void bind(const TcLayout &lo, char *base, DevLayer *dl, int32_t L, TcPlan *tp) {
   tp->n_rtiles = (int32_t)lo.rtiles.size();
   tp->qtiles = reinterpret_cast<int4 *>(base + lo.o_qtiles);
   tp->n_qtiles = (int32_t)lo.qtiles.size();
-  tp->gram_tiles = reinterpret_cast<int4 *>(base + lo.o_gtiles);
-  tp->n_gram_tiles = (int32_t)lo.gram_tiles.size();
   tp->trsm_tiles = reinterpret_cast<int4 *>(base + lo.o_ttiles);
   tp->n_trsm_tiles = (int32_t)lo.trsm_tiles.size();
   tp->precision = lo.precision;
@@ -250,7 +293,7 @@ cudaError_t encode_maps(const DevLayer *dl, int32_t L, LayerMaps *dst) {
                     encode_f32_2d(&m.PT, d.PT, d.m, d.r, (uint64_t)d.ldmt * 4, 32, 128) &&
                     encode_f32_2d(&m.PTraw_t, d.PT_raw, d.m, d.r, (uint64_t)d.ldmt * 4, 32, 32) &&
                     encode_f32_2d(&m.PT_t, d.PT, d.m, d.r, (uint64_t)d.ldmt * 4, 32, 32) &&
-                    encode_f32_2d(&m.Sst, d.S, d.r, d.r, p32, 32, 128) &&
+                    encode_f32_2d(&m.Sst, d.S, d.r, (d.s_parts - 1) * (d.s_stride / d.ldp) + d.r, p32, 32, 128) &&
                     encode_f32_2d(&m.Linv, d.Linv, d.r, d.r, p32, 32, 128) &&
                     encode_f32_2d(&m.Linv32, d.Linv, d.r, d.r, p32, 32, 32) &&
                     (d.P_lo == nullptr ||
@@ -279,7 +322,6 @@ cudaError_t init(const TcLayout &lo, char *base, const DevLayer *dl, int32_t L, 
   if (e == cudaSuccess) e = up(tp->utiles, lo.utiles);
   if (e == cudaSuccess) e = up(tp->rtiles, lo.rtiles);
   if (e == cudaSuccess) e = up(tp->qtiles, lo.qtiles);
-  if (e == cudaSuccess) e = up(tp->gram_tiles, lo.gram_tiles);
   if (e == cudaSuccess) e = up(tp->trsm_tiles, lo.trsm_tiles);
   for (const Schedule *sc : {&lo.s_update, &lo.s_bq, &lo.s_btp, &lo.s_gram, &lo.s_trsm}) {
     if (e == cudaSuccess && !sc->tiles.empty())

@@ -32,7 +32,7 @@ struct LayerMaps {
   CUtensorMap PT;     // r x m fp32 (P^T):    box {32, 128}  Gram operands
   CUtensorMap PTraw_t;  // r x m fp32: box {32, 32}  transposed output store
   CUtensorMap PT_t;     // r x m fp32: box {32, 32}  transposed output store
-  CUtensorMap Sst;    // r x r fp32:  box {32, 128}  Gram output
+  CUtensorMap Sst;    // r x r fp32 per part, parts one below the other:  box {32, 128}  Gram output
   CUtensorMap Linv;   // r x r fp32:  box {32, 128}  TRSM B operand (rows of L^{-1})
   CUtensorMap Linv32; // r x r fp32:  box {32, 32}   Cholesky trailing update (reduce-add)
   // BF16X3: the low halves, boxes as their high counterparts (zeroed maps in the other modes)
@@ -49,6 +49,7 @@ struct Schedule {
   std::vector<int4> tiles;
   std::vector<int> off;
   int grid = 0;
+  double makespan = 0.0;  // cost of the most loaded CTA
   size_t o_tiles = 0, o_off = 0;  // workspace offsets
 };
 
@@ -56,7 +57,7 @@ struct TcLayout {
   Schedule s_update, s_bq, s_btp, s_gram, s_trsm;
   size_t end = 0;
   size_t o_maps = 0;
-  size_t o_utiles = 0, o_rtiles = 0, o_qtiles = 0, o_gtiles = 0, o_ttiles = 0;
+  size_t o_utiles = 0, o_rtiles = 0, o_qtiles = 0, o_ttiles = 0;
   std::vector<size_t> o_phi, o_rhi, o_qnhi, o_bh, o_ptraw, o_pt, o_colsq, o_colinv;
   std::vector<size_t> o_bl, o_plo, o_rlo, o_qnlo;  // BF16X3 low halves
   std::vector<uint64_t> guards;  // offsets of the guard words after each region
@@ -85,8 +86,6 @@ struct TcPlan {
   int32_t n_rtiles = 0;
   int4 *qtiles = nullptr;
   int32_t n_qtiles = 0;
-  int4 *gram_tiles = nullptr;
-  int32_t n_gram_tiles = 0;
   int4 *trsm_tiles = nullptr;
   int32_t n_trsm_tiles = 0;
   int32_t max_r = 0;
@@ -108,6 +107,8 @@ struct TcPlan {
   int32_t n_utiles_simt = 0;
 };
 
+// Number of row ranges each layer's Gram is split into.
+std::vector<int32_t> gram_parts(const dion_layer *layers, int32_t L, int num_sms);
 // Workspace needs of the tensor-core path, appended after `start`.
 dion_status layout(const dion_layer *layers, int32_t L, int32_t precision, int num_sms, size_t start,
                    TcLayout *out);

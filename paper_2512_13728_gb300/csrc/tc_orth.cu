@@ -7,7 +7,9 @@
 //          the previous TRSM) writes next to X.  r <= 256: one pair tile.  r > 256: one tile for
 //          the two diagonal 256 x 256 blocks, whose A operands are read in place from their B
 //          boxes, and one for the block below the first; each loads two boxes per chunk, so a
-//          layer's tiles cost the same, run side by side and read X^T from DRAM about once.
+//          layer's tiles cost the same, run side by side and read X^T from DRAM about once.  A tile
+//          covers a range of X's rows (all of them, or one of the layer's s_parts ranges, whose
+//          partial sums of S the Cholesky kernel adds up in order).
 //   TRSM   Y = X L^{-T} (m x r).  Tile = 128 rows of X; K loop over r.  A = rows of X
 //          (K-major), B = rows of L^{-1} (K-major, lower triangular: K chunks above a column
 //          part are skipped).  Epilogue stores Y (row-major) and Y^T (transposed boxes) for
@@ -137,7 +139,7 @@ __device__ __forceinline__ bool part_needs(int kc, uint32_t part) {
 template <int KIND, bool X3>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(X3 ? O_THREADS_X3 : O_THREADS, 1)
     tc_orth_kernel(Shared sh, const int4 *__restrict__ tiles, const int *__restrict__ off, const LayerMaps *__restrict__ maps,
-                   int pass, int nstages, uint32_t stage_bytes, uint32_t tmem_cols) {
+                   int pass, int nstages, uint32_t stage_bytes, uint32_t tmem_cols, uint32_t slots) {
   if (sh.gate_scratch[kScratchActive] == 0ull) return;  // no layer takes the Dion branch
   if (pass == 2 && sh.gate_scratch[kScratchShifted] == 0ull) return;  // no layer took the shifted retry
   extern __shared__ uint8_t smem_raw[];
@@ -145,7 +147,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(X3 ? O_THREADS_X3 : 
   uint8_t *stg = smem + nstages * stage_bytes;  // 2 x (row box 16 KB + 4 transposed boxes 16 KB)
   uint64_t *bars = reinterpret_cast<uint64_t *>(stg + 4 * O_BOX);
   uint64_t *full = bars, *empty = bars + nstages;
-  // two accumulator slots (the TRSM alternates them; the Gram uses slot 0)
+  // two accumulator slots (the TRSM alternates them, and so does the Gram of a plan whose ranks fit
+  // 256 columns: `slots` = 2; else its tiles take both as one)
   uint64_t *acc_full = bars + 2 * nstages, *acc_empty = acc_full + 2, *drain = acc_full + 4;
   uint64_t *conv = drain + 1;  // BF16X3: a stage's boxes are split in both CTAs (used in CTA 0)
   const uint32_t lo_off = X3 ? stage_bytes / 2u : 0u;  // BF16X3: lo boxes, same layout as the hi half
@@ -222,8 +225,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(X3 ? O_THREADS_X3 : 
           }
           continue;
         }
-        const GramTile g = gram_tile(L.r, t.y);
-        for (int kc = 0; kc < kch; ++kc, ++it) {
+        const GramTile g = gram_tile(L.r, t.y & 0xff);
+        for (int kc = t.z; kc < t.z + t.w; ++kc, ++it) {
           const uint32_t s = it % nstages, ph = (it / nstages) & 1u;
           if (!ab.wait(&empty[s], ph ^ 1u, sh.status)) { ok = false; break; }
           uint8_t *sA = smem + s * stage_bytes, *sB = sA + O_BOX;
@@ -289,8 +292,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(X3 ? O_THREADS_X3 : 
         }
         continue;
       }
-      const GramTile g = gram_tile(L.r, t.y);
-      for (int kc = 0; kc < kch; ++kc, ++it) {
+      const GramTile g = gram_tile(L.r, t.y & 0xff);
+      for (int kc = t.z; kc < t.z + t.w; ++kc, ++it) {
         const uint32_t s = it % nstages, ph = (it / nstages) & 1u;
         if (!named_and(2, 128, ab.wait(&full[s], ph, sh.status))) { ok = false; break; }
         uint8_t *sA = smem + s * stage_bytes, *sB = sA + O_BOX;
@@ -343,10 +346,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(X3 ? O_THREADS_X3 : 
           }
           continue;
         }
-        const GramTile g = gram_tile(L.r, t.y);
-        if (!ab.wait(acc_empty, (tcount & 1u) ^ 1u, sh.status)) break;
+        const GramTile g = gram_tile(L.r, t.y & 0xff);
+        const uint32_t slot = slots == 2u ? (tcount & 1u) : 0u;
+        const uint32_t aph = slots == 2u ? ((tcount >> 1) & 1u) : (tcount & 1u);
+        if (!ab.wait(&acc_empty[slot], aph ^ 1u, sh.status)) break;
         tc_fence_after();
-        for (int kc = 0; kc < kch; ++kc, ++it) {
+        const uint32_t d0 = tmem + slot * 256u;
+        for (int kc = 0; kc < t.w; ++kc, ++it) {
           const uint32_t s = it % nstages, ph = (it / nstages) & 1u;
           if (!ab.wait(X3 ? &conv[s] : &full[s], ph, sh.status)) { ok = false; break; }
           tc_fence_after();
@@ -361,17 +367,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(X3 ? O_THREADS_X3 : 
               const uint32_t idesc = idesc_tf32(256, g.N[q], false, false);
               const uint64_t bd = smem_desc_sw128(bB + q * O_BOX + k8 * 32, 0, 1024);
               // the first chunk that feeds a part starts its accumulation
-              umma_pair_tf32(tmem + q * 256u, ad, bd, idesc, (kc | k8) ? 1u : 0u);
+              umma_pair_tf32(d0 + q * 256u, ad, bd, idesc, (kc | k8) ? 1u : 0u);
               if (X3) {  // hi.lo + lo.hi
-                umma_pair_tf32(tmem + q * 256u, ad, smem_desc_sw128(bB + lo_off + q * O_BOX + k8 * 32, 0, 1024), idesc, 1u);
-                umma_pair_tf32(tmem + q * 256u, smem_desc_sw128(aSrc + lo_off + k8 * 32, 0, 1024), bd, idesc, 1u);
+                umma_pair_tf32(d0 + q * 256u, ad, smem_desc_sw128(bB + lo_off + q * O_BOX + k8 * 32, 0, 1024), idesc, 1u);
+                umma_pair_tf32(d0 + q * 256u, smem_desc_sw128(aSrc + lo_off + k8 * 32, 0, 1024), bd, idesc, 1u);
               }
             }
           }
           umma_pair_commit_mc(&empty[s], 0x3);  // the stage is free in both CTAs
         }
         if (!ok) break;
-        umma_pair_commit_mc(acc_full, 0x3);
+        umma_pair_commit_mc(&acc_full[slot], 0x3);
         ++tcount;
       }
       umma_pair_commit(drain);  // every MMA of the pair has completed before TMEM is freed
@@ -392,7 +398,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(X3 ? O_THREADS_X3 : 
       orth_dims<KIND>(L, t.y, N, K);
       const int tr = 2 * t.y + (int)rank;
       const bool real = (int64_t)tr * 128 < L.m;  // TRSM: not the pair's empty second tile
-      const GramTile g = gram_tile(L.r, KIND == ORTH_GRAM ? t.y : 0);
+      const GramTile g = gram_tile(L.r, KIND == ORTH_GRAM ? (t.y & 0xff) : 0);
+      // first row of S of this tile's part (in 128-row tiles)
+      const int part_row = KIND == ORTH_GRAM ? (t.y >> 8) * (int)((L.r + 127) / 128) : 0;
       const int nch = (KIND == ORTH_GRAM) ? g.nch : real ? (int)((min((int64_t)N, L.r) + 31) / 32) : 0;
       // The solve that ends Orthogonalize writes only the bf16 copy of P that R = B^T P and the
       // update read: pass 1 unless a shifted retry asked for pass 2, and pass 2 itself.
@@ -402,8 +410,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(X3 ? O_THREADS_X3 : 
       const uint32_t nsub = (KIND == ORTH_TRSM) ? (N + 255) / 256 : 1u;
       bool stop = false;
       for (uint32_t q = 0; q < nsub; ++q) {
-        const uint32_t slot = (KIND == ORTH_TRSM) ? (tcount & 1u) : 0u;
-        const uint32_t aph = (KIND == ORTH_TRSM) ? ((tcount >> 1) & 1u) : (tcount & 1u);
+        const bool alt = KIND == ORTH_TRSM || slots == 2u;
+        const uint32_t slot = alt ? (tcount & 1u) : 0u, aph = alt ? ((tcount >> 1) & 1u) : (tcount & 1u);
         if (!named_and(1, 128, ab.wait(&acc_full[slot], aph, sh.status))) { stop = true; break; }
         tc_fence_after();
         // output chunks jb .. je - 1 (32 columns each); chunk j sits at TMEM column
@@ -492,7 +500,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(X3 ? O_THREADS_X3 : 
             fence_async_smem();
             named_sync(1, 128);
             if (leader) {
-              tma_store_2d(om.out, box, j * 32, otr * 128);
+              tma_store_2d(om.out, box, j * 32, (part_row + otr) * 128);
               if (store_t)
                 for (int w4 = 0; w4 < 4; ++w4)
                   if ((int64_t)tr * 128 + w4 * 32 < L.m)
@@ -539,18 +547,20 @@ void launch_orth(const Shared &sh, const TcPlan &tp, bool gram, int pass, cudaSt
   const uint32_t f = x3 ? 2u : 1u;  // BF16X3 stages hold the lo boxes too
   const uint32_t stage = f * O_BOX * (1 + tp.o_parts), tstage = f * 2u * O_BOX;  // TRSM: A box + one B box
   const int g = 2 * d.grid;
+  // two accumulator slots for the Gram where its tiles need at most 256 columns
+  const uint32_t slots = tp.max_r <= 256 ? 2u : 1u, gcols = slots == 2u ? 512u : tp.tmem_cols;
   if (gram && x3)
     tc_orth_kernel<ORTH_GRAM, true><<<g, O_THREADS_X3, tp.o_smem, s>>>(sh, d.tiles, d.off, tp.maps, pass,
-                                                                        tp.o_stages, stage, tp.tmem_cols);
+                                                                        tp.o_stages, stage, gcols, slots);
   else if (gram)
     tc_orth_kernel<ORTH_GRAM, false><<<g, O_THREADS, tp.o_smem, s>>>(sh, d.tiles, d.off, tp.maps, pass,
-                                                                      tp.o_stages, stage, tp.tmem_cols);
+                                                                      tp.o_stages, stage, gcols, slots);
   else if (x3)  // two 256-column accumulator slots
     tc_orth_kernel<ORTH_TRSM, true><<<g, O_THREADS_X3, tp.o_smem, s>>>(sh, d.tiles, d.off, tp.maps, pass,
-                                                                        tp.t_stages, tstage, 512u);
+                                                                        tp.t_stages, tstage, 512u, 2u);
   else
     tc_orth_kernel<ORTH_TRSM, false><<<g, O_THREADS, tp.o_smem, s>>>(sh, d.tiles, d.off, tp.maps, pass,
-                                                                      tp.t_stages, tstage, 512u);
+                                                                      tp.t_stages, tstage, 512u, 2u);
 }
 
 }  // namespace tc

@@ -642,3 +642,12 @@ def test_cholesky_mixed_ranks():
     w = wl.scaled(wl.WORKLOADS["gpt160m_block_r192"], "cholmix", [(520, 300), (300, 200), (400, 700), (200, 64)],
                   rank=300, steps=2)
     run_per_step(w, PRECS["bf16"], dict(gate_mode=oc.GATE_ALWAYS), w.steps, TOL_BF16)
+
+
+@pytest.mark.parametrize("prec,tol,rank", [("bf16x3", TOL_FP32, 24), ("bf16x3", TOL_FP32, 130), ("bf16", TOL_BF16, 260)])
+def test_gram_row_ranges(rank, prec, tol):
+    """Grams split into row ranges (a small plan splits every long layer): ranges of unequal length, a
+    last partial 32-row chunk, more than 8 ranges' worth of rows, and ranks with two output tiles."""
+    w = wl.scaled(wl.WORKLOADS["gpt160m_block_r192"], "ranges", [(289, 300), (300, 290), (545, 270), (3001, 265)],
+                  rank=rank, steps=2)
+    run_per_step(w, PRECS[prec], dict(gate_mode=oc.GATE_ALWAYS), w.steps, tol)
