@@ -254,6 +254,7 @@ __device__ int chol_inverse_tc(const float *S, float *__restrict__ W, int r, int
 }
 
 __global__ void __launch_bounds__(kThreads, 1) chol_inv_tc_kernel(Shared sh, const LayerMaps *__restrict__ maps) {
+  chain_enter();
   const int l = blockIdx.x;
   if (!sh.active[l]) return;
   const DevLayer &Ly = sh.layers[l];
@@ -347,7 +348,7 @@ cudaError_t prepare_chol_inv_tc(int32_t max_r, size_t *smem_out) {
 }
 
 void launch_chol_inv_tc(const Shared &sh, const tc::LayerMaps *maps, size_t smem, cudaStream_t s) {
-  if (sh.num_layers > 0) chol_inv_tc_kernel<<<sh.num_layers, kThreads, smem, s>>>(sh, maps);
+  if (sh.num_layers > 0) launch_chained(chol_inv_tc_kernel, sh.num_layers, kThreads, smem, s, sh, maps);
 }
 
 }  // namespace cd

@@ -233,6 +233,7 @@ __device__ int sweep(const float *S, const float *S2, float *__restrict__ W, int
 }
 
 __global__ void __launch_bounds__(kThreads, 1) chol_inv_tmem_kernel(Shared sh) {
+  chain_enter();
   const int l = blockIdx.x;
   if (!sh.active[l]) return;
   const DevLayer &Ly = sh.layers[l];
@@ -329,7 +330,7 @@ cudaError_t prepare_chol_inv_tmem(size_t *smem_out) {
 }
 
 void launch_chol_inv_tmem(const Shared &sh, size_t smem, cudaStream_t s) {
-  if (sh.num_layers > 0) chol_inv_tmem_kernel<<<sh.num_layers, kThreads, smem, s>>>(sh);
+  if (sh.num_layers > 0) launch_chained(chol_inv_tmem_kernel, sh.num_layers, kThreads, smem, s, sh);
 }
 
 }  // namespace cd

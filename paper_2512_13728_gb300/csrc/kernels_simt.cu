@@ -121,6 +121,7 @@ __device__ void form_b_tile(const DevLayer &L, int64_t row0, int64_t nrows, floa
 // layer), after which everything touches only the layers that sync and reads B from M.
 template <bool HALVES>
 __global__ void __launch_bounds__(kRowThreads, HALVES ? 5 : 8) form_b_kernel(Shared sh, const int4 *tiles) {
+  chain_enter();
   __shared__ double red[2 * (kRowThreads / 32)];
   const int4 t = tiles[blockIdx.x];
   DION_TILE_CHECK(t.x >= 0 && t.x < sh.num_layers, sh.status);
@@ -156,8 +157,8 @@ __global__ void __launch_bounds__(kRowThreads, HALVES ? 5 : 8) form_b_kernel(Sha
 
 void launch_form_b(const Shared &sh, const int4 *tiles, int32_t ntiles, cudaStream_t s, bool halves) {
   if (ntiles <= 0) return;
-  if (halves) form_b_kernel<true><<<ntiles, kRowThreads, 0, s>>>(sh, tiles);
-  else form_b_kernel<false><<<ntiles, kRowThreads, 0, s>>>(sh, tiles);
+  if (halves) launch_chained(form_b_kernel<true>, ntiles, kRowThreads, 0, s, sh, tiles);
+  else launch_chained(form_b_kernel<false>, ntiles, kRowThreads, 0, s, sh, tiles);
 }
 
 // BF16X3, after the gate: the two bf16 halves of B (already in M) for the Dion-branch layers,
@@ -165,6 +166,7 @@ void launch_form_b(const Shared &sh, const int4 *tiles, int32_t ntiles, cudaStre
 // row tile {layer, first row, rows, slot}.  `needed` false: the buffer pass already wrote them
 // (DION_GATE_ALWAYS), and every block returns at once.
 __global__ void __launch_bounds__(kRowThreads) split_b_kernel(Shared sh, const int4 *tiles, int needed) {
+  chain_enter();
   if (!needed) return;
   const int4 t = tiles[blockIdx.x];
   DION_TILE_CHECK(t.x >= 0 && t.x < sh.num_layers, sh.status);
@@ -203,7 +205,7 @@ __global__ void __launch_bounds__(kRowThreads) split_b_kernel(Shared sh, const i
 }
 
 void launch_split_b(const Shared &sh, const int4 *tiles, int32_t ntiles, bool needed, cudaStream_t s) {
-  if (ntiles > 0) split_b_kernel<<<ntiles, kRowThreads, 0, s>>>(sh, tiles, needed ? 1 : 0);
+  if (ntiles > 0) launch_chained(split_b_kernel, ntiles, kRowThreads, 0, s, sh, tiles, needed ? 1 : 0);
 }
 
 // =============================================================================== gate ===
@@ -287,6 +289,7 @@ __device__ void gate_finish(const Shared &sh, const StepArgs &a, int gflag, int 
 // layer and resets the scratch.
 constexpr int kGateWarps = 8;
 __global__ void __launch_bounds__(kGateWarps * 32) gate_kernel(Shared sh, StepArgs a) {
+  chain_enter();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int L = sh.num_layers;
   const int l = blockIdx.x * kGateWarps + warp;
@@ -316,7 +319,7 @@ __global__ void __launch_bounds__(kGateWarps * 32) gate_kernel(Shared sh, StepAr
 }
 
 void launch_gate(const Shared &sh, const StepArgs &a, cudaStream_t s) {
-  gate_kernel<<<std::max(1, (sh.num_layers + kGateWarps - 1) / kGateWarps), kGateWarps * 32, 0, s>>>(sh, a);
+  launch_chained(gate_kernel, std::max(1, (sh.num_layers + kGateWarps - 1) / kGateWarps), kGateWarps * 32, 0, s, sh, a);
 }
 
 // Data-parallel steps: Algorithm 2's branch from RMMC values the caller has already reduced
@@ -325,6 +328,7 @@ void launch_gate(const Shared &sh, const StepArgs &a, cudaStream_t s) {
 // branch mask of the gate mode.
 constexpr int kGateRedThreads = 256;
 __global__ void __launch_bounds__(kGateRedThreads) gate_reduced_kernel(Shared sh, StepArgs a) {
+  chain_enter();
   __shared__ double max_s[kGateRedThreads / 32];
   __shared__ int gflag_s, count_s;
   const int L = sh.num_layers, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -350,7 +354,7 @@ __global__ void __launch_bounds__(kGateRedThreads) gate_reduced_kernel(Shared sh
 }
 
 void launch_gate_reduced(const Shared &sh, const StepArgs &a, cudaStream_t s) {
-  gate_reduced_kernel<<<1, kGateRedThreads, 0, s>>>(sh, a);
+  launch_chained(gate_reduced_kernel, 1, kGateRedThreads, 0, s, sh, a);
 }
 
 // ==================================================================== grouped GEMM ===
@@ -377,6 +381,7 @@ __device__ __forceinline__ float4 ld4_rows(const float *base, int64_t row, int64
 
 __global__ void __launch_bounds__(kGemmThreads) gemm_kernel(Shared sh, const GemmProblem *probs,
                                                             const int4 *tiles) {
+  chain_enter();
   const int4 t = tiles[blockIdx.x];
   const GemmProblem p = probs[t.x];
   if (p.mode == GEMM_SHIFTED && sh.gate_scratch[kScratchShifted] == 0ull) return;  // no layer shifted
@@ -468,7 +473,7 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_kernel(Shared sh, const Gem
 
 void launch_gemm(const Shared &sh, const GemmProblem *probs, const int4 *tiles, int32_t ntiles,
                  cudaStream_t s) {
-  if (ntiles > 0) gemm_kernel<<<ntiles, kGemmThreads, 0, s>>>(sh, probs, tiles);
+  if (ntiles > 0) launch_chained(gemm_kernel, ntiles, kGemmThreads, 0, s, sh, probs, tiles);
 }
 
 // =========================================================== Cholesky + L^{-1} ===
@@ -716,6 +721,7 @@ __device__ __noinline__ float power_norm_sym(const float *S, int r, int64_t ls, 
 // resulting X L^{-T} is then orthonormal up to O(||E||_2^2).  The bound is ||E||_F when that
 // is small enough, else a power-iteration estimate of ||E||_2.
 __global__ void __launch_bounds__(kCholThreads, 1) chol_inv_kernel(Shared sh, int pass, float near_identity) {
+  chain_enter();
   const int l = blockIdx.x;
   if (pass == 2 && sh.gate_scratch[kScratchShifted] == 0ull) return;  // no layer took the shifted retry
   if (!sh.active[l]) return;
@@ -863,7 +869,7 @@ cudaError_t prepare_chol_inv(int32_t max_r, size_t *smem_out) {
 }
 
 void launch_chol_inv(const Shared &sh, size_t smem, int32_t pass, float near_identity, cudaStream_t s) {
-  if (sh.num_layers > 0) chol_inv_kernel<<<sh.num_layers, kCholThreads, smem, s>>>(sh, pass, near_identity);
+  if (sh.num_layers > 0) launch_chained(chol_inv_kernel, sh.num_layers, kCholThreads, smem, s, sh, pass, near_identity);
 }
 
 // ===================================================================== ColumnNormalize ===
@@ -874,6 +880,7 @@ void launch_chol_inv(const Shared &sh, size_t smem, int32_t pass, float near_ide
 constexpr int kColThreads = 256, kColRowGroups = kColThreads / 8, kColUnroll = 4;
 
 __global__ void __launch_bounds__(kColThreads) colnorm_kernel(Shared sh, const int4 *tiles, float eps_col) {
+  chain_enter();
   const int4 t = tiles[blockIdx.x];
   DION_TILE_CHECK(t.x >= 0 && t.x < sh.num_layers && t.y >= 0 && (int64_t)t.y * 32 < sh.layers[t.x].r, sh.status);
   if (!sh.active[t.x]) return;
@@ -950,7 +957,7 @@ __global__ void __launch_bounds__(kColThreads) colnorm_kernel(Shared sh, const i
 }
 
 void launch_colnorm(const Shared &sh, const int4 *tiles, int32_t ntiles, float eps_col, cudaStream_t s) {
-  if (ntiles > 0) colnorm_kernel<<<ntiles, kColThreads, 0, s>>>(sh, tiles, eps_col);
+  if (ntiles > 0) launch_chained(colnorm_kernel, ntiles, kColThreads, 0, s, sh, tiles, eps_col);
 }
 
 // =============================================================== error feedback + update ===
@@ -964,6 +971,7 @@ constexpr int UBM = kUpdTileM, UBN = kUpdTileN, UBK = 8, kUpdThreads = 256;
 
 __global__ void __launch_bounds__(kUpdThreads, 2) update_kernel(Shared sh, const int4 *tiles, float mu, float eta,
                                                              float keep) {
+  chain_enter();
   // P, R: ld ldp; Q: ld ldq; k slices stored transposed (K-th row = one k of every tile row)
   __shared__ __align__(16) float As[2][UBK][UBM + 4];
   __shared__ __align__(16) float Rs[2][UBK][UBN + 4];
@@ -1055,7 +1063,7 @@ __global__ void __launch_bounds__(kUpdThreads, 2) update_kernel(Shared sh, const
 
 void launch_update(const Shared &sh, const int4 *tiles, int32_t ntiles, float mu, float eta, float keep,
                    cudaStream_t s) {
-  if (ntiles > 0) update_kernel<<<ntiles, kUpdThreads, 0, s>>>(sh, tiles, mu, eta, keep);
+  if (ntiles > 0) launch_chained(update_kernel, ntiles, kUpdThreads, 0, s, sh, tiles, mu, eta, keep);
 }
 
 // ======================================================================== local branch ===
@@ -1095,6 +1103,7 @@ __device__ void local_tile(const DevLayer &L, int64_t row0, int64_t nrows, float
 }
 
 __global__ void __launch_bounds__(kRowThreads) local_kernel(Shared sh, const int4 *tiles, float eta_local, float keep) {
+  chain_enter();
   const int4 t = tiles[blockIdx.x];
   DION_TILE_CHECK(t.x >= 0 && t.x < sh.num_layers && t.y >= 0 && t.z >= 1 &&
                       (int64_t)t.y + t.z <= sh.layers[t.x].m, sh.status);
@@ -1105,7 +1114,7 @@ __global__ void __launch_bounds__(kRowThreads) local_kernel(Shared sh, const int
 }
 
 void launch_local(const Shared &sh, const int4 *tiles, int32_t ntiles, float eta_local, float keep, cudaStream_t s) {
-  if (ntiles > 0) local_kernel<<<ntiles, kRowThreads, 0, s>>>(sh, tiles, eta_local, keep);
+  if (ntiles > 0) launch_chained(local_kernel, ntiles, kRowThreads, 0, s, sh, tiles, eta_local, keep);
 }
 
 // ============================================================================ finalize ===
@@ -1113,6 +1122,7 @@ void launch_local(const Shared &sh, const int4 *tiles, int32_t ntiles, float eta
 // kernel's partials on synchronized layers and equals ||B_t|| on local layers (M = B).
 // One warp per layer: Equation 1 from the update's tile partials of ||M_t||^2.
 __global__ void __launch_bounds__(kGateWarps * 32) finalize_kernel(Shared sh, StepArgs a) {
+  chain_enter();
   if (a.eq1 == nullptr) return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int l = blockIdx.x * kGateWarps + warp; l < sh.num_layers; l += gridDim.x * kGateWarps) {
@@ -1136,7 +1146,7 @@ __global__ void __launch_bounds__(kGateWarps * 32) finalize_kernel(Shared sh, St
 
 void launch_finalize(const Shared &sh, const StepArgs &a, cudaStream_t s) {
   if (a.eq1 != nullptr)
-    finalize_kernel<<<std::max(1, (sh.num_layers + kGateWarps - 1) / kGateWarps), kGateWarps * 32, 0, s>>>(sh, a);
+    launch_chained(finalize_kernel, std::max(1, (sh.num_layers + kGateWarps - 1) / kGateWarps), kGateWarps * 32, 0, s, sh, a);
 }
 
 }  // namespace cd

@@ -194,6 +194,7 @@ template <int KIND, bool X3>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(R_THREADS, 1)
     tc_tma_gemm_kernel(Shared sh, const int4 *__restrict__ tiles, const int *__restrict__ off,
                        const LayerMaps *__restrict__ maps, int nstages, uint32_t stage_bytes, uint32_t tmem_cols) {
+  chain_enter();
   if (sh.gate_scratch[kScratchActive] == 0ull) return;  // no layer takes the Dion branch
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = align1024(smem_raw);
@@ -393,6 +394,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(FB_THREADS, 1)
     tc_form_bq_kernel(Shared sh, const int4 *__restrict__ tiles, const int *__restrict__ off,
                       const LayerMaps *__restrict__ maps, uint32_t qstage_bytes, uint32_t qring_bytes,
                       uint32_t tmem_cols, int gated) {
+  chain_enter();
   // gated: the norms pass and the gate ran first; only Dion-branch layers are processed and the
   // norm partials are not written again
   if (gated && sh.gate_scratch[kScratchActive] == 0ull) return;
@@ -748,7 +750,7 @@ cudaError_t setup_fused_bq_kernel(uint32_t smem) {
 
 void launch_fused_bq(const Shared &sh, const TcPlan &tp, bool gated, cudaStream_t s) {
   if (tp.d_bq.grid <= 0) return;
-  tc_form_bq_kernel<<<2 * tp.d_bq.grid, FB_THREADS, tp.fb_smem, s>>>(
+  launch_chained(tc_form_bq_kernel, 2 * tp.d_bq.grid, FB_THREADS, tp.fb_smem, s, 
       sh, tp.d_bq.tiles, tp.d_bq.off, tp.maps, tp.bq_boxes * BOX64, fused_bq_qring(tp.bq_boxes), tp.tmem_cols,
       gated ? 1 : 0);
 }
@@ -758,10 +760,10 @@ void launch_form_bq(const Shared &sh, const TcPlan &tp, cudaStream_t s) {
   const bool x3 = tp.precision == DION_PREC_BF16X3;
   const uint32_t stage = (x3 ? 2u : 1u) * (OPB_A + tp.bq_boxes * BOX64);
   if (x3)
-    tc_tma_gemm_kernel<GEMM_BQ, true><<<2 * tp.d_bq.grid, R_THREADS, tp.f_smem, s>>>(
+    launch_chained(tc_tma_gemm_kernel<GEMM_BQ, true>, 2 * tp.d_bq.grid, R_THREADS, tp.f_smem, s, 
         sh, tp.d_bq.tiles, tp.d_bq.off, tp.maps, tp.f_stages, stage, tp.tmem_cols);
   else
-    tc_tma_gemm_kernel<GEMM_BQ, false><<<2 * tp.d_bq.grid, R_THREADS, tp.f_smem, s>>>(
+    launch_chained(tc_tma_gemm_kernel<GEMM_BQ, false>, 2 * tp.d_bq.grid, R_THREADS, tp.f_smem, s, 
         sh, tp.d_bq.tiles, tp.d_bq.off, tp.maps, tp.f_stages, stage, tp.tmem_cols);
 }
 
@@ -770,16 +772,17 @@ void launch_btp(const Shared &sh, const TcPlan &tp, cudaStream_t s) {
   const bool x3 = tp.precision == DION_PREC_BF16X3;
   const uint32_t stage = (x3 ? 2u : 1u) * (OPB_A + tp.bq_boxes * BOX64);
   if (x3)
-    tc_tma_gemm_kernel<GEMM_BTP, true><<<2 * tp.d_btp.grid, R_THREADS, tp.r_smem, s>>>(
+    launch_chained(tc_tma_gemm_kernel<GEMM_BTP, true>, 2 * tp.d_btp.grid, R_THREADS, tp.r_smem, s, 
         sh, tp.d_btp.tiles, tp.d_btp.off, tp.maps, tp.r_stages, stage, tp.tmem_cols);
   else
-    tc_tma_gemm_kernel<GEMM_BTP, false><<<2 * tp.d_btp.grid, R_THREADS, tp.r_smem, s>>>(
+    launch_chained(tc_tma_gemm_kernel<GEMM_BTP, false>, 2 * tp.d_btp.grid, R_THREADS, tp.r_smem, s, 
         sh, tp.d_btp.tiles, tp.d_btp.off, tp.maps, tp.r_stages, stage, tp.tmem_cols);
 }
 
 // Data-parallel phases.  P_raw^T (r x m, the first Gram's operand) from the averaged P_raw:
 // tile = {layer, 128-row block of P_raw}, 32 x 32 sub-tiles through shared memory.
 __global__ void __launch_bounds__(256) transpose_praw_kernel(Shared sh, const int4 *tiles) {
+  chain_enter();
   const int4 t = tiles[blockIdx.x];
   DION_TILE_CHECK(t.x >= 0 && t.x < sh.num_layers && t.y >= 0 && (int64_t)t.y * 128 < sh.layers[t.x].m, sh.status);
   if (!sh.active[t.x]) return;
@@ -807,6 +810,7 @@ __global__ void __launch_bounds__(256) transpose_praw_kernel(Shared sh, const in
 // ColumnNormalize reads, from the averaged R: tile = {layer, 128-row block of R}; thread j
 // takes columns j and j + 256, rows in order (fp32 over 32 rows, then fp64).
 __global__ void __launch_bounds__(256) r_refresh_kernel(Shared sh, const int4 *tiles) {
+  chain_enter();
   const int4 t = tiles[blockIdx.x];
   DION_TILE_CHECK(t.x >= 0 && t.x < sh.num_layers && t.y >= 0 && (int64_t)t.y * 128 < sh.layers[t.x].n, sh.status);
   if (!sh.active[t.x]) return;
@@ -828,10 +832,10 @@ __global__ void __launch_bounds__(256) r_refresh_kernel(Shared sh, const int4 *t
 }
 
 void launch_transpose_praw(const Shared &sh, const TcPlan &tp, cudaStream_t s) {
-  if (tp.n_trsm_tiles > 0) transpose_praw_kernel<<<tp.n_trsm_tiles, 256, 0, s>>>(sh, tp.trsm_tiles);
+  if (tp.n_trsm_tiles > 0) launch_chained(transpose_praw_kernel, tp.n_trsm_tiles, 256, 0, s, sh, tp.trsm_tiles);
 }
 void launch_r_refresh(const Shared &sh, const TcPlan &tp, cudaStream_t s) {
-  if (tp.n_rtiles > 0) r_refresh_kernel<<<tp.n_rtiles, 256, 0, s>>>(sh, tp.rtiles);
+  if (tp.n_rtiles > 0) launch_chained(r_refresh_kernel, tp.n_rtiles, 256, 0, s, sh, tp.rtiles);
 }
 
 void launch_qn_refresh(const Shared &sh, const TcPlan &tp, cudaStream_t s) {
@@ -841,6 +845,7 @@ void launch_qn_refresh(const Shared &sh, const TcPlan &tp, cudaStream_t s) {
 // ColumnNormalize from the per-tile column sums of squares: colinv[j] = 1 / (||R_j|| + eps),
 // fixed-order fp64 sum over the R tiles of the layer.  Grid: one block per (layer, 32 columns).
 __global__ void __launch_bounds__(256) colnorm_reduce_kernel(Shared sh, const int4 *ctiles, float eps_col) {
+  chain_enter();
   const int4 t = ctiles[blockIdx.x];  // {layer, 32-column group, 0, 0}
   DION_TILE_CHECK(t.x >= 0 && t.x < sh.num_layers && t.y >= 0 && (int64_t)t.y * 32 < sh.layers[t.x].r, sh.status);
   if (!sh.active[t.x]) return;
@@ -869,6 +874,7 @@ __global__ void __launch_bounds__(256) colnorm_reduce_kernel(Shared sh, const in
 // written only inside its r columns; rows of R and of the bf16 copies are padded to 8.
 constexpr int kScaleThreads = 256;
 __global__ void __launch_bounds__(kScaleThreads, 8) colnorm_scale_kernel(Shared sh, const int4 *tiles) {
+  chain_enter();
   const int4 t = tiles[blockIdx.x];  // {layer, first row, rows, 0}
   DION_TILE_CHECK(t.x >= 0 && t.x < sh.num_layers && t.y >= 0 && t.z >= 1 &&
                       (int64_t)t.y + t.z <= sh.layers[t.x].n, sh.status);
@@ -916,10 +922,10 @@ __global__ void __launch_bounds__(kScaleThreads, 8) colnorm_scale_kernel(Shared 
 }
 
 void launch_colnorm_reduce(const Shared &sh, const int4 *ctiles, int32_t n_ctiles, float eps_col, cudaStream_t s) {
-  if (n_ctiles > 0) colnorm_reduce_kernel<<<n_ctiles, 256, 0, s>>>(sh, ctiles, eps_col);
+  if (n_ctiles > 0) launch_chained(colnorm_reduce_kernel, n_ctiles, 256, 0, s, sh, ctiles, eps_col);
 }
 void launch_colnorm_scale(const Shared &sh, const TcPlan &tp, cudaStream_t s) {
-  if (tp.n_qtiles > 0) colnorm_scale_kernel<<<tp.n_qtiles, kScaleThreads, 0, s>>>(sh, tp.qtiles);
+  if (tp.n_qtiles > 0) launch_chained(colnorm_scale_kernel, tp.n_qtiles, kScaleThreads, 0, s, sh, tp.qtiles);
 }
 
 }  // namespace tc

@@ -140,6 +140,7 @@ template <int KIND, bool X3>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(X3 ? O_THREADS_X3 : O_THREADS, 1)
     tc_orth_kernel(Shared sh, const int4 *__restrict__ tiles, const int *__restrict__ off, const LayerMaps *__restrict__ maps,
                    int pass, int nstages, uint32_t stage_bytes, uint32_t tmem_cols, uint32_t slots) {
+  chain_enter();
   if (sh.gate_scratch[kScratchActive] == 0ull) return;  // no layer takes the Dion branch
   if (pass == 2 && sh.gate_scratch[kScratchShifted] == 0ull) return;  // no layer took the shifted retry
   extern __shared__ uint8_t smem_raw[];
@@ -550,16 +551,16 @@ void launch_orth(const Shared &sh, const TcPlan &tp, bool gram, int pass, cudaSt
   // two accumulator slots for the Gram where its tiles need at most 256 columns
   const uint32_t slots = tp.max_r <= 256 ? 2u : 1u, gcols = slots == 2u ? 512u : tp.tmem_cols;
   if (gram && x3)
-    tc_orth_kernel<ORTH_GRAM, true><<<g, O_THREADS_X3, tp.o_smem, s>>>(sh, d.tiles, d.off, tp.maps, pass,
+    launch_chained(tc_orth_kernel<ORTH_GRAM, true>, g, O_THREADS_X3, tp.o_smem, s, sh, d.tiles, d.off, tp.maps, pass,
                                                                         tp.o_stages, stage, gcols, slots);
   else if (gram)
-    tc_orth_kernel<ORTH_GRAM, false><<<g, O_THREADS, tp.o_smem, s>>>(sh, d.tiles, d.off, tp.maps, pass,
+    launch_chained(tc_orth_kernel<ORTH_GRAM, false>, g, O_THREADS, tp.o_smem, s, sh, d.tiles, d.off, tp.maps, pass,
                                                                       tp.o_stages, stage, gcols, slots);
   else if (x3)  // two 256-column accumulator slots
-    tc_orth_kernel<ORTH_TRSM, true><<<g, O_THREADS_X3, tp.o_smem, s>>>(sh, d.tiles, d.off, tp.maps, pass,
+    launch_chained(tc_orth_kernel<ORTH_TRSM, true>, g, O_THREADS_X3, tp.o_smem, s, sh, d.tiles, d.off, tp.maps, pass,
                                                                         tp.t_stages, tstage, 512u, 2u);
   else
-    tc_orth_kernel<ORTH_TRSM, false><<<g, O_THREADS, tp.o_smem, s>>>(sh, d.tiles, d.off, tp.maps, pass,
+    launch_chained(tc_orth_kernel<ORTH_TRSM, false>, g, O_THREADS, tp.o_smem, s, sh, d.tiles, d.off, tp.maps, pass,
                                                                       tp.t_stages, tstage, 512u, 2u);
 }
 

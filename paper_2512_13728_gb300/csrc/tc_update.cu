@@ -65,6 +65,7 @@ template <bool X3, bool GIN, bool DEEP>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(U_THREADS, 1)
     tc_update_kernel(Shared sh, const int4 *__restrict__ tiles, const int *__restrict__ off, const LayerMaps *__restrict__ maps,
                      float mu, float eta, float keep) {
+  chain_enter();
   using Cfg = UpdCfg<X3, GIN, DEEP>;
   constexpr int U_STAGES = Cfg::STAGES, U_EBUF = Cfg::EBUF;
   constexpr uint32_t U_STAGE = Cfg::STAGE, U_EBUFB = Cfg::EBUFB;
@@ -362,7 +363,7 @@ cudaError_t setup_update_kernel(bool x3) {
 
 template <bool X3, bool GIN, bool DEEP>
 static void launch_as(const Shared &sh, const TcPlan &tp, float mu, float eta, float keep, cudaStream_t s) {
-  tc_update_kernel<X3, GIN, DEEP><<<2 * tp.d_update.grid, U_THREADS, UpdCfg<X3, GIN, DEEP>::SMEM, s>>>(
+  launch_chained(tc_update_kernel<X3, GIN, DEEP>, 2 * tp.d_update.grid, U_THREADS, UpdCfg<X3, GIN, DEEP>::SMEM, s, 
       sh, tp.d_update.tiles, tp.d_update.off, tp.maps, mu, eta, keep);
 }
 
