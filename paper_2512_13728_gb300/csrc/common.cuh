@@ -143,14 +143,15 @@ struct Shared {
 // A contraction C = op(A) op(B) for the CUDA-core path.
 // op(A)[i][k] = transA ? A[k*lda + i] : A[i*lda + k]   (i < Mrows, k < K)
 // op(B)[k][j] = transB ? B[j*ldb + k] : B[k*ldb + j]   (k < K, j < Ncols)
-// mode: GEMM_ACTIVE runs on active layers; GEMM_SHIFTED only where orth_shifted is set;
-// GEMM_SHIFTED_OR_COPY multiplies where orth_shifted is set and copies A to C elsewhere.
-enum : int32_t { GEMM_ACTIVE = 0, GEMM_SHIFTED = 1, GEMM_SHIFTED_OR_COPY = 2 };
+// mode: GEMM_ACTIVE runs on active layers; GEMM_SHIFTED only where orth_shifted is set.
+// B_unshifted, when not null, takes B's place where orth_shifted is not set: Orthogonalize leaves
+// its result in P after a third pass and in P_raw otherwise.
+enum : int32_t { GEMM_ACTIVE = 0, GEMM_SHIFTED = 1 };
 constexpr int kGemmTile = 128;  // output tile edge of the CUDA-core grouped GEMM
 constexpr int kUpdTileM = 128, kUpdTileN = 64;  // output tile of the CUDA-core update (FP32 mode)
 struct GemmProblem {
   const float *A;
-  const float *B;
+  const float *B, *B_unshifted;
   float *C;
   int64_t Mrows, Ncols, K, lda, ldb, ldc;
   int32_t transA, transB, layer, mode;

@@ -390,15 +390,8 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_kernel(Shared sh, const Gem
   if (!sh.active[p.layer]) return;
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   const int64_t i0 = (int64_t)t.y * GBM, j0 = (int64_t)t.z * GBN;
-  if (p.mode != GEMM_ACTIVE && !sh.orth_shifted[p.layer]) {
-    if (p.mode == GEMM_SHIFTED_OR_COPY) {  // C = A (same shape, A not transposed)
-      for (int e = tid; e < GBM * GBN; e += kGemmThreads) {
-        const int64_t gi = i0 + e / GBN, gj = j0 + e % GBN;
-        if (gi < p.Mrows && gj < p.Ncols) p.C[gi * p.ldc + gj] = p.A[gi * p.lda + gj];
-      }
-    }
-    return;
-  }
+  if (p.mode == GEMM_SHIFTED && !sh.orth_shifted[p.layer]) return;
+  const float *B = (p.B_unshifted != nullptr && !sh.orth_shifted[p.layer]) ? p.B_unshifted : p.B;
   __shared__ __align__(16) float As[2][GBK][GBM + 4];
   __shared__ __align__(16) float Bs[2][GBK][GBN + 4];
   // this thread's 16-byte share of a k slice of A (128 x 8) and of B (8 x 128): along the
@@ -408,8 +401,8 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_kernel(Shared sh, const Gem
   auto load = [&](int64_t k0, float4 &av, float4 &bv) {
     av = p.transA ? ld4_rows(p.A, k0 + a_r, i0 + a_c, p.K, p.Mrows, p.lda)   // A^T stored K x M
                   : ld4_rows(p.A, i0 + a_r, k0 + a_c, p.Mrows, p.K, p.lda);  // A stored M x K
-    bv = p.transB ? ld4_rows(p.B, j0 + b_r, k0 + b_c, p.Ncols, p.K, p.ldb)   // B^T stored N x K
-                  : ld4_rows(p.B, k0 + b_r, j0 + b_c, p.K, p.Ncols, p.ldb);  // B stored K x N
+    bv = p.transB ? ld4_rows(B, j0 + b_r, k0 + b_c, p.Ncols, p.K, p.ldb)   // B^T stored N x K
+                  : ld4_rows(B, k0 + b_r, j0 + b_c, p.K, p.Ncols, p.ldb);  // B stored K x N
   };
   auto store = [&](int buf, const float4 &av, const float4 &bv) {
     if (p.transA) {
@@ -982,6 +975,7 @@ __global__ void __launch_bounds__(kUpdThreads, 2) update_kernel(Shared sh, const
                       (int64_t)t.y * UBM < sh.layers[t.x].m && (int64_t)t.z * UBN < sh.layers[t.x].n, sh.status);
   if (!sh.active[t.x]) return;
   const DevLayer &L = sh.layers[t.x];
+  const float *P = sh.orth_shifted[t.x] ? L.P : L.P_raw;  // the last pass's result
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   const int64_t i0 = (int64_t)t.y * UBM, j0 = (int64_t)t.z * UBN, r = L.r, ldp = L.ldp;
   // this thread's share of a k slice: 4 consecutive k of one row of P, and of one row of R
@@ -989,7 +983,7 @@ __global__ void __launch_bounds__(kUpdThreads, 2) update_kernel(Shared sh, const
   const int pr = tid >> 1, kq = (tid & 1) * 4, br = (tid & 127) >> 1;
   const bool is_q = tid >= 128;
   auto load = [&](int64_t k0, float4 &pv, float4 &bv) {
-    pv = ld4_rows(L.P, i0 + pr, k0 + kq, L.m, r, ldp);
+    pv = ld4_rows(P, i0 + pr, k0 + kq, L.m, r, ldp);
     bv = is_q ? ld4_rows(L.Q, j0 + br, k0 + kq, L.n, r, L.ldq) : ld4_rows(L.R, j0 + br, k0 + kq, L.n, r, ldp);
   };
   auto store = [&](int buf, const float4 &pv, const float4 &bv) {

@@ -304,9 +304,7 @@ dion_status dion_plan_create(const dion_layer *layers, int32_t num_layers, int32
         q.mode = (k == 3) ? GEMM_SHIFTED : GEMM_ACTIVE;
       } else if (k <= 6) {
         q.Mrows = ly.m; q.Ncols = ly.r; q.K = ly.r; q.lda = ldp; q.ldb = ldp; q.ldc = ldp; q.transB = 1;
-        // the third solve runs on shifted layers only; it also copies the second pass's result
-        // into P for the others
-        q.mode = (k == 6) ? GEMM_SHIFTED_OR_COPY : GEMM_ACTIVE;
+        q.mode = (k == 6) ? GEMM_SHIFTED : GEMM_ACTIVE;  // the third solve: shifted layers only
       } else {
         q.Mrows = ly.n; q.Ncols = ly.r; q.K = ly.m; q.lda = ly.ldm; q.ldb = ldp; q.ldc = ldp; q.transA = 1;
       }
@@ -344,7 +342,7 @@ dion_status dion_plan_create(const dion_layer *layers, int32_t num_layers, int32
       if (k == 0) { q.A = d.M; q.B = d.Q; q.C = d.P_raw; }
       else if (k <= 3) { q.A = Xs[k - 1]; q.B = Xs[k - 1]; q.C = d.S; }
       else if (k <= 6) { q.A = Xs[k - 4]; q.B = d.Linv; q.C = Xs[k - 3]; }
-      else { q.A = d.M; q.B = d.P; q.C = d.R; }
+      else { q.A = d.M; q.B = d.P; q.B_unshifted = d.P_raw; q.C = d.R; }
     }
     p->probs[k] = reinterpret_cast<GemmProblem *>(base + o_gp[k]);
     p->gtiles[k] = reinterpret_cast<int4 *>(base + o_gt[k]);
