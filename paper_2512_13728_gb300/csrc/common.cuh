@@ -147,7 +147,7 @@ struct Shared {
 // B_unshifted, when not null, takes B's place where orth_shifted is not set: Orthogonalize leaves
 // its result in P after a third pass and in P_raw otherwise.
 enum : int32_t { GEMM_ACTIVE = 0, GEMM_SHIFTED = 1 };
-constexpr int kGemmTile = 128;  // output tile edge of the CUDA-core grouped GEMM
+constexpr int kGemmTile = 128, kGemmSmallTile = 32;  // output tile edges of the CUDA-core grouped GEMMs
 constexpr int kUpdTileM = 128, kUpdTileN = 64;  // output tile of the CUDA-core update (FP32 mode)
 struct GemmProblem {
   const float *A;
@@ -211,7 +211,7 @@ void launch_split_b(const Shared &sh, const int4 *tiles, int32_t ntiles, bool ne
 void launch_gate(const Shared &sh, const StepArgs &a, cudaStream_t s);
 // the branch from RMMC values already in a.rmmc (reduced over data-parallel workers)
 void launch_gate_reduced(const Shared &sh, const StepArgs &a, cudaStream_t s);
-void launch_gemm(const Shared &sh, const GemmProblem *probs, const int4 *tiles, int32_t ntiles,
+void launch_gemm(const Shared &sh, const GemmProblem *probs, const int4 *tiles, int32_t ntiles, bool small,
                  cudaStream_t s);
 cudaError_t prepare_chol_inv(int32_t max_r, size_t *smem_out);
 // near_identity: Frobenius bound on S - I below which passes 1 and 2 use the first-order factor

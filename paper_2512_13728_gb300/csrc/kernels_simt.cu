@@ -464,9 +464,107 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_kernel(Shared sh, const Gem
   }
 }
 
-void launch_gemm(const Shared &sh, const GemmProblem *probs, const int4 *tiles, int32_t ntiles,
+// The same contractions in 32 x 32 output tiles, for plans with too few 128 x 128 tiles to fill the
+// chip: the 8 warps of a block split K in chunks of 16 (warp w takes chunks w, w + 8, ...), each
+// with its own shared-memory slice and the next chunk's loads in flight, and add their partial
+// tiles in warp order at the end.  Bound by the latency of a
+// warp's K / 128 chunks on small plans, by its shared-memory reads (3 for 32 multiply-adds) on large
+// ones; gemm_tiles (plan.cu) chooses and has both kernels' figures.
+constexpr int GST = kGemmSmallTile, GSK = 16;
+__global__ void __launch_bounds__(kGemmThreads) gemm_small_kernel(Shared sh, const GemmProblem *probs,
+                                                                  const int4 *tiles) {
+  chain_enter();
+  const int4 t = tiles[blockIdx.x];
+  const GemmProblem p = probs[t.x];
+  if (p.mode == GEMM_SHIFTED && sh.gate_scratch[kScratchShifted] == 0ull) return;  // no layer shifted
+  DION_TILE_CHECK(p.layer >= 0 && p.layer < sh.num_layers && t.y >= 0 && t.z >= 0 &&
+                      (int64_t)t.y * GST < p.Mrows && (int64_t)t.z * GST < p.Ncols, sh.status);
+  if (!sh.active[p.layer]) return;
+  if (p.mode == GEMM_SHIFTED && !sh.orth_shifted[p.layer]) return;
+  const float *B = (p.B_unshifted != nullptr && !sh.orth_shifted[p.layer]) ? p.B_unshifted : p.B;
+  __shared__ __align__(16) float smem[8][2][GSK][GST + 4];  // per warp: A and B slices, k-major
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t i0 = (int64_t)t.y * GST, j0 = (int64_t)t.z * GST;
+  float(*As)[GST + 4] = smem[warp][0], (*Bs)[GST + 4] = smem[warp][1];
+  // a chunk of an operand in four 16-byte loads per lane, along its contiguous dimension
+  const int kr = lane >> 3, cc = (lane & 7) * 4;  // stored k x row: k = kr + 4 u, rows cc ..
+  const int rr = lane >> 2, kc = (lane & 3) * 4;  // stored row x k: row = rr + 8 u, k = kc ..
+  float4 av[4], bv[4];
+  auto load = [&](int64_t k0) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      av[u] = p.transA ? ld4_rows(p.A, k0 + kr + 4 * u, i0 + cc, p.K, p.Mrows, p.lda)
+                       : ld4_rows(p.A, i0 + rr + 8 * u, k0 + kc, p.Mrows, p.K, p.lda);
+      bv[u] = p.transB ? ld4_rows(B, j0 + rr + 8 * u, k0 + kc, p.Ncols, p.K, p.ldb)
+                       : ld4_rows(B, k0 + kr + 4 * u, j0 + cc, p.K, p.Ncols, p.ldb);
+    }
+  };
+  auto put = [&](float(*s)[GST + 4], const float4 &v, bool by_k, int u) {
+    if (by_k) {
+      *reinterpret_cast<float4 *>(&s[kr + 4 * u][cc]) = v;
+    } else {
+      s[kc + 0][rr + 8 * u] = v.x; s[kc + 1][rr + 8 * u] = v.y;
+      s[kc + 2][rr + 8 * u] = v.z; s[kc + 3][rr + 8 * u] = v.w;
+    }
+  };
+  const int ry = (lane >> 2) * 4, cx = (lane & 3) * 8;  // this lane's 4 x 8 outputs
+  float acc[4][8] = {};
+  int64_t k0 = (int64_t)warp * GSK;
+  if (k0 < p.K) load(k0);
+  for (; k0 < p.K; k0 += 8 * GSK) {
+    __syncwarp();  // the previous chunk has been read
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      put(As, av[u], p.transA != 0, u);
+      put(Bs, bv[u], p.transB == 0, u);
+    }
+    __syncwarp();
+    if (k0 + 8 * GSK < p.K) load(k0 + 8 * GSK);  // in flight during this chunk's products
+#pragma unroll 4
+    for (int kk = 0; kk < GSK; ++kk) {
+      const float4 a4 = *reinterpret_cast<const float4 *>(&As[kk][ry]);
+      const float4 b0 = *reinterpret_cast<const float4 *>(&Bs[kk][cx]), b1 = *reinterpret_cast<const float4 *>(&Bs[kk][cx + 4]);
+      const float a[4] = {a4.x, a4.y, a4.z, a4.w}, b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+    }
+  }
+  // the warps' partial tiles (32 x 32 each, over the slices), added in warp order: four outputs a thread
+  __syncthreads();
+  float(*part)[GST * GST] = reinterpret_cast<float(*)[GST * GST]>(&smem[0][0][0][0]);
+  static_assert(sizeof(smem) >= 8 * GST * GST * sizeof(float), "the partial tiles fit the slices");
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    *reinterpret_cast<float4 *>(&part[warp][(ry + i) * GST + cx]) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+    *reinterpret_cast<float4 *>(&part[warp][(ry + i) * GST + cx + 4]) = make_float4(acc[i][4], acc[i][5], acc[i][6], acc[i][7]);
+  }
+  __syncthreads();
+  const int e = threadIdx.x * 4;
+  float o[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+  for (int w = 0; w < 8; ++w) {
+    const float4 x = *reinterpret_cast<const float4 *>(&part[w][e]);
+    o[0] += x.x; o[1] += x.y; o[2] += x.z; o[3] += x.w;
+  }
+  const int64_t gi = i0 + e / GST, gj = j0 + e % GST;
+  if (gi >= p.Mrows) return;
+  float *c = p.C + gi * p.ldc + gj;
+  if (gj + 4 <= p.Ncols) {
+    *reinterpret_cast<float4 *>(c) = make_float4(o[0], o[1], o[2], o[3]);
+  } else {
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (gj + q < p.Ncols) c[q] = o[q];
+  }
+}
+
+void launch_gemm(const Shared &sh, const GemmProblem *probs, const int4 *tiles, int32_t ntiles, bool small,
                  cudaStream_t s) {
-  if (ntiles > 0) launch_chained(gemm_kernel, ntiles, kGemmThreads, 0, s, sh, probs, tiles);
+  if (ntiles <= 0) return;
+  if (small) launch_chained(gemm_small_kernel, ntiles, kGemmThreads, 0, s, sh, probs, tiles);
+  else launch_chained(gemm_kernel, ntiles, kGemmThreads, 0, s, sh, probs, tiles);
 }
 
 // =========================================================== Cholesky + L^{-1} ===
@@ -478,7 +576,7 @@ void launch_gemm(const Shared &sh, const GemmProblem *probs, const int4 *tiles, 
 // upper-triangular matrix with positive diagonal, so the final P is the Q factor of the
 // thin QR of the original P with a positive-diagonal triangular factor.
 //
-// One CTA per layer (r <= 512), 16 warps.  S (full, symmetric) is only read; the factor and
+// One CTA per layer (r <= 512), 16 warps.  S (its lower triangle) is only read; the factor and
 // its inverse are built in place in the L^{-1} buffer W by one right-looking sweep over
 // 32-wide block columns k (k0 = 32 k).  Before step k, for rows i >= k0:
 //   W[i][j], j >= k0 : the Schur complement S - L[:, :k0] L[:, :k0]^T (lower triangle),

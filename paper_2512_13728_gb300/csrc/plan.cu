@@ -31,6 +31,7 @@ struct dion_plan {
   GemmProblem *probs[kSets] = {};
   int4 *gtiles[kSets] = {};
   int32_t n_gtiles[kSets] = {};
+  bool gemm_small[kSets] = {};  // the set's tiles are kGemmSmallTile wide
   size_t chol_smem = 0;
   tc::TcPlan tcp{};  // tensor-core path (BF16 / BF16X3)
   int32_t launches_per_step = 0;  // of the last step (before the first: of an ALWAYS step)
@@ -143,6 +144,40 @@ int64_t row_tile_elems(const dion_layer *layers, int32_t num_layers, int sms) {
   int64_t total = 0;
   for (int32_t l = 0; l < num_layers; ++l) total += layers[l].m * layers[l].n;
   return std::min<int64_t>(65536, std::max<int64_t>(1024, total / (4 * std::max(sms, 1))));
+}
+
+// The output tiles of a set of problems, those with the longest K first (the last wave then holds
+// short ones: 3.72 / 3.41 ms for B Q on the 350M stack).  lower: tiles above the diagonal are left
+// out (a Gram, whose lower triangle alone is read).  *small: 32 x 32 tiles (K split over a block's
+// warps) instead of 128 x 128, where an estimate from both kernels' measured rates says so.  Large
+// tiles: 22e6 multiply-adds per us in all, and 0.117 us per k of the longest tile alone on its SM,
+// 0.16 with a second one beside it; small ones: 15.5e6, and 5 us + 0.0125 us per k.  Measured, large /
+// small: 256 x 512 rank 16 B Q 68 / 14 us, Gram 37 / 10; one 1024-wide block at rank 256 B Q 491 /
+// 215, Gram 475 / 58, solve 39 / 57; four 768-wide blocks at rank 192 B Q 502 / 360; the 350M stack
+// B Q 3407 / 4852, Gram 665 / 496, solve 706 / 1196.
+std::vector<int4> gemm_tiles(const std::vector<GemmProblem> &probs, bool lower, int sms, bool *small) {
+  int64_t longest = 0;
+  for (const GemmProblem &q : probs) longest = std::max(longest, q.K);
+  auto tiles_of = [&](int64_t edge, double *macs) {
+    std::vector<int4> t;
+    *macs = 0.0;
+    for (size_t i = 0; i < probs.size(); ++i)
+      for (int64_t ti = 0; ti < (probs[i].Mrows + edge - 1) / edge; ++ti)
+        for (int64_t tj = 0; tj < (probs[i].Ncols + edge - 1) / edge; ++tj) {
+          if (lower && tj > ti) continue;
+          t.push_back(make_int4((int)i, (int)ti, (int)tj, 0));
+          *macs += (double)edge * edge * probs[i].K;
+        }
+    return t;
+  };
+  double macs_l, macs_s;
+  std::vector<int4> t = tiles_of(kGemmTile, &macs_l), ts = tiles_of(kGemmSmallTile, &macs_s);
+  const double us_l = std::max(macs_l / 22e6, ((int64_t)t.size() > sms ? 0.16 : 0.117) * (double)longest);
+  const double us_s = std::max(macs_s / 15.5e6, 5.0 + 0.0125 * (double)longest);
+  *small = us_s < us_l;
+  if (*small) t = std::move(ts);
+  std::stable_sort(t.begin(), t.end(), [&](const int4 &a, const int4 &b) { return probs[a.x].K > probs[b.x].K; });
+  return t;
 }
 
 template <class T>
@@ -292,7 +327,7 @@ dion_status dion_plan_create(const dion_layer *layers, int32_t num_layers, int32
   const size_t o_shift = cv.take<uint8_t>(std::max(num_layers, 1));
   size_t o_gp[kSets], o_gt[kSets];
   for (int k = 0; k < kSets; ++k) {
-    for (int32_t l = 0; l < num_layers; ++l) {
+    for (int32_t l = 0; l < num_layers && precision == DION_PREC_FP32; ++l) {
       const dion_layer &ly = layers[l];
       const int64_t ldp = dl[l].ldp;
       GemmProblem q{};
@@ -308,12 +343,9 @@ dion_status dion_plan_create(const dion_layer *layers, int32_t num_layers, int32
       } else {
         q.Mrows = ly.n; q.Ncols = ly.r; q.K = ly.m; q.lda = ly.ldm; q.ldb = ldp; q.ldc = ldp; q.transA = 1;
       }
-      const int32_t pi = (int32_t)gp[k].size();
       gp[k].push_back(q);
-      for (int64_t ti = 0; ti < (q.Mrows + kGemmTile - 1) / kGemmTile; ++ti)
-        for (int64_t tj = 0; tj < (q.Ncols + kGemmTile - 1) / kGemmTile; ++tj)
-          gt[k].push_back(make_int4(pi, (int)ti, (int)tj, 0));
     }
+    gt[k] = gemm_tiles(gp[k], k >= 1 && k <= 3, sms, &p->gemm_small[k]);
     o_gp[k] = cv.take<GemmProblem>(std::max<size_t>(gp[k].size(), 1));
     o_gt[k] = cv.take<int4>(std::max<size_t>(gt[k].size(), 1));
   }
@@ -386,9 +418,6 @@ dion_status dion_plan_create(const dion_layer *layers, int32_t num_layers, int32
     e = cudaMemset(p->sh.gate_scratch, 0, kScratchSlots * sizeof(unsigned long long));  // key 0 < every RMMC
   if (e == cudaSuccess && num_layers > 0) e = prepare_chol_inv(p->max_r, &p->chol_smem);
   if (e == cudaSuccess && precision != DION_PREC_FP32) {
-    p->tcp.probs = p->probs;
-    p->tcp.gtiles = p->gtiles;
-    p->tcp.n_gtiles = p->n_gtiles;
     e = tc::init(tcl, base, dl.data(), num_layers, &p->tcp);
     if (e == cudaSuccess) {  // the tensor-core path works from a bf16 copy of Q
       tc::refresh(p->tcp, p->sh, nullptr);
@@ -453,20 +482,20 @@ void enqueue_step(dion_plan *p, const Shared &sh, const tc::TcPlan &tcp, const d
     tick(p, s, "form_b");
     launch_gate(sh, a, s);
     tick(p, s, "gate");
-    launch_gemm(sh, p->probs[0], p->gtiles[0], p->n_gtiles[0], s);  // P = B Q
+    launch_gemm(sh, p->probs[0], p->gtiles[0], p->n_gtiles[0], p->gemm_small[0], s);  // P = B Q
     tick(p, s, "gemm_bq");
     static const char *kGram[3] = {"gemm_gram0", "gemm_gram1", "gemm_gram2"};
     static const char *kChol[3] = {"chol_inv0", "chol_inv1", "chol_inv2"};
     static const char *kTrsm[3] = {"gemm_trsm0", "gemm_trsm1", "gemm_trsm2"};
     for (int pass = 0; pass < 3; ++pass) {  // CholeskyQR2, third pass only after a shifted retry
-      launch_gemm(sh, p->probs[1 + pass], p->gtiles[1 + pass], p->n_gtiles[1 + pass], s);  // S = X^T X
+      launch_gemm(sh, p->probs[1 + pass], p->gtiles[1 + pass], p->n_gtiles[1 + pass], p->gemm_small[1 + pass], s);  // S = X^T X
       tick(p, s, kGram[pass]);
       launch_chol_inv(sh, p->chol_smem, pass, 1e-3f, s);  // L, L^{-1}
       tick(p, s, kChol[pass]);
-      launch_gemm(sh, p->probs[4 + pass], p->gtiles[4 + pass], p->n_gtiles[4 + pass], s);  // X L^{-T}
+      launch_gemm(sh, p->probs[4 + pass], p->gtiles[4 + pass], p->n_gtiles[4 + pass], p->gemm_small[4 + pass], s);  // X L^{-T}
       tick(p, s, kTrsm[pass]);
     }
-    launch_gemm(sh, p->probs[7], p->gtiles[7], p->n_gtiles[7], s);  // R = B^T P
+    launch_gemm(sh, p->probs[7], p->gtiles[7], p->n_gtiles[7], p->gemm_small[7], s);  // R = B^T P
     tick(p, s, "gemm_btp");
     launch_colnorm(sh, p->ctiles, p->n_ctiles, a.eps_col, s);       // Q = ColumnNormalize(R)
     tick(p, s, "colnorm");
@@ -504,15 +533,15 @@ void enqueue_phase(dion_plan *p, const StepArgs &a, int32_t phase, cudaStream_t 
       break;
     case DION_PHASE_POWER:  // the branch from the reduced RMMC, then P = B Q on the Dion layers
       launch_gate_reduced(sh, a, s);
-      launch_gemm(sh, p->probs[0], p->gtiles[0], p->n_gtiles[0], s);
+      launch_gemm(sh, p->probs[0], p->gtiles[0], p->n_gtiles[0], p->gemm_small[0], s);
       break;
     case DION_PHASE_ORTHO:  // Orthogonalize the averaged P, then R = B^T P
       for (int pass = 0; pass < 3; ++pass) {
-        launch_gemm(sh, p->probs[1 + pass], p->gtiles[1 + pass], p->n_gtiles[1 + pass], s);
+        launch_gemm(sh, p->probs[1 + pass], p->gtiles[1 + pass], p->n_gtiles[1 + pass], p->gemm_small[1 + pass], s);
         launch_chol_inv(sh, p->chol_smem, pass, 1e-3f, s);
-        launch_gemm(sh, p->probs[4 + pass], p->gtiles[4 + pass], p->n_gtiles[4 + pass], s);
+        launch_gemm(sh, p->probs[4 + pass], p->gtiles[4 + pass], p->n_gtiles[4 + pass], p->gemm_small[4 + pass], s);
       }
-      launch_gemm(sh, p->probs[7], p->gtiles[7], p->n_gtiles[7], s);
+      launch_gemm(sh, p->probs[7], p->gtiles[7], p->n_gtiles[7], p->gemm_small[7], s);
       break;
     default:  // UPDATE: Q_t from the averaged R, error feedback and parameter update, local branch
       launch_colnorm(sh, p->ctiles, p->n_ctiles, a.eps_col, s);

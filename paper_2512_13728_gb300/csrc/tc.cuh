@@ -99,12 +99,6 @@ struct TcPlan {
   uint32_t fb_smem = 0;
   size_t chol_tc_smem = 0, chol_tmem_smem = 0;  // the first pass's Cholesky on tensor cores
   int32_t min_r = 0;
-  // CUDA-core pieces reused by this path (set by the plan)
-  const GemmProblem *const *probs = nullptr;
-  const int4 *const *gtiles = nullptr;
-  const int32_t *n_gtiles = nullptr;
-  const int4 *utiles_simt = nullptr;
-  int32_t n_utiles_simt = 0;
 };
 
 // Number of row ranges each layer's Gram is split into.
