@@ -357,18 +357,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(R_THREADS, 1)
 // Algorithm 1/2 with bf16 gradients: B = M_{t-1} + G is formed on the fly from TMA tiles of M
 // (fp32) and G (bf16) and fed to the pair MMA of P = B Q_{t-1}, so B is read from HBM once.
 // Per {layer, pair p} (CTA c owns 128-row tile 2 p + c) and 64-column k-chunk:
-//   warps 12..15 M through the load/store path: 16-byte cp.async copies written in the same
-//               swizzled layout as two 128 x 32 fp32 SW128 boxes, into the M ring (zero-filled
-//               past the matrix); their landing completes the slot's barrier.  (Each SM's TMA
-//               unit already carries G, Q, Bh and P: M, the largest stream, goes around it);
+//   FB_WM       TMA: M as two 128 x 32 fp32 SW128 boxes into the M ring;
 //   warp 0      TMA: G as one 128 x 64 bf16 SW128 box into the A ring;
-//   warps 6..9  B = M + G in fp32, rounded to bf16 and written in place over the G box, which
+//   converters  (from warp 6) B = M + G in fp32, rounded to bf16 and written in place over the G box, which
 //               has the layout of the K-major A operand; the per-tile sums of B^2 and M_{t-1}^2
 //               (Algorithm 2's ||B|| and Equation 1's ||M_{t-1}||).  The M stage is free again
 //               as soon as it is converted;
-//   warp 11     TMA store of each converted box to Bh (the operand of B^T P); the A slot is
+//   FB_WS       TMA store of each converted box to Bh (the operand of B^T P); the A slot is
 //               refilled once that store has read it and the chunk's MMAs have completed;
-//   warp 10     TMA: this CTA's half of the Q_{t-1} chunk (MN-major boxes, bytes counted on
+//   FB_WQ       TMA: this CTA's half of the Q_{t-1} chunk (MN-major boxes, bytes counted on
 //               CTA 0's barrier) into the Q ring;
 //   warp 1      (CTA 0) the pair MMAs of the chunk once both CTAs' A boxes and Q halves are in;
 //   warps 2..5  drain the 128 x r accumulator into P_raw and its transpose (as in B Q), staged
@@ -379,11 +376,20 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(R_THREADS, 1)
 // With `gated` (the gated modes) the norms pass has already written B into M, computed the
 // norms and run the gate: every role skips the layers that stay local, warp 0 loads no G (it
 // only marks the A slot full) and the converters round M itself and form no norms.
+// HBM-bound on stacks (1.3B, rank 512: 1.85 ms for 11.5 GB; 160M, rank 48: 124 us for 0.72 GB).  M
+// came through 16-byte cp.async copies of four warps before, which kept about 16 KB in flight per SM
+// (4100 cycles per chunk), and each chunk's arrival in CTA 0 took 2700 cycles more (see
+// mbar_arrive_cluster): 2417 us on the 1.3B stack, 174 / 207 us on the 160M stack at ranks 48 / 192
+// (now 124 / 152), 119 us on the 160M block (now 56).
 constexpr int FB_MSTAGES = 3;  // M ring (2 x 16 KB per slot)
 constexpr int FB_ASTAGES = 4;  // G / A ring (16 KB per slot)
-constexpr int FB_QSTAGES = 2;  // Q ring (also the epilogue's staging)
-constexpr int FB_THREADS = 16 * 32;
-constexpr int FB_LOADERS = 128;  // threads of warps 12..15
+// Q ring (also the epilogue's staging, which sets its size to 64 KB at least): 2 stages of 32 KB at
+// r > 256, 4 of 16 KB below
+constexpr int FB_QSTAGES = 4;  // the most
+__host__ __device__ constexpr int fb_qstages(uint32_t bq_boxes) { return bq_boxes <= 2u ? 4 : 2; }
+constexpr int FB_CW = 8;  // converter warps (6 .. 5 + FB_CW; four: 45 us for 43 on ragged blocks); then Q, Bh store, M
+constexpr int FB_CT = FB_CW * 32, FB_WQ = 6 + FB_CW, FB_WS = 7 + FB_CW, FB_WM = 8 + FB_CW;
+constexpr int FB_THREADS = (9 + FB_CW) * 32;
 constexpr uint32_t FB_MBOX = 128u * 32u * 4u;  // 128 x 32 fp32 box of M (16 KB)
 constexpr uint32_t FB_GBOX = 128u * 64u * 2u;  // 128 x 64 bf16 box of G, then of B (16 KB)
 constexpr uint32_t FB_MSLOT = 2u * FB_MBOX;
@@ -392,7 +398,7 @@ constexpr uint32_t FB_Q_OFF = FB_A_OFF + FB_ASTAGES * FB_GBOX;
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(FB_THREADS, 1)
     tc_form_bq_kernel(Shared sh, const int4 *__restrict__ tiles, const int *__restrict__ off,
-                      const LayerMaps *__restrict__ maps, uint32_t qstage_bytes, uint32_t qring_bytes,
+                      const LayerMaps *__restrict__ maps, uint32_t qstage_bytes, uint32_t nq, uint32_t qring_bytes,
                       uint32_t tmem_cols, int gated) {
   chain_enter();
   // gated: the norms pass and the gate ran first; only Dion-branch layers are processed and the
@@ -411,14 +417,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(FB_THREADS, 1)
            *drain = acc_full + 3;
   __shared__ uint32_t tmem_base_s;
   __shared__ int abort_s;
-  __shared__ double red_s[2][4];
+  __shared__ double red_s[2][FB_CW];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const Abort ab{&abort_s};
   const uint32_t rank = cluster_ctarank();
   const int seg = blockIdx.x >> 1;
   if (threadIdx.x == 0) {
     for (int i = 0; i < FB_MSTAGES; ++i) {
-      mbar_init(&mfull[i], FB_LOADERS);  // every loader thread's copies of this CTA's M chunk
+      mbar_init(&mfull[i], 1);   // this CTA's M boxes
       mbar_init(&mempty[i], 1);  // converted
     }
     for (int i = 0; i < FB_ASTAGES; ++i) {
@@ -474,38 +480,30 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(FB_THREADS, 1)
       for (uint32_t k = (it > (uint32_t)FB_ASTAGES ? it - FB_ASTAGES : 0); k < it; ++k)
         mbar_wait(&gempty[k % FB_ASTAGES], (k / FB_ASTAGES) & 1u, sh.status);
     }
-  } else if (warp >= 12) {  // M loads (cp.async)
-    const int lt = threadIdx.x - 12 * 32;  // 0..127
-    uint32_t it = 0;
-    for (int ti = off[seg]; ti < off[seg + 1]; ++ti) {
-      const int4 t = tiles[ti];
-      if (gated && !sh.active[t.x]) continue;
-      const DevLayer &L = sh.layers[t.x];
-      const int kch = (int)((L.n + 63) / 64);
-      const int64_t row0 = (int64_t)(2 * t.y + (int)rank) * 128;
+  } else if (warp == FB_WM) {  // M loads
+    if (lane == 0) {
+      uint32_t it = 0;
       bool ok = true;
-      for (int kc = 0; kc < kch; ++kc, ++it) {
-        const uint32_t sm = it % FB_MSTAGES, pm = (it / FB_MSTAGES) & 1u;
-        if (!named_and(3, FB_LOADERS, ab.wait(&mempty[sm], pm ^ 1u, sh.status))) { ok = false; break; }
-        uint8_t *sM = smem + sm * FB_MSLOT;
-#pragma unroll 4
-        for (int i = 0; i < 16; ++i) {
-          // copy e: row e >> 4, 16-byte chunk e & 15 of the row's 64 columns (a warp covers two
-          // whole 256-byte row segments); box = chunk >> 3, swizzled chunk within the box
-          const uint32_t e = (uint32_t)(i * FB_LOADERS + lt), row = e >> 4, c16 = e & 15u;
-          const uint32_t box = c16 >> 3, ch = c16 & 7u;
-          uint8_t *dst = sM + box * FB_MBOX + row * 128u + ((ch ^ (row & 7u)) << 4);
-          const int64_t gr = row0 + row, gc = (int64_t)kc * 64 + 4 * c16;
-          const bool in = gr < L.m && gc < L.n;
-          const uint32_t bytes = in ? (uint32_t)((L.n - gc < 4 ? L.n - gc : 4) * 4) : 0u;
-          cp_async16(dst, in ? (const void *)(L.M + gr * L.ldm + gc) : (const void *)L.M, bytes);
+      for (int ti = off[seg]; ti < off[seg + 1] && ok; ++ti) {
+        const int4 t = tiles[ti];
+        if (gated && !sh.active[t.x]) continue;
+        const CUtensorMap *map = &maps[t.x].Mf;
+        const int kch = (int)((sh.layers[t.x].n + 63) / 64);
+        const int row0 = (2 * t.y + (int)rank) * 128;  // rows past the matrix read as zeros
+        for (int kc = 0; kc < kch; ++kc, ++it) {
+          const uint32_t sm = it % FB_MSTAGES, pm = (it / FB_MSTAGES) & 1u;
+          if (!ab.wait(&mempty[sm], pm ^ 1u, sh.status)) { ok = false; break; }
+          uint8_t *sM = smem + sm * FB_MSLOT;
+          mbar_expect_tx(&mfull[sm], FB_MSLOT);
+          tma_load_2d(sM, map, &mfull[sm], kc * 64, row0);
+          tma_load_2d(sM + FB_MBOX, map, &mfull[sm], kc * 64 + 32, row0);
         }
-        cp_async_arrive(&mfull[sm]);
       }
-      if (!ok) break;
+      // drain: the last slots' loads have landed (after an abort nothing else waits for them)
+      for (uint32_t k = (it > (uint32_t)FB_MSTAGES ? it - FB_MSTAGES : 0); k < it; ++k)
+        mbar_wait(&mfull[k % FB_MSTAGES], (k / FB_MSTAGES) & 1u, sh.status);
     }
-    cp_async_wait_all();
-  } else if (warp == 10) {  // Q loads
+  } else if (warp == FB_WQ) {  // Q loads
     if (lane == 0) {
       uint32_t it = 0, tcount = 0;
       bool ok = true;
@@ -522,7 +520,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(FB_THREADS, 1)
         if (tcount > 0 && !ab.wait(epi_free, (tcount - 1) & 1u, sh.status)) break;
         ++tcount;
         for (int kc = 0; kc < kch; ++kc, ++it) {
-          const uint32_t s = it % FB_QSTAGES, ph = (it / FB_QSTAGES) & 1u;
+          const uint32_t s = it % nq, ph = (it / nq) & 1u;
           if (!ab.wait(&qempty[s], ph ^ 1u, sh.status)) { ok = false; break; }
           uint8_t *sQ = qring + s * qstage_bytes;
           const uint32_t qb = cluster_addr(&qfull[s], 0);
@@ -535,10 +533,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(FB_THREADS, 1)
           }
         }
       }
-      for (uint32_t k = (it > (uint32_t)FB_QSTAGES ? it - FB_QSTAGES : 0); k < it; ++k)
-        mbar_wait(&qempty[k % FB_QSTAGES], (k / FB_QSTAGES) & 1u, sh.status);
+      for (uint32_t k = (it > nq ? it - nq : 0); k < it; ++k) mbar_wait(&qempty[k % nq], (k / nq) & 1u, sh.status);
     }
-  } else if (warp == 11) {  // Bh stores
+  } else if (warp == FB_WS) {  // Bh stores
     if (lane == 0) {
       uint32_t it = 0;
       bool ok = true;
@@ -576,7 +573,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(FB_THREADS, 1)
         tc_fence_after();
         for (int kc = 0; kc < kch; ++kc, ++it) {
           const uint32_t sg = it % FB_ASTAGES, pg = (it / FB_ASTAGES) & 1u;
-          const uint32_t q = it % FB_QSTAGES, qph = (it / FB_QSTAGES) & 1u;
+          const uint32_t q = it % nq, qph = (it / nq) & 1u;
           if (!ab.wait(&qfull[q], qph, sh.status) || !ab.wait(&afull[sg], pg, sh.status)) { ok = false; break; }
           tc_fence_after();
           const uint32_t aB = smem_u32(aring + sg * FB_GBOX), bB = smem_u32(qring + q * qstage_bytes);
@@ -622,8 +619,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(FB_THREADS, 1)
       ++tcount;
     }
     if (leader) bulk_wait<0>();
-  } else {  // warps 6..9: B = M + G
-    const int ct = threadIdx.x - 6 * 32, cw = warp - 6;  // 0..127, 0..3
+  } else {  // converters: B = M + G
+    const int ct = threadIdx.x - 6 * 32, cw = warp - 6;  // 0 .. FB_CT - 1, 0 .. FB_CW - 1
     uint32_t it = 0;
     for (int ti = off[seg]; ti < off[seg + 1]; ++ti) {
       const int4 t = tiles[ti];
@@ -642,10 +639,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(FB_THREADS, 1)
           uint8_t *sG = aring + sg * FB_GBOX;
           float fb = 0.f, fm = 0.f;
 #pragma unroll 4
-          for (int i = 0; i < 8; ++i) {
+          for (int i = 0; i < 1024 / FB_CT; ++i) {
             // element group e: rows 8 (e >> 6) + (e & 7), 16-byte chunk (e >> 3) & 7 (8 columns);
             // the 8 threads of a shared-memory phase take 8 rows of one chunk (distinct banks)
-            const uint32_t e = (uint32_t)(i * 128 + ct);
+            const uint32_t e = (uint32_t)(i * FB_CT + ct);
             const uint32_t row = (e & 7u) + 8u * (e >> 6), c = (e >> 3) & 7u, sw = row & 7u;
             uint4 *ga = reinterpret_cast<uint4 *>(sG + row * 128u + ((c ^ sw) << 4));
             const uint4 g = gated ? make_uint4(0u, 0u, 0u, 0u) : *ga;  // gated: B is in M, no G
@@ -673,7 +670,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(FB_THREADS, 1)
           accm += (double)fm;
           fence_async_smem();  // the A box is read by the MMA and the Bh store (async proxy)
         }
-        if (!named_and(2, 128, in)) { ok = false; break; }
+        if (!named_and(2, FB_CT, in)) { ok = false; break; }
         if (ct == 0) {
           mbar_arrive(&mempty[sm]);
           mbar_arrive_cluster(cluster_addr(&afull[sg], 0));
@@ -691,11 +688,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(FB_THREADS, 1)
         red_s[0][cw] = accb;
         red_s[1][cw] = accm;
       }
-      named_sync(2, 128);
+      named_sync(2, FB_CT);
       if (ct == 0 && !gated && (int64_t)tr * 128 < L.m) {
         const int slot = L.bpart_off + tr;
-        sh.bpart[2 * slot] = (red_s[0][0] + red_s[0][1]) + (red_s[0][2] + red_s[0][3]);
-        sh.bpart[2 * slot + 1] = (red_s[1][0] + red_s[1][1]) + (red_s[1][2] + red_s[1][3]);
+        double sb = 0.0, sm = 0.0;
+        for (int w = 0; w < FB_CW; ++w) {
+          sb += red_s[0][w];
+          sm += red_s[1][w];
+        }
+        sh.bpart[2 * slot] = sb;
+        sh.bpart[2 * slot + 1] = sm;
       }
     }
   }
@@ -727,8 +729,8 @@ uint32_t form_bq_smem(int nstages, uint32_t stage_bytes) {
   return 1024u + nstages * stage_bytes + STG_BYTES + 512u;  // + barriers
 }
 uint32_t btp_smem(int nstages, uint32_t stage_bytes) { return form_bq_smem(nstages, stage_bytes); }
-// Q ring of the fused kernel: FB_QSTAGES Q chunks, at least the epilogue's 4 staging boxes
-uint32_t fused_bq_qring(uint32_t bq_boxes) { return std::max(FB_QSTAGES * bq_boxes * BOX64, 4u * EPI_BOX); }
+// Q ring of the fused kernel: its stages, at least the epilogue's 4 staging boxes
+uint32_t fused_bq_qring(uint32_t bq_boxes) { return std::max(fb_qstages(bq_boxes) * bq_boxes * BOX64, 4u * EPI_BOX); }
 uint32_t fused_bq_smem(uint32_t bq_boxes) { return 1024u + FB_Q_OFF + fused_bq_qring(bq_boxes) + 512u; }
 
 cudaError_t setup_bq_kernels(uint32_t f_smem, uint32_t r_smem, bool x3) {
@@ -751,7 +753,7 @@ cudaError_t setup_fused_bq_kernel(uint32_t smem) {
 void launch_fused_bq(const Shared &sh, const TcPlan &tp, bool gated, cudaStream_t s) {
   if (tp.d_bq.grid <= 0) return;
   launch_chained(tc_form_bq_kernel, 2 * tp.d_bq.grid, FB_THREADS, tp.fb_smem, s, 
-      sh, tp.d_bq.tiles, tp.d_bq.off, tp.maps, tp.bq_boxes * BOX64, fused_bq_qring(tp.bq_boxes), tp.tmem_cols,
+      sh, tp.d_bq.tiles, tp.d_bq.off, tp.maps, tp.bq_boxes * BOX64, (uint32_t)fb_qstages(tp.bq_boxes), fused_bq_qring(tp.bq_boxes), tp.tmem_cols,
       gated ? 1 : 0);
 }
 

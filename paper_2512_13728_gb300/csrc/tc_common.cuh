@@ -180,8 +180,13 @@ __device__ __forceinline__ void tma_load_2d_pair(void *dst, const CUtensorMap *m
       "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1)
       : "memory");
 }
+// Arrival on a barrier of either CTA (`bar` is a shared::cluster address), with the instruction's
+// default release at CTA scope: what it publishes are shared-memory writes that each writer has
+// fenced to the async proxy (fence_async_smem) before a barrier among them, and TMEM reads ordered
+// by tcgen05.fence.  With .release.cluster the arriving thread waited ~2700 cycles here, per
+// 64-column chunk in the fused buffer kernel.
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
 // ------------------------------------------------------------------------ cluster ---
@@ -276,18 +281,6 @@ __device__ __forceinline__ void tma_reduce_add_2d(const CUtensorMap *map, const 
 // Orders this thread's generic-proxy global accesses with async-proxy (TMA) accesses, both ways.
 __device__ __forceinline__ void fence_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 
-// ------------------------------------------- per-thread async copies (load/store path) ---
-// 16-byte global -> shared copy through L2 (not L1); bytes past src_bytes (0..16) are zero.
-__device__ __forceinline__ void cp_async16(void *dst, const void *src, uint32_t src_bytes) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(src_bytes)
-               : "memory");
-}
-// One arrival on `bar` once every cp.async this thread issued so far has landed (the arrival
-// counts toward the barrier's expected count).
-__device__ __forceinline__ void cp_async_arrive(uint64_t *bar) {
-  asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 // wait until at most N committed bulk groups of this thread still read shared memory
 template <int N>
 __device__ __forceinline__ void bulk_wait_read() {
