@@ -16,8 +16,8 @@
 // TB/s at rank 48, these 6.3); the pair MMA halves the R and Q_t bytes each SM receives, which pays
 // for the larger stream buffers.  Measured before (a CTA per 128 x 128 tile, 64-byte segments issued
 // by the epilogue's first thread, a barrier per sub-chunk), with a stream warp alone, and now:
-// 290 / 262 / 256 us on the 160M stack at rank 192, 542 / 475 / 437 us on half of the 350M stack
-// (B in M), 1003 / 917 / 908 us on all of it with split operands, 3826 / 4075 / 3726 us on the 1.3B
+// 290 / 262 / 250 us on the 160M stack at rank 192, 542 / 475 / 455 us on half of the 350M stack
+// (B in M), 1003 / 917 / 829 us on all of it with split operands, 3826 / 4075 / 3650 us on the 1.3B
 // stack at rank 512.  The same loads as cp.async copies from four more warps: 257, 459, 943, 4024.
 #include "tc.cuh"
 #include "tc_common.cuh"
@@ -39,20 +39,22 @@ constexpr uint32_t U_IDESC = idesc_bf16(256, 128, false, false);
 // + Pl Rh^T, the same for P Q_t^T), in 32-wide K chunks (64-byte swizzle): 32 KB either way.  The
 // rest of shared memory holds stream sub-chunks of M, X and, where the kernel forms B = M + G
 // itself (GIN), G: 40 KB or 32 KB each.
-// DEEP takes a fourth operand stage in place of a stream buffer, for ranks above kDeepRank: there a
+// DEEP takes a fourth operand stage and a stream buffer less, for ranks above kDeepRank: there a
 // tile's operands (r / 64 chunks of 32 KB) outweigh its streams, and more stream loads in flight
-// only delay them: 3726 us against 4553 on the 1.3B stack at rank 512, 1041 / 1108 on twelve
-// 1536-wide blocks at rank 384, 1051 / 1058 at rank 320, and the other way round at 272 (1067 /
-// 1034); with B in M 959 / 993 at rank 384, 936 / 941 at 320.
-constexpr int kDeepRank = 304;  // between the ranks measured on either side
+// only delay them.  DEEP / not, us: forming B itself (GIN) 459 / 484 on twelve 1024-wide blocks at
+// rank 256, 255 / 250 on the 160M stack at rank 192; with B in M 977 / 1058 on twelve 1536-wide
+// blocks at rank 384, 461 / 468 on eight 1280-wide ones at rank 320, 440 / 410 at rank 256.  Four
+// stream buffers with B in M: 484 us for 455 with three on half of the 350M stack.  BF16X3 fits four
+// stages and three buffers: 829 us on the 350M stack, 905 with three stages.
+constexpr int kDeepRankG = 224, kDeepRank = 288;  // with G; with B in M (between the ranks measured on either side)
 template <bool X3, bool GIN, bool DEEP>
 struct UpdCfg {
   static constexpr uint32_t KW = X3 ? 32u : 64u;  // K chunk width (bf16 elements per operand row)
   static constexpr uint32_t PB = 128u * KW * 2u, BB = 64u * KW * 2u;  // bytes of a P box, of an R or Q_t box
   static constexpr uint32_t HALF = PB + 2u * BB;  // P, R, Q_t; BF16X3: then their low halves
-  static constexpr int STAGES = DEEP ? 4 : 3;
+  static constexpr int STAGES = DEEP || X3 ? 4 : 3;
   static constexpr uint32_t STAGE = (X3 ? 2u : 1u) * HALF;
-  static constexpr int EBUF = GIN ? (DEEP ? 2 : 3) : (DEEP ? 3 : 4);
+  static constexpr int EBUF = DEEP ? 2 : 3;
   static constexpr uint32_t EBUFB = 2u * U_EBOX + (GIN ? U_GBOX : 0u);  // bytes of one sub-chunk buffer
   static constexpr uint32_t SMEM = 1024u + STAGES * STAGE + EBUF * EBUFB + 256u;
   static_assert(EBUFB % 1024u == 0 && HALF % 1024u == 0, "every box stays aligned to its swizzle atom");
@@ -370,7 +372,7 @@ static void launch_as(const Shared &sh, const TcPlan &tp, float mu, float eta, f
 void launch_update(const Shared &sh, const TcPlan &tp, float mu, float eta, float keep, cudaStream_t s) {
   if (tp.d_update.grid <= 0) return;
   const bool gin = tp.defers && !sh.b_in_m;  // else B is in M
-  const bool deep = tp.max_r > kDeepRank;
+  const bool deep = tp.max_r > (gin ? kDeepRankG : kDeepRank);
   if (tp.precision == DION_PREC_BF16X3) launch_as<true, false, false>(sh, tp, mu, eta, keep, s);
   else if (gin && deep) launch_as<false, true, true>(sh, tp, mu, eta, keep, s);
   else if (gin) launch_as<false, true, false>(sh, tp, mu, eta, keep, s);

@@ -617,9 +617,9 @@ def test_column_scaling_ranks(rank):
 
 
 @pytest.mark.parametrize("gate", ["always", "per_layer"])
-@pytest.mark.parametrize("rank", [64, 65, 256, 304, 305, 352])
+@pytest.mark.parametrize("rank", [64, 65, 224, 225, 288, 289, 304, 305, 352])
 def test_update_pair_tiles(rank, gate):
-    """The update's pair tiles at the edges of its K chunks (64) and of its two ring shapes (rank 304),
+    """The update's pair tiles at the edges of its K chunks (64) and of its ring shapes (ranks 224 and 288),
     with an odd number of row tiles (the pair's second tile empty), a column tile narrower than one
     CTA's half, and a last 32-column sub-chunk that is partial; G added in the update (always) and B
     already in M (per layer)."""
