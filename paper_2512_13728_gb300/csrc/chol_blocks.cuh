@@ -7,7 +7,7 @@
 
 namespace cd {
 
-constexpr int CB = 32, CBP = CB + 1;
+constexpr int CB = 32;
 
 // Row-tile index of tile p in a lower trapezoid whose row tile b holds c1 + b tiles: the
 // largest b with b c1 + b (b - 1) / 2 <= p.
@@ -30,38 +30,8 @@ __device__ __forceinline__ void store8(float *p, const float w[8]) {
   *reinterpret_cast<float4 *>(p + 4) = make_float4(w[4], w[5], w[6], w[7]);
 }
 
-// The 32 x 32 diagonal-block kernels below are unrolled through template recursion so that
-// every register array is indexed by constants (no local-memory copies).
-// Column J of the Cholesky factor of a 32 x 32 block held one row per lane.
-template <int J>
-__device__ __forceinline__ void chol32_col(float (&v)[CB], float *rd, int lane, bool &ok) {
-  if constexpr (J < CB) {
-    const float piv = __shfl_sync(0xffffffffu, v[J], J);
-    ok = ok && (piv > 0.f) && (piv < INFINITY);  // uniform: every lane sees the same pivot
-    const float rs = rsqrtf(piv), sq = piv * rs;
-    v[J] = (lane == J) ? sq : (lane > J ? v[J] * rs : 0.f);
-    if (lane == 0) rd[J] = rs;
-#pragma unroll
-    for (int k = J + 1; k < CB; ++k) {
-      const float lkj = __shfl_sync(0xffffffffu, v[J], k);
-      if (lane >= k) v[k] = fmaf(-v[J], lkj, v[k]);
-    }
-    chol32_col<J + 1>(v, rd, lane, ok);
-  }
-}
-
-// Row I of the forward substitution L x = e_lane (lane c computes column c of L^{-1}).
-template <int I>
-__device__ __forceinline__ void trinv32_row(float (&x)[CB], const float *D, const float *rd, int lane) {
-  if constexpr (I < CB) {
-    float a = (I == lane) ? 1.f : 0.f;
-#pragma unroll
-    for (int k = 0; k < I; ++k) a = fmaf(-D[I * CBP + k], x[k], a);
-    x[I] = a * rd[I];
-    trinv32_row<I + 1>(x, D, rd, lane);
-  }
-}
-
+// Unrolled through template recursion so that every register array is indexed by constants (no
+// local-memory copies).
 // v <- T v for a lower-triangular 32 x 32 T (row-major, row pitch LD), in place from the bottom.
 template <int C, int LD = CB>
 __device__ __forceinline__ void trmv32(float (&v)[CB], const float *T) {
@@ -83,8 +53,8 @@ __device__ __forceinline__ void trmv32(float (&v)[CB], const float *T) {
 // move down one place per column (v[0] is the current column), so that the code stays small (fully
 // unrolled columns cost 20K cycles of instruction fetches the first time through) and the work
 // shrinks with the segments.  Bound by the elimination's chain from column to column; about 5K
-// cycles against 12.6K for chol32_col and trinv32_row in one warp.
-struct DiagScratch {
+// cycles against 12.6K for one warp that factored with unrolled shuffles and then inverted.
+struct alignas(16) DiagScratch {
   // current column, unscaled, from the pivot down; [CB]: the next diagonal entry ([CB + 1]: dump for
   // the lanes that do not hold it, which spares the loop a divergent branch)
   float col[2][CB + 4];

@@ -6,7 +6,7 @@
 // starts as the lower triangle of S (+ the shift on the diagonal).  Before step k, for rows
 // i >= k0, W[i][j] holds the Schur complement for j >= k0 and U[i][j] = -sum_{K < k} L[i, K]
 // L^{-1}[K, j] for j < k0.  Step k:
-//   warp 0     factors and inverts the 32 x 32 diagonal block in registers (D_k = L_kk^{-1});
+//   warps 0, 15 factor and invert the 32 x 32 diagonal block (D_k = L_kk^{-1}, chol_blocks.cuh);
 //   warps 1..  finish block row k of L^{-1} (D_k U[k, :k0]) and form the panel
 //              L[i, k] = A[i, k] D_k^T below the block; block k's columns of those rows are
 //              then zeroed (their U values start from zero);
@@ -110,7 +110,7 @@ __device__ __forceinline__ void issue_unit(const TcState &ts, uint32_t g, int a0
 // 0: factored; 1: a pivot was not positive and finite (uniform over the block); 2: a wait for
 // the tensor cores gave up.
 __device__ int chol_inverse_tc(const float *S, float *__restrict__ W, int r, int64_t ls, float shift,
-                               float *D, float *DI, float *rd, int *bad, TcState &ts, int32_t *status) {
+                               float *DI, DiagScratch &diag, int *bad, TcState &ts, int32_t *status) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, q = tid - 32;
   // W <- lower triangle of S + shift I (coalesced; the upper triangle is never read before each
   // row's own step overwrites it)
@@ -139,14 +139,7 @@ __device__ int chol_inverse_tc(const float *S, float *__restrict__ W, int r, int
         if (j > lane) v[j] = 0.f;
         if (j == lane && lane >= nb) v[j] = 1.f;
       }
-      bool ok = true;
-      chol32_col<0>(v, rd, lane, ok);
-#pragma unroll
-      for (int j = 0; j < CB; ++j) D[lane * CBP + j] = v[j];
-      __syncwarp();
-      trinv32_row<0>(v, D, rd, lane);  // lane c: column c of D_k = L_kk^{-1}
-#pragma unroll
-      for (int i = 0; i < CB; ++i) DI[i * CB + lane] = v[i];
+      const bool ok = diag_factor<1>(v, diag, lane);
       if (lane == 0) *bad = ok ? 0 : 1;
     } else if (q < k0) {
       // ---- column q of U[k, :k0]
@@ -160,6 +153,7 @@ __device__ int chol_inverse_tc(const float *S, float *__restrict__ W, int r, int
       load8(p + 16, v + 16);
       load8(p + 24, v + 24);
     }
+    if (warp == kThreads / 32 - 1) diag_invert<1, CB>(diag, DI, lane);  // D_k, a segment behind warp 0
     __syncthreads();
     if (*bad) return 1;
     if (warp > 0 && q < k0 + t) {
@@ -270,10 +264,9 @@ __global__ void __launch_bounds__(kThreads, 1) chol_inv_tc_kernel(Shared sh, con
   ts.yth = smem;
   ts.ytl = smem + (size_t)ts.ya * 128;
   ts.box = ts.ytl + (size_t)ts.ya * 128;
-  float *D = reinterpret_cast<float *>(ts.box + (kThreads / 32) * kBox);  // CB x CBP
-  float *rd = D + CB * CBP;                                                 // CB
-  float *DI = rd + 32;                                                      // CB x CB
-  ts.bars = reinterpret_cast<uint64_t *>(DI + CB * CB);
+  float *DI = reinterpret_cast<float *>(ts.box + (kThreads / 32) * kBox);  // CB x CB
+  DiagScratch &diag = *reinterpret_cast<DiagScratch *>(DI + CB * CB);
+  ts.bars = reinterpret_cast<uint64_t *>(&diag + 1);
   ts.unit = 0;
   ts.wmap = &maps[l].Linv32;
   __shared__ uint32_t tmem_base_s;
@@ -300,7 +293,7 @@ __global__ void __launch_bounds__(kThreads, 1) chol_inv_tc_kernel(Shared sh, con
   tc_fence_after();
   ts.tmem = tmem_base_s;
 
-  int res = chol_inverse_tc(S, Li, r, ls, 0.f, D, DI, rd, &bad, ts, sh.status);
+  int res = chol_inverse_tc(S, Li, r, ls, 0.f, DI, diag, &bad, ts, sh.status);
   bool shifted = false;
   if (res == 1) {  // shifted retry from S + s I (shifted CholeskyQR, as in chol_inv_kernel)
     double tr = 0.0;
@@ -311,7 +304,7 @@ __global__ void __launch_bounds__(kThreads, 1) chol_inv_tc_kernel(Shared sh, con
     const double u = 5.9604644775390625e-8;  // 2^-24
     const double sft = 11.0 * ((double)Ly.m * r + (double)r * (r + 1)) * u * trace_s;
     shifted = true;
-    res = (trace_s > 0.0 && isfinite(trace_s)) ? chol_inverse_tc(S, Li, r, ls, (float)sft, D, DI, rd, &bad, ts, sh.status)
+    res = (trace_s > 0.0 && isfinite(trace_s)) ? chol_inverse_tc(S, Li, r, ls, (float)sft, DI, diag, &bad, ts, sh.status)
                                                : 1;
   }
   if (tid == 0) {
@@ -338,7 +331,7 @@ __global__ void __launch_bounds__(kThreads, 1) chol_inv_tc_kernel(Shared sh, con
 
 size_t chol_tc_smem(int32_t max_r) {
   return 1024 + 2 * (size_t)yt_rows(max_r) * 128 + (kThreads / 32) * (size_t)kBox +
-         sizeof(float) * (CB * CBP + 32 + CB * CB) + 64;
+         sizeof(float) * CB * CB + sizeof(DiagScratch) + 64;
 }
 
 cudaError_t prepare_chol_inv_tc(int32_t max_r, size_t *smem_out) {

@@ -582,8 +582,8 @@ void launch_gemm(const Shared &sh, const GemmProblem *probs, const int4 *tiles, 
 //   W[i][j], j >= k0 : the Schur complement S - L[:, :k0] L[:, :k0]^T (lower triangle),
 //   W[i][j], j <  k0 : U[i][j] = -sum_{K < k} L[i, K] L^{-1}[K, j],
 // and rows above k0 hold their final L^{-1}.  Step k:
-//   warp 0     factors the 32 x 32 diagonal block in registers (shuffles) and inverts it
-//              (D_k = L_kk^{-1}), while warps 1..15 load the rest of block row k's U and the
+//   warps 0, 15 factor and invert the 32 x 32 diagonal block (D_k = L_kk^{-1}; chol_blocks.cuh),
+//              while warps 1..15 load the rest of block row k's U and the
 //              panel rows below the block;
 //   warps 1..  finish block row k: L^{-1}[k, :k0] = D_k U[k, :k0], and form the panel
 //              L[i, k] = A[i, k] D_k^T of every row below;
@@ -611,11 +611,10 @@ __device__ __forceinline__ void load8y(const float *row, int c0, float w[8]) {  
 }
 
 // W <- L^{-1} with L L^T = S + shift I (lower triangle of S read).  Returns false, uniformly
-// over the block, on a pivot that is not positive and finite.  Shared memory: D (CB x CBP),
-// DI (CB x CB), rd (CB reciprocal pivots), Y (CB x ldy, ldy >= r rounded up to 8, columns
+// over the block, on a pivot that is not positive and finite.  Shared memory: DI (CB x CB), Y (CB x ldy, ldy >= r rounded up to 8, columns
 // >= r zero).
 __device__ bool chol_inverse(const float *S, float *__restrict__ W, int r, int64_t ls, float shift,
-                             float *D, float *DI, float *rd, float *Y, int ldy, int *bad) {
+                             float *DI, DiagScratch &diag, float *Y, int ldy, int *bad) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, q = tid - 32;
   for (int k0 = 0; k0 < r; k0 += CB) {
     const int nb = min(CB, r - k0), R0 = k0 + nb, t = r - R0;
@@ -639,15 +638,7 @@ __device__ bool chol_inverse(const float *S, float *__restrict__ W, int r, int64
         if (j > lane) v[j] = 0.f;
         if (j == lane) v[j] = (lane < nb) ? v[j] + dshift : 1.f;
       }
-      bool ok = true;
-      chol32_col<0>(v, rd, lane, ok);
-#pragma unroll
-      for (int j = 0; j < CB; ++j) D[lane * CBP + j] = v[j];
-      __syncwarp();
-      // lane c: column c of D_k = L_kk^{-1} by forward substitution on e_c
-      trinv32_row<0>(v, D, rd, lane);
-#pragma unroll
-      for (int i = 0; i < CB; ++i) DI[i * CB + lane] = v[i];
+      const bool ok = diag_factor<1>(v, diag, lane);
       if (lane == 0) *bad = ok ? 0 : 1;
     } else if (q < k0) {
       // ---- column q of U[k, :k0]
@@ -661,6 +652,7 @@ __device__ bool chol_inverse(const float *S, float *__restrict__ W, int r, int64
       load8(p + 16, v + 16);
       load8(p + 24, v + 24);
     }
+    if (warp == kCholThreads / 32 - 1) diag_invert<1, CB>(diag, DI, lane);  // D_k, a segment behind warp 0
     __syncthreads();
     if (*bad) return false;
     if (warp > 0 && q < k0 + t) {
@@ -824,10 +816,9 @@ __global__ void __launch_bounds__(kCholThreads, 1) chol_inv_kernel(Shared sh, in
   float *Li = Ly.Linv;
   sum_gram_parts<kCholThreads>(Ly.S, r, ls, Ly.s_parts, Ly.s_stride);
   extern __shared__ __align__(16) float smem[];
-  float *D = smem;                 // CB x CBP
-  float *rd = D + CB * CBP;        // CB
-  float *DI = rd + 32;             // CB x CB (16-byte aligned)
-  float *Y = DI + CB * CB;         // CB x ldy
+  float *DI = smem;                // CB x CB
+  DiagScratch &diag = *reinterpret_cast<DiagScratch *>(DI + CB * CB);
+  float *Y = reinterpret_cast<float *>(&diag + 1);  // CB x ldy
   const int ldy = (r + 7) / 8 * 8;
   __shared__ int bad;
   __shared__ double red[kCholThreads / 32];
@@ -926,7 +917,7 @@ __global__ void __launch_bounds__(kCholThreads, 1) chol_inv_kernel(Shared sh, in
     if (ysw(e % ldy) >= r) Y[e] = 0.f;
   __syncthreads();
 
-  bool ok = chol_inverse(S, Li, r, ls, 0.f, D, DI, rd, Y, ldy, &bad);
+  bool ok = chol_inverse(S, Li, r, ls, 0.f, DI, diag, Y, ldy, &bad);
   bool shifted = false;
   if (!ok) {  // shifted retry from S + s I
     double tr = 0.0;
@@ -938,7 +929,7 @@ __global__ void __launch_bounds__(kCholThreads, 1) chol_inv_kernel(Shared sh, in
     const double u = 5.9604644775390625e-8;  // 2^-24
     const double shift = 11.0 * ((double)Ly.m * r + (double)r * (r + 1)) * u * trace_s;
     shifted = true;
-    ok = (trace_s > 0.0) && isfinite(trace_s) && chol_inverse(S, Li, r, ls, (float)shift, D, DI, rd, Y, ldy, &bad);
+    ok = (trace_s > 0.0) && isfinite(trace_s) && chol_inverse(S, Li, r, ls, (float)shift, DI, diag, Y, ldy, &bad);
   }
   if (tid == 0) {
     if (pass == 0) sh.orth_shifted[l] = shifted ? 1 : 0;
@@ -954,7 +945,7 @@ __global__ void __launch_bounds__(kCholThreads, 1) chol_inv_kernel(Shared sh, in
 
 cudaError_t prepare_chol_inv(int32_t max_r, size_t *smem_out) {
   const int ldy = (max_r + 7) / 8 * 8;
-  const size_t smem = sizeof(float) * (CB * CBP + 32 + CB * CB + (size_t)CB * std::max(ldy, 8));
+  const size_t smem = sizeof(DiagScratch) + sizeof(float) * (CB * CB + (size_t)CB * std::max(ldy, 8));
   *smem_out = smem;
   return cudaFuncSetAttribute(chol_inv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
