@@ -782,54 +782,114 @@ void launch_btp(const Shared &sh, const TcPlan &tp, cudaStream_t s) {
 }
 
 // Data-parallel phases.  P_raw^T (r x m, the first Gram's operand) from the averaged P_raw:
-// tile = {layer, 128-row block of P_raw}, 32 x 32 sub-tiles through shared memory.
+// tile = {layer, 128-row block of P_raw}, 128 x 32 at a time through shared memory (16 independent
+// loads per thread between barriers, 512-byte runs of P_raw^T; 32 x 32 at a time took 72 us on
+// the 160M stack at rank 192, 23 us now).
 __global__ void __launch_bounds__(256) transpose_praw_kernel(Shared sh, const int4 *tiles) {
   chain_enter();
   const int4 t = tiles[blockIdx.x];
   DION_TILE_CHECK(t.x >= 0 && t.x < sh.num_layers && t.y >= 0 && (int64_t)t.y * 128 < sh.layers[t.x].m, sh.status);
   if (!sh.active[t.x]) return;
   const DevLayer &L = sh.layers[t.x];
-  __shared__ float tile[32][33];
+  __shared__ float tile[128][33];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t row_end = min((int64_t)t.y * 128 + 128, L.m);
-  for (int64_t r0 = (int64_t)t.y * 128; r0 < row_end; r0 += 32) {
-    for (int64_t c0 = 0; c0 < L.r; c0 += 32) {
-      for (int i = warp; i < 32; i += 8) {  // rows r0 + i, columns c0 + lane of P_raw
-        const int64_t row = r0 + i, col = c0 + lane;
-        tile[i][lane] = (row < row_end && col < L.r) ? L.P_raw[row * L.ldp + col] : 0.f;
-      }
-      __syncthreads();
-      for (int i = warp; i < 32; i += 8) {  // row c0 + i of P_raw^T, columns r0 + lane
-        const int64_t col = c0 + i, row = r0 + lane;
-        if (col < L.r && row < row_end) L.PT_raw[col * L.ldmt + row] = tile[lane][i];
-      }
-      __syncthreads();
+  const int64_t row0 = (int64_t)t.y * 128;
+  const int nrows = (int)min((int64_t)128, L.m - row0), r = (int)L.r;
+  const int64_t ldp = L.ldp, ldmt = L.ldmt;
+  const float *src = L.P_raw + row0 * ldp;
+  float *dst = L.PT_raw + row0;
+  float v[16];  // rows warp + 8 u, column c0 + lane of P_raw; the next columns' loads run under the stores
+  auto load = [&](int c0) {
+#pragma unroll
+    for (int u = 0; u < 16; ++u) {
+      const int i = warp + 8 * u;
+      v[u] = (i < nrows && c0 + lane < r) ? src[i * ldp + c0 + lane] : 0.f;
     }
+  };
+  load(0);
+  for (int c0 = 0; c0 < r; c0 += 32) {
+#pragma unroll
+    for (int u = 0; u < 16; ++u) tile[warp + 8 * u][lane] = v[u];
+    __syncthreads();
+    if (c0 + 32 < r) load(c0 + 32);
+#pragma unroll
+    for (int u = 0; u < 16; ++u) {  // row c0 + c of P_raw^T, columns row0 + i
+      const int c = warp + 8 * (u & 3), i = lane + 32 * (u >> 2);
+      if (c0 + c < r && i < nrows) dst[(c0 + c) * ldmt + i] = tile[i][c];
+    }
+    __syncthreads();
   }
 }
 
 // R's bf16 copy (and low half in BF16X3) and the per-tile column sums of squares that
-// ColumnNormalize reads, from the averaged R: tile = {layer, 128-row block of R}; thread j
-// takes columns j and j + 256, rows in order (fp32 over 32 rows, then fp64).
+// ColumnNormalize reads, from the averaged R: tile = {layer, 128-row block of R}.  A thread owns a
+// 16-byte group of columns of every rg-th row, as in colnorm_scale_kernel (a column per thread, one
+// 4-byte load at a time down 128 rows, took 86 us on the 160M stack at rank 192, 24 us now);
+// squares are summed in fp32 over at most 32 rows, then in fp64, in a fixed order.
 __global__ void __launch_bounds__(256) r_refresh_kernel(Shared sh, const int4 *tiles) {
   chain_enter();
   const int4 t = tiles[blockIdx.x];
   DION_TILE_CHECK(t.x >= 0 && t.x < sh.num_layers && t.y >= 0 && (int64_t)t.y * 128 < sh.layers[t.x].n, sh.status);
   if (!sh.active[t.x]) return;
   const DevLayer &L = sh.layers[t.x];
-  const int64_t r0 = (int64_t)t.y * 128, r1 = min(r0 + 128, L.n);
-  for (int64_t c = threadIdx.x; c < L.r; c += 256) {
-    double acc = 0.0;
-    float f = 0.f;
-    for (int64_t i = r0; i < r1; ++i) {
-      const float v = L.R[i * L.ldp + c];
-      f = fmaf(v, v, f);
-      if (((i - r0) & 31) == 31) { acc += (double)f; f = 0.f; }
-      const __nv_bfloat16 h = __float2bfloat16_rn(v);
-      L.R_hi[i * L.ldp + c] = h;
-      if (L.R_lo != nullptr) L.R_lo[i * L.ldp + c] = __float2bfloat16_rn(v - __bfloat162float(h));
+  __shared__ double part[256][4];
+  const int r = (int)L.r, r4 = (r + 3) / 4;  // r <= 512: at most 128 groups
+  int lg = 7;
+  while (lg > 0 && (1 << (lg - 1)) >= r4) --lg;
+  const int c4 = threadIdx.x & ((1 << lg) - 1), rg = threadIdx.x >> lg, nrg = 256 >> lg;
+  const int64_t r0 = (int64_t)t.y * 128, ldp = L.ldp;
+  const int nrows = (int)min((int64_t)128, L.n - r0);
+  if (c4 < r4) {  // the last group may reach into the rows' padding, which nothing reads
+    const float *R = L.R + r0 * ldp + 4 * c4;
+    __nv_bfloat16 *hi = L.R_hi + r0 * ldp + 4 * c4;
+    __nv_bfloat16 *lo = L.R_lo == nullptr ? nullptr : L.R_lo + r0 * ldp + 4 * c4;
+    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+    float f[4] = {0.f, 0.f, 0.f, 0.f};
+    int cnt = 0;
+    for (int i0 = rg; i0 < nrows; i0 += 8 * nrg) {
+      float4 v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        v[u] = i0 + u * nrg < nrows ? *reinterpret_cast<const float4 *>(R + (i0 + u * nrg) * ldp)
+                                    : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        if (i0 + u * nrg >= nrows) break;
+        const int64_t o = (i0 + u * nrg) * ldp;
+        f[0] = fmaf(v[u].x, v[u].x, f[0]); f[1] = fmaf(v[u].y, v[u].y, f[1]);
+        f[2] = fmaf(v[u].z, v[u].z, f[2]); f[3] = fmaf(v[u].w, v[u].w, f[3]);
+        const __nv_bfloat162 h01 = __floats2bfloat162_rn(v[u].x, v[u].y), h23 = __floats2bfloat162_rn(v[u].z, v[u].w);
+        uint2 hv;
+        hv.x = *reinterpret_cast<const uint32_t *>(&h01);
+        hv.y = *reinterpret_cast<const uint32_t *>(&h23);
+        *reinterpret_cast<uint2 *>(hi + o) = hv;
+        if (lo != nullptr) {
+          const float2 f01 = __bfloat1622float2(h01), f23 = __bfloat1622float2(h23);
+          const __nv_bfloat162 l01 = __floats2bfloat162_rn(v[u].x - f01.x, v[u].y - f01.y);
+          const __nv_bfloat162 l23 = __floats2bfloat162_rn(v[u].z - f23.x, v[u].w - f23.y);
+          uint2 lv;
+          lv.x = *reinterpret_cast<const uint32_t *>(&l01);
+          lv.y = *reinterpret_cast<const uint32_t *>(&l23);
+          *reinterpret_cast<uint2 *>(lo + o) = lv;
+        }
+      }
+      if (++cnt == 4) {  // 32 rows
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          acc[e] += (double)f[e];
+          f[e] = 0.f;
+        }
+        cnt = 0;
+      }
     }
-    L.colsq[(int64_t)t.y * L.ldp + c] = acc + (double)f;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) part[threadIdx.x][e] = acc[e] + (double)f[e];
+  }
+  __syncthreads();
+  for (int c = threadIdx.x; c < r; c += 256) {
+    double s = 0.0;
+    for (int g = 0; g < nrg; ++g) s += part[(g << lg) + (c >> 2)][c & 3];
+    L.colsq[(int64_t)t.y * ldp + c] = s;
   }
 }
 
