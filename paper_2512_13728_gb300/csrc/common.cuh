@@ -188,6 +188,41 @@ __device__ __forceinline__ float bf16_bits_to_float(uint32_t bits16) {
   return __uint_as_float(bits16 << 16);
 }
 
+// The fp64 sum over a warp's lanes of N non-negative fp32 values each, the same in every lane.  The
+// partial sums are unevaluated pairs of fp32 values (Knuth's two-sum keeps each addition's rounding
+// error: about 48 bits), added in a fixed shuffle tree in which the order of two operands does not
+// change the result: sm_103a runs fp64 at two lanes per SM, and the same tree in fp64 (7 N + 5 fp64
+// instructions per warp) held a small tile's block back by microseconds.  Values near the end of
+// fp32's range, infinities and NaN take that fp64 tree.
+template <int N>
+__device__ __forceinline__ double warp_sum_pairs(const float (&v)[N]) {
+  bool plain = true;  // false for NaN
+#pragma unroll
+  for (int i = 0; i < N; ++i) plain = plain && v[i] < 1e36f;
+  if (__all_sync(0xffffffffu, plain)) {
+    float hi = v[0], lo = 0.f;
+    auto add = [&](float x, float xl) {
+      const float s = __fadd_rn(hi, x), b = __fadd_rn(s, -hi);
+      lo = __fadd_rn(__fadd_rn(lo, xl), __fadd_rn(__fadd_rn(hi, -__fadd_rn(s, -b)), __fadd_rn(x, -b)));
+      hi = s;
+    };
+#pragma unroll
+    for (int i = 1; i < N; ++i) add(v[i], 0.f);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const float oh = __shfl_xor_sync(0xffffffffu, hi, o), ol = __shfl_xor_sync(0xffffffffu, lo, o);
+      add(oh, ol);
+    }
+    return (double)hi + (double)lo;
+  }
+  double d = 0.0;
+#pragma unroll
+  for (int i = 0; i < N; ++i) d += (double)v[i];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+  return d;
+}
+
 // Deterministic block sum of one double per thread (fixed shuffle tree + fixed warp order).
 template <int THREADS>
 __device__ __forceinline__ double block_sum(double v, double *red /* >= THREADS/32 */) {

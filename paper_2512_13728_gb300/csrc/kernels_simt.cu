@@ -44,7 +44,7 @@ __device__ __forceinline__ float load_g1(const void *G, int64_t off) {
 // next rows, so that short rows leave no thread idle.  One group of each operand per thread is in
 // flight and 2048 threads per SM hide the latency (launch bounds of 8 blocks where the kernel
 // fits 32 registers): the 10 B/element norms pass of the 302M-element stack took 610 us with
-// four rows in flight per thread and 4 blocks per SM (60 registers), 463 us so; the local branch
+// four rows in flight per thread and 4 blocks per SM (60 registers), 453 us so; the local branch
 // 450 us against 575 us with four rows in flight.
 struct RowWalk {
   int c, r, cw, rp;  // first group and row of this thread, groups / rows between its next ones
@@ -136,12 +136,7 @@ __global__ void __launch_bounds__(kRowThreads, HALVES ? 5 : 8) form_b_kernel(Sha
     else form_b_tile<DT_FP32, false>(L, t.y, t.z, sb, sm);
   }
   // both sums in one fixed-order reduction (a barrier, after which all warps but the first leave)
-  double b = ((double)sb[0] + sb[1]) + ((double)sb[2] + sb[3]), mo = ((double)sm[0] + sm[1]) + ((double)sm[2] + sm[3]);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    b += __shfl_xor_sync(0xffffffffu, b, o);
-    mo += __shfl_xor_sync(0xffffffffu, mo, o);
-  }
+  const double b = warp_sum_pairs<4>(sb), mo = warp_sum_pairs<4>(sm);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (lane == 0) {
     red[warp] = b;

@@ -135,15 +135,15 @@ dion_status validate_layer(const dion_layer &ly) {
 }
 
 // Elements of a row tile (whole rows of one layer) of the buffer, norms and local kernels: 64K
-// where the plan has enough for four or more blocks per SM, fewer on smaller plans, so that they
-// still spread over the chip (down to 1K, four elements per thread).  The buffer pass of a
-// 256 x 512 matrix took 57 us in two 64K tiles and takes 8.5 us in 128 of 1K; on the 302M-element
-// stack 32K and 64K measured the same, but idle blocks (a branch no layer takes) cost 2 us per
-// thousand.
+// where the plan has 16 or more such tiles per SM (two waves of eight blocks), fewer on smaller
+// plans, so that the last wave stays a small part and small plans still spread over the chip (down
+// to 1K, four elements per thread).  The buffer pass of a 256 x 512 matrix took 57 us in two 64K
+// tiles and takes 8 us in 128 of 1K; norms and local passes of the 160M stack 170 + 170 us in 1.1
+// waves of 64K, 141 + 139 so; idle blocks (a branch no layer takes) cost 2 us per thousand.
 int64_t row_tile_elems(const dion_layer *layers, int32_t num_layers, int sms) {
   int64_t total = 0;
   for (int32_t l = 0; l < num_layers; ++l) total += layers[l].m * layers[l].n;
-  return std::min<int64_t>(65536, std::max<int64_t>(1024, total / (4 * std::max(sms, 1))));
+  return std::min<int64_t>(65536, std::max<int64_t>(1024, total / (16 * std::max(sms, 1))));
 }
 
 // The output tiles of a set of problems, those with the longest K first (the last wave then holds
@@ -275,7 +275,8 @@ dion_status dion_plan_create(const dion_layer *layers, int32_t num_layers, int32
     o_S[l] = cv.take<float>((d.s_parts - 1) * d.s_stride + ly.r * d.ldp);
     o_Li[l] = cv.take<float>(ly.r * d.ldp);
     // row tiles of the buffer, norms and local kernels
-    const int64_t rows = std::max<int64_t>(1, std::min<int64_t>(ly.m, tile_elems / ly.n));
+    int64_t rows = 1;  // a power of two (tiles of 57 rows of 1024 took 468 us where 64 took 450)
+    while (2 * rows <= std::min<int64_t>(ly.m, tile_elems / ly.n)) rows *= 2;
     d.bpart_off = (int32_t)bt.size();
     for (int64_t r0 = 0; r0 < ly.m; r0 += rows)
       bt.push_back(make_int4(l, (int)r0, (int)std::min(rows, ly.m - r0), (int)bt.size()));

@@ -329,9 +329,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(U_THREADS, 1)
       ecount += ns;
       // per-tile ||M_t||^2 (rows/columns outside the matrix hold 0), fixed reduction order;
       // the barrier also ends every thread's TMEM reads of this accumulator
-      double v = (double)ss;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      const float ss1[1] = {ss};
+      const double v = warp_sum_pairs<1>(ss1);
       if (lane == 0) red_s[warp - 2] = v;
       tc_fence_before();
       if (!named_and(1, 128, ok)) break;

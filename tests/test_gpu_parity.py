@@ -667,3 +667,27 @@ def test_fp32_large_gemm_tiles():
     other tests take the 32 x 32 one), with partial tiles."""
     w = wl.scaled(wl.WORKLOADS["gpt160m_block_r192"], "largegemm", [(1100, 1030)] * 14, rank=250, steps=1)
     run_per_step(w, PRECS["fp32"], dict(gate_mode=oc.GATE_ALWAYS), w.steps, TOL_FP32)
+
+
+@pytest.mark.parametrize("scale", [1.0, 1e17, 1e18])
+def test_norms_near_the_end_of_fp32(scale):
+    """||B|| where squares are ordinary and where a warp's sum of them nears or leaves fp32's range (the
+    fp64 branch of the norm sums): every layer local, so that nothing but the norms squares B."""
+    import paper_2512_13728_gb300 as cd
+
+    g = torch.Generator(device="cuda")
+    g.manual_seed(3)
+    M = torch.randn((600, 520), generator=g, device="cuda") * scale
+    G = torch.randn((600, 520), generator=g, device="cuda") * scale
+    want_b, want_m = float((M.double() + G.double()).norm()), float(M.double().norm())
+    X, Q = torch.zeros_like(M), torch.ones((520, 4), device="cuda")
+    plan = cd.Plan([X], [M], [Q], [G], [float("inf")], cd.DION_PREC_FP32)
+    try:
+        plan.step(cd.hparams(step=1, gate_mode=cd.DION_GATE_PER_LAYER, eta=0.0))
+        torch.cuda.synchronize()
+        got = float(plan.prev_norm[0])
+        eq1 = float(plan.rmmc_eq1[0])
+    finally:
+        plan.close()
+    assert abs(got - want_b) <= RMMC_RTOL * want_b
+    assert abs(eq1 - abs(want_b - want_m) / want_m) <= RMMC_RTOL
