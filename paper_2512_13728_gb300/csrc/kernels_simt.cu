@@ -809,7 +809,6 @@ __global__ void __launch_bounds__(kCholThreads, 1) chol_inv_kernel(Shared sh, in
   const int64_t ls = Ly.ldp;  // leading dimension of S and L^{-1} (a multiple of 8)
   const float *S = Ly.S;
   float *Li = Ly.Linv;
-  sum_gram_parts<kCholThreads>(Ly.S, r, ls, Ly.s_parts, Ly.s_stride);
   extern __shared__ __align__(16) float smem[];
   float *DI = smem;                // CB x CB
   DiagScratch &diag = *reinterpret_cast<DiagScratch *>(DI + CB * CB);
@@ -820,13 +819,16 @@ __global__ void __launch_bounds__(kCholThreads, 1) chol_inv_kernel(Shared sh, in
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
   if (pass >= 1) {
-    // ||E||_F^2 from the lower triangle (E symmetric), fixed-order reduction.  The 16-byte
-    // groups (i, j4) on or below the diagonal (4 j4 <= i) are taken in a flat order (rows 4 b ..
-    // 4 b + 3 hold b + 1 groups each), consecutive threads on consecutive groups, kFoBatch
-    // groups per thread in flight, every one of them a load (a group's columns past the
-    // diagonal are masked)
-    const int r4 = (r + 3) / 4, nb4 = r / 4;
-    const int64_t lgroups = 2ll * nb4 * (nb4 + 1) + (int64_t)(r % 4) * (nb4 + 1);
+    // One pass over the lower triangle of S adds its partial sums up (and keeps the sum in the
+    // first part for the paths below), accumulates ||E||_F^2 (E symmetric, fixed-order reduction)
+    // and writes the first-order factor, which the sweep overwrites where the bound says no.  The
+    // 16-byte groups (i, j4) on or below the diagonal (4 j4 <= i) are taken in a flat order (rows
+    // 4 b .. 4 b + 3 hold b + 1 groups each), consecutive threads on consecutive groups, kFoBatch
+    // groups per thread in flight, every one of them a load (a group's columns past the diagonal
+    // are masked).  Bound by one CTA's loads in flight: FOFIGS
+    const int r4 = (r + 3) / 4, nb4 = r / 4, parts = Ly.s_parts;
+    const int64_t lgroups = 2ll * nb4 * (nb4 + 1) + (int64_t)(r % 4) * (nb4 + 1), stride = Ly.s_stride;
+    float *S0 = Ly.S;
     double fs = 0.0;
     for (int64_t g0 = tid; g0 < lgroups; g0 += (int64_t)kCholThreads * kFoBatch) {
       float4 v[kFoBatch];
@@ -834,78 +836,64 @@ __global__ void __launch_bounds__(kCholThreads, 1) chol_inv_kernel(Shared sh, in
 #pragma unroll
       for (int u = 0; u < kFoBatch; ++u) {
         const int64_t g = g0 + (int64_t)u * kCholThreads;
-        lower_group(g, gi[u], gj[u]);
-        v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (g < lgroups) v[u] = *reinterpret_cast<const float4 *>(S + (int64_t)gi[u] * ls + 4 * gj[u]);
-        else gi[u] = -1;  // past the last group: every column masked below
+        lower_group(g < lgroups ? g : 0, gi[u], gj[u]);
+        v[u] = *reinterpret_cast<const float4 *>(S0 + (int64_t)gi[u] * ls + 4 * gj[u]);
+      }
+      for (int q = 1; q < parts; ++q) {
+        float4 w[kFoBatch];
+#pragma unroll
+        for (int u = 0; u < kFoBatch; ++u)
+          w[u] = *reinterpret_cast<const float4 *>(S0 + q * stride + (int64_t)gi[u] * ls + 4 * gj[u]);
+#pragma unroll
+        for (int u = 0; u < kFoBatch; ++u) {
+          v[u].x += w[u].x; v[u].y += w[u].y; v[u].z += w[u].z; v[u].w += w[u].w;
+        }
       }
       float a = 0.f;
 #pragma unroll
       for (int u = 0; u < kFoBatch; ++u) {
-        const int i = gi[u];
+        if (g0 + (int64_t)u * kCholThreads >= lgroups) break;
+        const int i = gi[u], j4 = gj[u];
+        if (parts > 1) *reinterpret_cast<float4 *>(S0 + (int64_t)i * ls + 4 * j4) = v[u];
         const float ve[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+        float o[4];
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-          const int j = 4 * gj[u] + c;
+          const int j = 4 * j4 + c;
           const float e = (j <= i) ? ve[c] - (i == j ? 1.f : 0.f) : 0.f;
           a = fmaf((j < i ? 2.f : 1.f) * e, e, a);
+          o[c] = (j < i) ? -ve[c] : (j == i ? 1.f - 0.5f * (ve[c] - 1.f) : 0.f);
+        }
+        float *dst = Li + (int64_t)i * ls + 4 * j4;
+        if (4 * j4 + 4 <= r) {
+          *reinterpret_cast<float4 *>(dst) = make_float4(o[0], o[1], o[2], o[3]);
+        } else {  // a group that straddles column r
+#pragma unroll
+          for (int c = 0; c < 4; ++c)
+            if (4 * j4 + c < r) dst[c] = o[c];
         }
       }
       fs += (double)a;
     }
+    for (int i = warp; i < r; i += kCholThreads / 32) {  // zeros above, a warp per row
+      for (int j4 = i / 4 + 1 + lane; j4 < r4; j4 += 32) {
+        float *dst = Li + (int64_t)i * ls + 4 * j4;
+        if (4 * j4 + 4 <= r) {
+          *reinterpret_cast<float4 *>(dst) = make_float4(0.f, 0.f, 0.f, 0.f);
+        } else {
+          for (int c = 0; 4 * j4 + c < r; ++c) dst[c] = 0.f;
+        }
+      }
+    }
     fs = block_sum<kCholThreads>(fs, red);
     __shared__ float lam_s;
     if (tid == 0) lam_s = (float)sqrt(fs);
-    __syncthreads();
+    __syncthreads();  // also: S is whole for what follows
     float lam = lam_s;
-    if (!(isfinite(lam) && 1.5f * lam < near_identity)) {
-      lam = power_norm_sym(S, r, ls, Y, ldy);
-    }
-    if (isfinite(lam) && 1.5f * lam < near_identity) {
-      // the groups on or below the diagonal in the same order, 16-byte loads and stores (a group
-      // that straddles column r is stored element-wise), then zeros above them, a warp per row
-      for (int64_t g0 = tid; g0 < lgroups; g0 += (int64_t)kCholThreads * kFoBatch) {
-        float4 v[kFoBatch];
-        int gi[kFoBatch], gj[kFoBatch];
-#pragma unroll
-        for (int u = 0; u < kFoBatch; ++u) {
-          const int64_t g = g0 + (int64_t)u * kCholThreads;
-          lower_group(g, gi[u], gj[u]);
-          v[u] = g < lgroups ? *reinterpret_cast<const float4 *>(S + (int64_t)gi[u] * ls + 4 * gj[u])
-                             : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-#pragma unroll
-        for (int u = 0; u < kFoBatch; ++u) {
-          if (g0 + (int64_t)u * kCholThreads >= lgroups) break;
-          const int i = gi[u], j4 = gj[u];
-          float o[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
-#pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            const int j = 4 * j4 + c;
-            o[c] = (j < i) ? -o[c] : (j == i ? 1.f - 0.5f * (o[c] - 1.f) : 0.f);
-          }
-          float *dst = Li + (int64_t)i * ls + 4 * j4;
-          if (4 * j4 + 4 <= r) {
-            *reinterpret_cast<float4 *>(dst) = make_float4(o[0], o[1], o[2], o[3]);
-          } else {
-#pragma unroll
-            for (int c = 0; c < 4; ++c)
-              if (4 * j4 + c < r) dst[c] = o[c];
-          }
-        }
-      }
-      for (int i = warp; i < r; i += kCholThreads / 32) {
-        for (int j4 = i / 4 + 1 + lane; j4 < r4; j4 += 32) {
-          float *dst = Li + (int64_t)i * ls + 4 * j4;
-          if (4 * j4 + 4 <= r) {
-            *reinterpret_cast<float4 *>(dst) = make_float4(0.f, 0.f, 0.f, 0.f);
-          } else {
-            for (int c = 0; 4 * j4 + c < r; ++c) dst[c] = 0.f;
-          }
-        }
-      }
-      return;
-    }
+    if (!(isfinite(lam) && 1.5f * lam < near_identity)) lam = power_norm_sym(S, r, ls, Y, ldy);
+    if (isfinite(lam) && 1.5f * lam < near_identity) return;
+  } else {
+    sum_gram_parts<kCholThreads>(Ly.S, r, ls, Ly.s_parts, Ly.s_stride);
   }
   // Y: zero the columns past r once (the update's tiles read up to the next multiple of 8)
   for (int e = tid; e < CB * ldy; e += kCholThreads)
