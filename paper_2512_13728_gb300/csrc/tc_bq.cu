@@ -280,40 +280,44 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(R_THREADS, 1)
     }
   } else if (warp == 1) {
     if (lane == 0 && rank == 0) {
-      uint32_t it = 0, tcount = 0;
+      uint32_t tcount = 0;
+      RingPos rp;
       bool ok = true;
+      // A: K-major (B Q) advances 32 bytes per 16 k; MN-major (B^T P) two 8-row groups
+      constexpr uint32_t A_K16 = (KIND == GEMM_BQ) ? 32u : 2048u;
+      const uint64_t ad0 = smem_desc_sw128(smem_u32(smem), (KIND == GEMM_BQ) ? 0u : BOX64, 1024);
+      const uint64_t bd0 = smem_desc_sw128(smem_u32(smem) + A_BYTES, BOX64, 1024);
       for (int ti = off[seg]; ti < off[seg + 1] && ok; ++ti) {
         const int4 t = tiles[ti];
         if (!sh.active[t.x]) continue;
         const DevLayer &L = sh.layers[t.x];
         const int kch = (int)(((KIND == GEMM_BQ ? L.n : L.m) + 63) / 64);
         const uint32_t np = rpad16(L.r), nparts = (np + 255) / 256;
+        const uint32_t id0 = idesc_bf16(256, 2u * half_cols(np, 0), KIND == GEMM_BTP, true);
+        const uint32_t id1 = nparts > 1u ? idesc_bf16(256, 2u * half_cols(np, 1), KIND == GEMM_BTP, true) : 0u;
         if (!ab.wait(acc_empty, (tcount & 1u) ^ 1u, sh.status)) break;
         tc_fence_after();
-        for (int kc = 0; kc < kch; ++kc, ++it) {
-          const uint32_t s = it % nstages, ph = (it / nstages) & 1u;
-          if (!ab.wait(&full[s], ph, sh.status)) { ok = false; break; }
+        for (int kc = 0; kc < kch; ++kc) {
+          if (!ab.wait(&full[rp.s], rp.ph, sh.status)) { ok = false; break; }
           tc_fence_after();
-          const uint32_t aB = smem_u32(smem + s * stage_bytes), bB = aB + A_BYTES;
+          const uint64_t ads = desc_at(ad0, rp.s * stage_bytes), bds = desc_at(bd0, rp.s * stage_bytes);
 #pragma unroll
           for (int k16 = 0; k16 < 4; ++k16) {
-            // A: K-major (B Q) advances 32 bytes per 16 k; MN-major (B^T P) two 8-row groups
-            const uint32_t ak = (KIND == GEMM_BQ) ? (uint32_t)k16 * 32u : (uint32_t)k16 * 2048u;
-            const uint32_t albo = (KIND == GEMM_BQ) ? 0u : BOX64;
-            const uint64_t ad = smem_desc_sw128(aB + ak, albo, 1024);
-            for (uint32_t part = 0; part < nparts; ++part) {
-              const uint32_t n_here = 2u * half_cols(np, part);
-              const uint32_t idesc = idesc_bf16(256, n_here, KIND == GEMM_BTP, true);
-              const uint32_t bo = part * 2u * BOX64 + k16 * 2048;
-              const uint64_t bd = smem_desc_sw128(bB + bo, BOX64, 1024);
-              umma_pair_bf16(tmem + part * 256u, ad, bd, idesc, (kc | k16) ? 1u : 0u);
+            const uint64_t ad = desc_at(ads, k16 * A_K16);
+#pragma unroll
+            for (uint32_t part = 0; part < 2u; ++part) {
+              if (part >= nparts) break;
+              const uint32_t idesc = part ? id1 : id0, d = tmem + part * 256u;
+              const uint64_t bd = desc_at(bds, part * 2u * BOX64 + k16 * 2048u);
+              umma_pair_bf16(d, ad, bd, idesc, (kc | k16) ? 1u : 0u);
               if (X3) {
-                umma_pair_bf16(tmem + part * 256u, ad, smem_desc_sw128(bB + b_half + bo, BOX64, 1024), idesc, 1u);
-                umma_pair_bf16(tmem + part * 256u, smem_desc_sw128(aB + OPB_A + ak, albo, 1024), bd, idesc, 1u);
+                umma_pair_bf16(d, ad, desc_at(bd, b_half), idesc, 1u);
+                umma_pair_bf16(d, desc_at(ad, OPB_A), bd, idesc, 1u);
               }
             }
           }
-          umma_pair_commit_mc(&empty[s], 0x3);  // the stage is free in both CTAs
+          umma_pair_commit_mc(&empty[rp.s], 0x3);  // the stage is free in both CTAs
+          rp.next(nstages);
         }
         if (!ok) break;
         umma_pair_commit_mc(acc_full, 0x3);
@@ -561,33 +565,38 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(FB_THREADS, 1)
     }
   } else if (warp == 1) {  // MMA issue (CTA 0)
     if (lane == 0 && rank == 0) {
-      uint32_t it = 0, tcount = 0;
+      uint32_t tcount = 0;
+      RingPos ra, rq;
       bool ok = true;
+      const uint64_t ad0 = smem_desc_sw128(smem_u32(aring), 0, 1024);
+      const uint64_t bd0 = smem_desc_sw128(smem_u32(qring), BOX64, 1024);
       for (int ti = off[seg]; ti < off[seg + 1] && ok; ++ti) {
         const int4 t = tiles[ti];
         if (gated && !sh.active[t.x]) continue;
         const DevLayer &L = sh.layers[t.x];
         const int kch = (int)((L.n + 63) / 64);
         const uint32_t np = rpad16(L.r), nparts = (np + 255) / 256;
+        const uint32_t id0 = idesc_bf16(256, 2u * half_cols(np, 0), false, true);
+        const uint32_t id1 = nparts > 1u ? idesc_bf16(256, 2u * half_cols(np, 1), false, true) : 0u;
         if (!ab.wait(acc_empty, (tcount & 1u) ^ 1u, sh.status)) break;
         tc_fence_after();
-        for (int kc = 0; kc < kch; ++kc, ++it) {
-          const uint32_t sg = it % FB_ASTAGES, pg = (it / FB_ASTAGES) & 1u;
-          const uint32_t q = it % nq, qph = (it / nq) & 1u;
-          if (!ab.wait(&qfull[q], qph, sh.status) || !ab.wait(&afull[sg], pg, sh.status)) { ok = false; break; }
+        for (int kc = 0; kc < kch; ++kc) {
+          if (!ab.wait(&qfull[rq.s], rq.ph, sh.status) || !ab.wait(&afull[ra.s], ra.ph, sh.status)) { ok = false; break; }
           tc_fence_after();
-          const uint32_t aB = smem_u32(aring + sg * FB_GBOX), bB = smem_u32(qring + q * qstage_bytes);
+          const uint64_t ads = desc_at(ad0, ra.s * FB_GBOX), bds = desc_at(bd0, rq.s * qstage_bytes);
 #pragma unroll
           for (int k16 = 0; k16 < 4; ++k16) {
-            const uint64_t ad = smem_desc_sw128(aB + k16 * 32, 0, 1024);
-            for (uint32_t part = 0; part < nparts; ++part) {
-              const uint32_t n_here = 2u * half_cols(np, part);
-              const uint64_t bd = smem_desc_sw128(bB + part * 2u * BOX64 + k16 * 2048, BOX64, 1024);
-              umma_pair_bf16(tmem + part * 256u, ad, bd, idesc_bf16(256, n_here, false, true), (kc | k16) ? 1u : 0u);
+#pragma unroll
+            for (uint32_t part = 0; part < 2u; ++part) {
+              if (part >= nparts) break;
+              umma_pair_bf16(tmem + part * 256u, desc_at(ads, k16 * 32u), desc_at(bds, part * 2u * BOX64 + k16 * 2048u),
+                             part ? id1 : id0, (kc | k16) ? 1u : 0u);
             }
           }
-          umma_pair_commit_mc(&gempty[sg], 0x3);
-          umma_pair_commit_mc(&qempty[q], 0x3);
+          umma_pair_commit_mc(&gempty[ra.s], 0x3);
+          umma_pair_commit_mc(&qempty[rq.s], 0x3);
+          ra.next(FB_ASTAGES);
+          rq.next(nq);
         }
         if (!ok) break;
         umma_pair_commit_mc(acc_full, 0x3);

@@ -230,6 +230,24 @@ __device__ __forceinline__ uint64_t smem_desc_sw64(uint32_t saddr, uint32_t sbo)
   return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | (1ull << 46) |
          (4ull << 61);
 }
+// The same operand `bytes` (a multiple of 16) further on: the address field is the low 14 bits, in
+// units of 16 bytes.  The MMA issuers build one descriptor per stage and step it with constants:
+// building both descriptors and the instruction descriptor for every MMA, and dividing by the ring
+// depth for every stage, cost the issuing thread 1230 cycles per 64-wide chunk of B^T P (170 per
+// MMA), more than the chunk's loads.
+__device__ __forceinline__ uint64_t desc_at(uint64_t desc, uint32_t bytes) { return desc + (bytes >> 4); }
+
+// A ring's stage index and the parity of its current use, stepped without divisions.
+struct RingPos {
+  uint32_t s = 0, ph = 0;
+  __device__ __forceinline__ void next(uint32_t n) {
+    if (++s == n) {
+      s = 0;
+      ph ^= 1u;
+    }
+  }
+};
+
 // Instruction descriptor of kind::f16 with bf16 A and B, fp32 D; a_mn / b_mn select
 // MN-major operands.  M = 128, N a multiple of 16 in [16, 256].
 __host__ __device__ constexpr uint32_t idesc_bf16(uint32_t M, uint32_t N, bool a_mn, bool b_mn) {

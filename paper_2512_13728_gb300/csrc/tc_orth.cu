@@ -307,8 +307,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(X3 ? O_THREADS_X3 : 
     }
   } else if (warp == 1) {
     if (lane == 0 && rank == 0) {
-      uint32_t it = 0, tcount = 0;
+      uint32_t tcount = 0;
+      RingPos rp;
       bool ok = true;
+      uint64_t *const ready = X3 ? conv : full;
+      const uint64_t sd0 = smem_desc_sw128(smem_u32(smem), 0, 1024);  // the A box; the B boxes follow
       for (int ti = off[seg]; ti < off[seg + 1] && ok; ++ti) {
         const int4 t = tiles[ti];
         if (skip(t.x)) continue;
@@ -324,22 +327,22 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(X3 ? O_THREADS_X3 : 
             if (!ab.wait(&acc_empty[slot], ((tcount >> 1) & 1u) ^ 1u, sh.status)) { ok = false; break; }
             tc_fence_after();
             const int kq = min(kch, (int)(8u * (q + 1u)));
-            const uint32_t idesc = idesc_tf32(256, 2u * half_rows(N, q), false, false);
-            for (int kc = 0; kc < kq; ++kc, ++it) {
-              const uint32_t s = it % nstages, ph = (it / nstages) & 1u;
-              if (!ab.wait(X3 ? &conv[s] : &full[s], ph, sh.status)) { ok = false; break; }
+            const uint32_t idesc = idesc_tf32(256, 2u * half_rows(N, q), false, false), d = tmem + slot * 256u;
+            for (int kc = 0; kc < kq; ++kc) {
+              if (!ab.wait(&ready[rp.s], rp.ph, sh.status)) { ok = false; break; }
               tc_fence_after();
-              const uint32_t aB = smem_u32(smem + s * stage_bytes), bB = aB + O_BOX;
+              const uint64_t as = desc_at(sd0, rp.s * stage_bytes);
 #pragma unroll
               for (int k8 = 0; k8 < 4; ++k8) {
-                const uint64_t ad = smem_desc_sw128(aB + k8 * 32, 0, 1024), bd = smem_desc_sw128(bB + k8 * 32, 0, 1024);
-                umma_pair_tf32(tmem + slot * 256u, ad, bd, idesc, (kc | k8) ? 1u : 0u);
+                const uint64_t ad = desc_at(as, k8 * 32u), bd = desc_at(as, O_BOX + k8 * 32u);
+                umma_pair_tf32(d, ad, bd, idesc, (kc | k8) ? 1u : 0u);
                 if (X3) {  // hi.lo + lo.hi
-                  umma_pair_tf32(tmem + slot * 256u, ad, smem_desc_sw128(bB + lo_off + k8 * 32, 0, 1024), idesc, 1u);
-                  umma_pair_tf32(tmem + slot * 256u, smem_desc_sw128(aB + lo_off + k8 * 32, 0, 1024), bd, idesc, 1u);
+                  umma_pair_tf32(d, ad, desc_at(bd, lo_off), idesc, 1u);
+                  umma_pair_tf32(d, desc_at(ad, lo_off), bd, idesc, 1u);
                 }
               }
-              umma_pair_commit_mc(&empty[s], 0x3);  // the stage is free in both CTAs
+              umma_pair_commit_mc(&empty[rp.s], 0x3);  // the stage is free in both CTAs
+              rp.next(nstages);
             }
             if (!ok) break;
             umma_pair_commit_mc(&acc_full[slot], 0x3);
@@ -353,29 +356,30 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(X3 ? O_THREADS_X3 : 
         if (!ab.wait(&acc_empty[slot], aph ^ 1u, sh.status)) break;
         tc_fence_after();
         const uint32_t d0 = tmem + slot * 256u;
-        for (int kc = 0; kc < t.w; ++kc, ++it) {
-          const uint32_t s = it % nstages, ph = (it / nstages) & 1u;
-          if (!ab.wait(X3 ? &conv[s] : &full[s], ph, sh.status)) { ok = false; break; }
+        // per part: its instruction and its A box (in place in a B box, or the stage's own)
+        const uint32_t id[2] = {idesc_tf32(256, g.N[0], false, false), idesc_tf32(256, max(g.N[1], 16u), false, false)};
+        const uint32_t ao[2] = {g.a_box[0] >= 0 ? (uint32_t)(1 + g.a_box[0]) * O_BOX : 0u,
+                                g.a_box[1] >= 0 ? (uint32_t)(1 + g.a_box[1]) * O_BOX : 0u};
+        for (int kc = 0; kc < t.w; ++kc) {
+          if (!ab.wait(&ready[rp.s], rp.ph, sh.status)) { ok = false; break; }
           tc_fence_after();
-          const uint32_t aB = smem_u32(smem + s * stage_bytes), bB = aB + O_BOX;
+          const uint64_t as = desc_at(sd0, rp.s * stage_bytes);
 #pragma unroll
           for (int k8 = 0; k8 < 4; ++k8) {
 #pragma unroll
             for (uint32_t q = 0; q < 2u; ++q) {
               if (q >= g.nparts) break;
-              const uint32_t aSrc = g.a_box[q] >= 0 ? bB + (uint32_t)g.a_box[q] * O_BOX : aB;
-              const uint64_t ad = smem_desc_sw128(aSrc + k8 * 32, 0, 1024);
-              const uint32_t idesc = idesc_tf32(256, g.N[q], false, false);
-              const uint64_t bd = smem_desc_sw128(bB + q * O_BOX + k8 * 32, 0, 1024);
+              const uint64_t ad = desc_at(as, ao[q] + k8 * 32u), bd = desc_at(as, (1u + q) * O_BOX + k8 * 32u);
               // the first chunk that feeds a part starts its accumulation
-              umma_pair_tf32(d0 + q * 256u, ad, bd, idesc, (kc | k8) ? 1u : 0u);
+              umma_pair_tf32(d0 + q * 256u, ad, bd, id[q], (kc | k8) ? 1u : 0u);
               if (X3) {  // hi.lo + lo.hi
-                umma_pair_tf32(d0 + q * 256u, ad, smem_desc_sw128(bB + lo_off + q * O_BOX + k8 * 32, 0, 1024), idesc, 1u);
-                umma_pair_tf32(d0 + q * 256u, smem_desc_sw128(aSrc + lo_off + k8 * 32, 0, 1024), bd, idesc, 1u);
+                umma_pair_tf32(d0 + q * 256u, ad, desc_at(bd, lo_off), id[q], 1u);
+                umma_pair_tf32(d0 + q * 256u, desc_at(ad, lo_off), bd, id[q], 1u);
               }
             }
           }
-          umma_pair_commit_mc(&empty[s], 0x3);  // the stage is free in both CTAs
+          umma_pair_commit_mc(&empty[rp.s], 0x3);  // the stage is free in both CTAs
+          rp.next(nstages);
         }
         if (!ok) break;
         umma_pair_commit_mc(&acc_full[slot], 0x3);

@@ -166,6 +166,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(U_THREADS, 1)
     if (lane == 0 && rank == 0) {
       uint32_t it = 0, tcount = 0;
       bool ok = true;
+      const uint64_t sd0 = X3 ? smem_desc_sw64(smem_u32(stage), 512) : smem_desc_sw128(smem_u32(stage), 0, 1024);
       for (int ti = off[seg]; ti < off[seg + 1] && ok; ++ti) {
         const int4 t = tiles[ti];
         if (!sh.active[t.x]) continue;
@@ -178,12 +179,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(U_THREADS, 1)
           const uint32_t s = it % U_STAGES, ph = (it / U_STAGES) & 1u;
           if (!ab.wait(&full[s], ph, sh.status)) { ok = false; break; }
           tc_fence_after();
-          const uint32_t base = smem_u32(stage + s * U_STAGE);
+          const uint64_t sd = desc_at(sd0, s * U_STAGE);
           // K-major operand box at offset o of the stage, advanced by k16 steps of 16 elements (32 bytes)
-          auto desc = [&](uint32_t o, int k16) {
-            const uint32_t a = base + o + (uint32_t)k16 * 32u;
-            return X3 ? smem_desc_sw64(a, 512) : smem_desc_sw128(a, 0, 1024);
-          };
+          auto desc = [&](uint32_t o, int k16) { return desc_at(sd, o + (uint32_t)k16 * 32u); };
 #pragma unroll
           for (int k16 = 0; k16 < (int)(KW / 16u); ++k16) {
             const uint64_t ad = desc(0, k16), rd = desc(PB, k16), qd = desc(PB + BB, k16);
