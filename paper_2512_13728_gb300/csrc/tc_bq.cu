@@ -193,7 +193,8 @@ enum : int { GEMM_BQ = 0, GEMM_BTP = 1 };
 template <int KIND, bool X3>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(R_THREADS, 1)
     tc_tma_gemm_kernel(Shared sh, const int4 *__restrict__ tiles, const int *__restrict__ off,
-                       const LayerMaps *__restrict__ maps, int nstages, uint32_t stage_bytes, uint32_t tmem_cols) {
+                       const LayerMaps *__restrict__ maps, int nstages, uint32_t stage_bytes, uint32_t tmem_cols,
+                       uint32_t slots) {
   chain_enter();
   if (sh.gate_scratch[kScratchActive] == 0ull) return;  // no layer takes the Dion branch
   extern __shared__ uint8_t smem_raw[];
@@ -203,7 +204,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(R_THREADS, 1)
   constexpr uint32_t A_BYTES = (X3 ? 2u : 1u) * OPB_A;  // the A halves of a stage
   const uint32_t b_half = X3 ? (stage_bytes - A_BYTES) / 2u : 0u;  // offset of the B low boxes
   uint64_t *full = bars, *empty = bars + nstages;
-  uint64_t *acc_full = bars + 2 * nstages, *acc_empty = acc_full + 1, *drain = acc_full + 2;
+  uint64_t *acc_full = bars + 2 * nstages, *acc_empty = acc_full + 2, *drain = acc_full + 4;
   __shared__ uint32_t tmem_base_s;
   __shared__ int abort_s;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -215,8 +216,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(R_THREADS, 1)
       mbar_init(&full[i], 1);   // used in CTA 0: its arm, both CTAs' bytes
       mbar_init(&empty[i], 1);  // pair commit after the stage's MMAs
     }
-    mbar_init(acc_full, 1);   // pair commit after the tile's MMAs
-    mbar_init(acc_empty, 2);  // used in CTA 0: one arrival per CTA's epilogue
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&acc_full[i], 1);   // pair commit after the tile's MMAs
+      mbar_init(&acc_empty[i], 2);  // used in CTA 0: one arrival per CTA's epilogue
+    }
     mbar_init(drain, 1);
     abort_s = 0;
     fence_mbar_init();
@@ -280,8 +283,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(R_THREADS, 1)
     }
   } else if (warp == 1) {
     if (lane == 0 && rank == 0) {
-      uint32_t tcount = 0;
-      RingPos rp;
+      RingPos rp, acc;
       bool ok = true;
       // A: K-major (B Q) advances 32 bytes per 16 k; MN-major (B^T P) two 8-row groups
       constexpr uint32_t A_K16 = (KIND == GEMM_BQ) ? 32u : 2048u;
@@ -295,7 +297,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(R_THREADS, 1)
         const uint32_t np = rpad16(L.r), nparts = (np + 255) / 256;
         const uint32_t id0 = idesc_bf16(256, 2u * half_cols(np, 0), KIND == GEMM_BTP, true);
         const uint32_t id1 = nparts > 1u ? idesc_bf16(256, 2u * half_cols(np, 1), KIND == GEMM_BTP, true) : 0u;
-        if (!ab.wait(acc_empty, (tcount & 1u) ^ 1u, sh.status)) break;
+        const uint32_t slot = acc.s;
+        if (!ab.wait(&acc_empty[slot], acc.ph ^ 1u, sh.status)) break;
         tc_fence_after();
         for (int kc = 0; kc < kch; ++kc) {
           if (!ab.wait(&full[rp.s], rp.ph, sh.status)) { ok = false; break; }
@@ -307,7 +310,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(R_THREADS, 1)
 #pragma unroll
             for (uint32_t part = 0; part < 2u; ++part) {
               if (part >= nparts) break;
-              const uint32_t idesc = part ? id1 : id0, d = tmem + part * 256u;
+              const uint32_t idesc = part ? id1 : id0, d = tmem + (slot + part) * 256u;
               const uint64_t bd = desc_at(bds, part * 2u * BOX64 + k16 * 2048u);
               umma_pair_bf16(d, ad, bd, idesc, (kc | k16) ? 1u : 0u);
               if (X3) {
@@ -320,33 +323,34 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(R_THREADS, 1)
           rp.next(nstages);
         }
         if (!ok) break;
-        umma_pair_commit_mc(acc_full, 0x3);
-        ++tcount;
+        umma_pair_commit_mc(&acc_full[slot], 0x3);
+        acc.next(slots);
       }
       umma_pair_commit(drain);  // every MMA of the pair has completed before TMEM is freed
       mbar_wait(drain, 0, sh.status);
     }
   } else {
     const bool leader = (warp == 2 && lane == 0);
-    uint32_t tcount = 0, ecount = 0;
+    uint32_t ecount = 0;
+    RingPos acc;
     for (int ti = off[seg]; ti < off[seg + 1]; ++ti) {
       const int4 t = tiles[ti];
       if (!sh.active[t.x]) continue;
       const DevLayer &L = sh.layers[t.x];
       const int tr = 2 * t.y + (int)rank;
-      if (!named_and(1, 128, ab.wait(acc_full, tcount & 1u, sh.status))) break;
+      if (!named_and(1, 128, ab.wait(&acc_full[acc.s], acc.ph, sh.status))) break;
       tc_fence_after();
       if ((int64_t)tr * 128 < (KIND == GEMM_BQ ? L.m : L.n)) {  // not the pair's empty second tile
         if (KIND == GEMM_BQ)
-          store_accumulator(tmem, warp, lane, leader, stg, &maps[t.x].Praw, &maps[t.x].PTraw_t, L.r, L.m, tr * 128,
+          store_accumulator(tmem + acc.s * 256u, warp, lane, leader, stg, &maps[t.x].Praw, &maps[t.x].PTraw_t, L.r, L.m, tr * 128,
                             ecount, 1, 0, 1);
         else
-          store_r_tile<X3>(tmem, warp, lane, leader, stg, maps[t.x], L, tr, ecount);
+          store_r_tile<X3>(tmem + acc.s * 256u, warp, lane, leader, stg, maps[t.x], L, tr, ecount);
       }
       tc_fence_before();
       named_sync(1, 128);  // every thread's TMEM reads of this accumulator are done
-      if (leader) mbar_arrive_cluster(cluster_addr(acc_empty, 0));
-      ++tcount;
+      if (leader) mbar_arrive_cluster(cluster_addr(&acc_empty[acc.s], 0));
+      acc.next(slots);
     }
     if (leader) bulk_wait<0>();
   }
@@ -766,16 +770,22 @@ void launch_fused_bq(const Shared &sh, const TcPlan &tp, bool gated, cudaStream_
       gated ? 1 : 0);
 }
 
+// Two accumulator slots where a tile needs at most 256 columns: the next tile's MMAs run under the
+// epilogue's stores (B^T P, one / two: 71 / 66 us on the 160M stack at rank 192, 410 / 373 us on the 350M stack with
+// split operands).
+static uint32_t gemm_slots(const TcPlan &tp) { return tp.max_r <= 256 ? 2u : 1u; }
+static uint32_t gemm_cols(const TcPlan &tp) { return tp.max_r <= 256 ? 512u : tp.tmem_cols; }
+
 void launch_form_bq(const Shared &sh, const TcPlan &tp, cudaStream_t s) {
   if (tp.d_bq.grid <= 0) return;
   const bool x3 = tp.precision == DION_PREC_BF16X3;
   const uint32_t stage = (x3 ? 2u : 1u) * (OPB_A + tp.bq_boxes * BOX64);
   if (x3)
     launch_chained(tc_tma_gemm_kernel<GEMM_BQ, true>, 2 * tp.d_bq.grid, R_THREADS, tp.f_smem, s, 
-        sh, tp.d_bq.tiles, tp.d_bq.off, tp.maps, tp.f_stages, stage, tp.tmem_cols);
+        sh, tp.d_bq.tiles, tp.d_bq.off, tp.maps, tp.f_stages, stage, gemm_cols(tp), gemm_slots(tp));
   else
     launch_chained(tc_tma_gemm_kernel<GEMM_BQ, false>, 2 * tp.d_bq.grid, R_THREADS, tp.f_smem, s, 
-        sh, tp.d_bq.tiles, tp.d_bq.off, tp.maps, tp.f_stages, stage, tp.tmem_cols);
+        sh, tp.d_bq.tiles, tp.d_bq.off, tp.maps, tp.f_stages, stage, gemm_cols(tp), gemm_slots(tp));
 }
 
 void launch_btp(const Shared &sh, const TcPlan &tp, cudaStream_t s) {
@@ -784,10 +794,10 @@ void launch_btp(const Shared &sh, const TcPlan &tp, cudaStream_t s) {
   const uint32_t stage = (x3 ? 2u : 1u) * (OPB_A + tp.bq_boxes * BOX64);
   if (x3)
     launch_chained(tc_tma_gemm_kernel<GEMM_BTP, true>, 2 * tp.d_btp.grid, R_THREADS, tp.r_smem, s, 
-        sh, tp.d_btp.tiles, tp.d_btp.off, tp.maps, tp.r_stages, stage, tp.tmem_cols);
+        sh, tp.d_btp.tiles, tp.d_btp.off, tp.maps, tp.r_stages, stage, gemm_cols(tp), gemm_slots(tp));
   else
     launch_chained(tc_tma_gemm_kernel<GEMM_BTP, false>, 2 * tp.d_btp.grid, R_THREADS, tp.r_smem, s, 
-        sh, tp.d_btp.tiles, tp.d_btp.off, tp.maps, tp.r_stages, stage, tp.tmem_cols);
+        sh, tp.d_btp.tiles, tp.d_btp.off, tp.maps, tp.r_stages, stage, gemm_cols(tp), gemm_slots(tp));
 }
 
 // Data-parallel phases.  P_raw^T (r x m, the first Gram's operand) from the averaged P_raw:
