@@ -238,47 +238,58 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(R_THREADS, 1)
 
   if (warp == 0) {
     if (lane == 0) {
-      uint32_t it = 0;
+      uint32_t issued = 0;
+      RingPos rp;
       bool ok = true;
+      const uint32_t fb0 = cluster_addr(full, 0);
       for (int ti = off[seg]; ti < off[seg + 1] && ok; ++ti) {
         const int4 t = tiles[ti];
         if (!sh.active[t.x]) continue;
         const DevLayer &L = sh.layers[t.x];
         const LayerMaps *mp = maps + t.x;
         const int kch = (int)(((KIND == GEMM_BQ ? L.n : L.m) + 63) / 64);
-        const int tr = 2 * t.y + (int)rank;  // past the last tile: zero-filled, not stored
+        const int row = (2 * t.y + (int)rank) * 128;  // past the last tile: zero-filled, not stored
+        // this CTA's B boxes of a k-chunk: up to two 64-column boxes from x0[part]
         const uint32_t np = rpad16(L.r), nparts = (np + 255) / 256;
-        uint32_t nbox = 0;  // 64-column B boxes per CTA and k-chunk
-        for (uint32_t part = 0; part < nparts; ++part) nbox += (half_cols(np, part) + 63) / 64;
-        for (int kc = 0; kc < kch; ++kc, ++it) {
-          const uint32_t s = it % nstages, ph = (it / nstages) & 1u;
-          if (!ab.wait(&empty[s], ph ^ 1u, sh.status)) { ok = false; break; }
-          uint8_t *sA = smem + s * stage_bytes, *sB = sA + A_BYTES;
-          const uint32_t fb = cluster_addr(&full[s], 0);
-          if (rank == 0) mbar_expect_tx(&full[s], 2u * (X3 ? 2u : 1u) * (OPB_A + nbox * BOX64));
+        int x0[2] = {0, 0}, nb[2] = {0, 0};
+#pragma unroll
+        for (uint32_t part = 0; part < 2u; ++part) {
+          if (part >= nparts) break;
+          const uint32_t hc = half_cols(np, part);
+          x0[part] = (int)(part * 256u + rank * hc);
+          nb[part] = (int)((hc + 63) / 64);
+        }
+        const uint32_t bytes = 2u * (X3 ? 2u : 1u) * (OPB_A + (uint32_t)(nb[0] + nb[1]) * BOX64);
+        for (int kc = 0; kc < kch; ++kc, ++issued) {
+          if (!ab.wait(&empty[rp.s], rp.ph ^ 1u, sh.status)) { ok = false; break; }
+          uint8_t *sA = smem + rp.s * stage_bytes, *sB = sA + A_BYTES;
+          const uint32_t fb = fb0 + rp.s * 8u;  // this stage's barrier in CTA 0
+          if (rank == 0) mbar_expect_tx(&full[rp.s], bytes);
+#pragma unroll
           for (int hl = 0; hl < (X3 ? 2 : 1); ++hl) {  // high half, then (BF16X3) low half
             uint8_t *a = sA + hl * OPB_A;
             if (KIND == GEMM_BQ) {
-              tma_load_2d_pair(a, hl ? &mp->Bl_k : &mp->Bh_k, fb, kc * 64, tr * 128);
+              tma_load_2d_pair(a, hl ? &mp->Bl_k : &mp->Bh_k, fb, kc * 64, row);
             } else {
               const CUtensorMap *am = hl ? &mp->Bl_mn : &mp->Bh_mn;
-              tma_load_2d_pair(a, am, fb, tr * 128, kc * 64);
-              tma_load_2d_pair(a + BOX64, am, fb, tr * 128 + 64, kc * 64);
+              tma_load_2d_pair(a, am, fb, row, kc * 64);
+              tma_load_2d_pair(a + BOX64, am, fb, row + 64, kc * 64);
             }
             const CUtensorMap *bmap = (KIND == GEMM_BQ) ? (hl ? &mp->Qn_lo_mn : &mp->Qn_mn)
                                                         : (hl ? &mp->P_lo_mn : &mp->P_mn);
-            uint8_t *b = sB + hl * b_half;
-            for (uint32_t part = 0; part < nparts; ++part) {
-              const uint32_t hc = half_cols(np, part);
-              const int x0 = (int)(part * 256u + rank * hc);
-              for (uint32_t j = 0; j < (hc + 63) / 64; ++j)
-                tma_load_2d_pair(b + (part * 2u + j) * BOX64, bmap, fb, x0 + (int)j * 64, kc * 64);
-            }
+            uint8_t *bp = sB + hl * b_half;
+#pragma unroll
+            for (int part = 0; part < 2; ++part)
+#pragma unroll
+              for (int j = 0; j < 2; ++j)
+                if (j < nb[part])
+                  tma_load_2d_pair(bp + (part * 2 + j) * BOX64, bmap, fb, x0[part] + j * 64, kc * 64);
           }
+          rp.next(nstages);
         }
       }
       // drain: the last stages' loads have landed and been consumed (their stage was freed)
-      for (uint32_t k = (it > (uint32_t)nstages ? it - nstages : 0); k < it; ++k)
+      for (uint32_t k = (issued > (uint32_t)nstages ? issued - nstages : 0); k < issued; ++k)
         mbar_wait(&empty[k % nstages], (k / nstages) & 1u, sh.status);
     }
   } else if (warp == 1) {

@@ -198,7 +198,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(X3 ? O_THREADS_X3 : 
 
   if (warp == 0) {
     if (lane == 0) {
-      uint32_t it = 0;
+      uint32_t issued = 0;
+      RingPos rp;
       bool ok = true;
       for (int ti = off[seg]; ti < off[seg + 1] && ok; ++ti) {
         const int4 t = tiles[ti];
@@ -214,32 +215,35 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(X3 ? O_THREADS_X3 : 
         if constexpr (KIND == ORTH_TRSM) {
           // sub-tile q: K chunks below 256 (q + 1); A chunk and part q's B box in each stage
           for (uint32_t q = 0; q < nparts && ok; ++q) {
-            const int kq = min(kch, (int)(8u * (q + 1u)));
-            for (int kc = 0; kc < kq; ++kc, ++it) {
-              const uint32_t s = it % nstages, ph = (it / nstages) & 1u;
-              if (!ab.wait(&empty[s], ph ^ 1u, sh.status)) { ok = false; break; }
-              uint8_t *sA = smem + s * stage_bytes, *sB = sA + O_BOX;
-              expect(s, 2u);
-              load(sA, om.A, s, kc * 32, tr * 128);
-              load(sB, om.B, s, kc * 32, (int)(q * 256u + rank * half_rows(N, q)));
+            const int kq = min(kch, (int)(8u * (q + 1u))), brow = (int)(q * 256u + rank * half_rows(N, q));
+            for (int kc = 0; kc < kq; ++kc, ++issued) {
+              if (!ab.wait(&empty[rp.s], rp.ph ^ 1u, sh.status)) { ok = false; break; }
+              uint8_t *sA = smem + rp.s * stage_bytes, *sB = sA + O_BOX;
+              expect(rp.s, 2u);
+              load(sA, om.A, rp.s, kc * 32, tr * 128);
+              load(sB, om.B, rp.s, kc * 32, brow);
+              rp.next(nstages);
             }
           }
           continue;
         }
         const GramTile g = gram_tile(L.r, t.y & 0xff);
-        for (int kc = t.z; kc < t.z + t.w; ++kc, ++it) {
-          const uint32_t s = it % nstages, ph = (it / nstages) & 1u;
-          if (!ab.wait(&empty[s], ph ^ 1u, sh.status)) { ok = false; break; }
-          uint8_t *sA = smem + s * stage_bytes, *sB = sA + O_BOX;
-          expect(s, (g.sep_a ? 1u : 0u) + g.nparts);
-          if (g.sep_a) load(sA, om.A, s, kc * 32, g.a_row + (int)rank * 128);
+        const int arow = g.a_row + (int)rank * 128;
+        const int brow[2] = {(int)(g.b_row[0] + rank * (g.N[0] / 2u)), (int)(g.b_row[1] + rank * (g.N[1] / 2u))};
+        const uint32_t boxes = (g.sep_a ? 1u : 0u) + g.nparts;
+        for (int kc = t.z; kc < t.z + t.w; ++kc, ++issued) {
+          if (!ab.wait(&empty[rp.s], rp.ph ^ 1u, sh.status)) { ok = false; break; }
+          uint8_t *sA = smem + rp.s * stage_bytes, *sB = sA + O_BOX;
+          expect(rp.s, boxes);
+          if (g.sep_a) load(sA, om.A, rp.s, kc * 32, arow);
 #pragma unroll
           for (uint32_t q = 0; q < 2u; ++q)
-            if (q < g.nparts) load(sB + q * O_BOX, om.B, s, kc * 32, (int)(g.b_row[q] + rank * (g.N[q] / 2u)));
+            if (q < g.nparts) load(sB + q * O_BOX, om.B, rp.s, kc * 32, brow[q]);
+          rp.next(nstages);
         }
       }
       // drain: the last stages' loads have landed and been consumed (their stage was freed)
-      for (uint32_t k = (it > (uint32_t)nstages ? it - nstages : 0); k < it; ++k)
+      for (uint32_t k = (issued > (uint32_t)nstages ? issued - nstages : 0); k < issued; ++k)
         mbar_wait(&empty[k % nstages], (k / nstages) & 1u, sh.status);
     }
   } else if (X3 && warp >= 6) {
