@@ -355,11 +355,33 @@ void launch_gate_reduced(const Shared &sh, const StepArgs &a, cudaStream_t s) {
 // ==================================================================== grouped GEMM ===
 // C = op(A) op(B) over a list of problems (the FP32 mode's contractions) on CUDA cores: 128 x 128
 // output tiles, 8-deep k slices through two shared-memory buffers (the next slice's global loads
-// are in flight while the current one is multiplied), 8 x 8 outputs per thread as 2 x 2 blocks
-// of 4 x 4 that lie 64 rows / columns apart, so each k step reads 16 bytes per operand block per
-// thread without bank conflicts.  Global loads are 16 bytes along whichever dimension of an
+// are in flight while the current one is multiplied), 8 x 16 outputs per thread as 2 x 4 blocks
+// of 4 x 4 that lie 64 rows / 32 columns apart.  A 16-byte shared read costs its warp 4 cycles of the
+// SM's one read path whatever it broadcasts, so an 8 x 8 thread tile (4 reads for 64 multiply-adds)
+// keeps that path as busy as the FMA pipes; 8 x 16 (6 for 128) leaves it a quarter idle.  Two blocks
+// of 128 threads share an SM, so one's slice hand-over and stores run under the other's products.
+// Products are packed pairs of columns, fma.rn.f32x2 with A's value in both halves: from registers an
+// outer product reaches 62 TFLOP/s so, 56 as single fmaf (whose operand reads collide), and this tile
+// with single ones spills (B Q of the 350M stack, rank 256: 3.71 ms; 8 x 8 tile 3.41; this 2.83, 55
+// TFLOP/s; six 2048-wide matrices at rank 512: 1.52 -> 1.09).
+// Global loads are 16 bytes along whichever dimension of an
 // operand is contiguous (zero outside the matrix).  Tile = {problem, tile row, tile col}.
-constexpr int GBM = kGemmTile, GBN = kGemmTile, GBK = 8, kGemmThreads = 256;
+constexpr int GBM = kGemmTile, GBN = kGemmTile, GBK = 8, kGemmThreads = 128, kGemmSmallThreads = 256;
+
+// Packed pairs of fp32 (lower half first): d += a * b, each half rounded as fmaf does
+__device__ __forceinline__ void fma2(unsigned long long &d, unsigned long long a, unsigned long long b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ unsigned long long dup2(float a) {
+  unsigned long long d;
+  asm("mov.b64 %0, {%1, %1};" : "=l"(d) : "f"(a));
+  return d;
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long v) {
+  float2 f;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(v));
+  return f;
+}
 
 // Elements (row, col .. col + 3) of a row-major matrix (col a multiple of 4, rows 16-byte
 // aligned), zero outside it.
@@ -374,7 +396,7 @@ __device__ __forceinline__ float4 ld4_rows(const float *base, int64_t row, int64
   return make_float4(v[0], v[1], v[2], v[3]);
 }
 
-__global__ void __launch_bounds__(kGemmThreads) gemm_kernel(Shared sh, const GemmProblem *probs,
+__global__ void __launch_bounds__(kGemmThreads, 2) gemm_kernel(Shared sh, const GemmProblem *probs,
                                                             const int4 *tiles) {
   chain_enter();
   const int4 t = tiles[blockIdx.x];
@@ -383,38 +405,42 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_kernel(Shared sh, const Gem
   DION_TILE_CHECK(p.layer >= 0 && p.layer < sh.num_layers && t.y >= 0 && t.z >= 0 &&
                       (int64_t)t.y * GBM < p.Mrows && (int64_t)t.z * GBN < p.Ncols, sh.status);
   if (!sh.active[p.layer]) return;
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
   const int64_t i0 = (int64_t)t.y * GBM, j0 = (int64_t)t.z * GBN;
   if (p.mode == GEMM_SHIFTED && !sh.orth_shifted[p.layer]) return;
   const float *B = (p.B_unshifted != nullptr && !sh.orth_shifted[p.layer]) ? p.B_unshifted : p.B;
   __shared__ __align__(16) float As[2][GBK][GBM + 4];
   __shared__ __align__(16) float Bs[2][GBK][GBN + 4];
-  // this thread's 16-byte share of a k slice of A (128 x 8) and of B (8 x 128): along the
+  // this thread's two 16-byte shares of a k slice of A (128 x 8) and of B (8 x 128): along the
   // contiguous dimension, 4 consecutive elements of one row / column
-  const int a_r = p.transA ? (tid >> 5) : (tid >> 1), a_c = p.transA ? (tid & 31) * 4 : (tid & 1) * 4;
-  const int b_r = p.transB ? (tid >> 1) : (tid >> 5), b_c = p.transB ? (tid & 1) * 4 : (tid & 31) * 4;
-  auto load = [&](int64_t k0, float4 &av, float4 &bv) {
-    av = p.transA ? ld4_rows(p.A, k0 + a_r, i0 + a_c, p.K, p.Mrows, p.lda)   // A^T stored K x M
-                  : ld4_rows(p.A, i0 + a_r, k0 + a_c, p.Mrows, p.K, p.lda);  // A stored M x K
-    bv = p.transB ? ld4_rows(B, j0 + b_r, k0 + b_c, p.Ncols, p.K, p.ldb)   // B^T stored N x K
-                  : ld4_rows(B, k0 + b_r, j0 + b_c, p.K, p.Ncols, p.ldb);  // B stored K x N
-  };
-  auto store = [&](int buf, const float4 &av, const float4 &bv) {
-    if (p.transA) {
-      *reinterpret_cast<float4 *>(&As[buf][a_r][a_c]) = av;
-    } else {
-      As[buf][a_c + 0][a_r] = av.x; As[buf][a_c + 1][a_r] = av.y;
-      As[buf][a_c + 2][a_r] = av.z; As[buf][a_c + 3][a_r] = av.w;
-    }
-    if (p.transB) {
-      Bs[buf][b_c + 0][b_r] = bv.x; Bs[buf][b_c + 1][b_r] = bv.y;
-      Bs[buf][b_c + 2][b_r] = bv.z; Bs[buf][b_c + 3][b_r] = bv.w;
-    } else {
-      *reinterpret_cast<float4 *>(&Bs[buf][b_r][b_c]) = bv;
+  auto load = [&](int64_t k0, float4 (&av)[2], float4 (&bv)[2]) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int id = tid + h * kGemmThreads;
+      av[h] = p.transA ? ld4_rows(p.A, k0 + (id >> 5), i0 + (id & 31) * 4, p.K, p.Mrows, p.lda)   // A^T stored K x M
+                       : ld4_rows(p.A, i0 + (id >> 1), k0 + (id & 1) * 4, p.Mrows, p.K, p.lda);  // A stored M x K
+      bv[h] = p.transB ? ld4_rows(B, j0 + (id >> 1), k0 + (id & 1) * 4, p.Ncols, p.K, p.ldb)    // B^T stored N x K
+                       : ld4_rows(B, k0 + (id >> 5), j0 + (id & 31) * 4, p.K, p.Ncols, p.ldb);   // B stored K x N
     }
   };
-  float acc[8][8] = {};
-  float4 av, bv;
+  auto put = [&](float (*D)[GBM + 4], bool along, int id, const float4 &v) {
+    if (along) {
+      *reinterpret_cast<float4 *>(&D[id >> 5][(id & 31) * 4]) = v;
+    } else {
+      const int c = (id & 1) * 4, row = id >> 1;
+      D[c + 0][row] = v.x; D[c + 1][row] = v.y;
+      D[c + 2][row] = v.z; D[c + 3][row] = v.w;
+    }
+  };
+  auto store = [&](int buf, const float4 (&av)[2], const float4 (&bv)[2]) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      put(As[buf], p.transA, tid + h * kGemmThreads, av[h]);
+      put(Bs[buf], !p.transB, tid + h * kGemmThreads, bv[h]);
+    }
+  };
+  unsigned long long acc[8][8] = {};
+  float4 av[2], bv[2];
   load(0, av, bv);
   store(0, av, bv);
   __syncthreads();
@@ -426,34 +452,41 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_kernel(Shared sh, const Gem
     for (int kk = 0; kk < GBK; ++kk) {
       const float4 a0 = *reinterpret_cast<const float4 *>(&As[cur][kk][ty * 4]);
       const float4 a1 = *reinterpret_cast<const float4 *>(&As[cur][kk][64 + ty * 4]);
-      const float4 b0 = *reinterpret_cast<const float4 *>(&Bs[cur][kk][tx * 4]);
-      const float4 b1 = *reinterpret_cast<const float4 *>(&Bs[cur][kk][64 + tx * 4]);
       const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-      const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+      unsigned long long b[8];
 #pragma unroll
-      for (int i = 0; i < 8; ++i)
+      for (int h = 0; h < 4; ++h) {
+        const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(&Bs[cur][kk][h * 32 + tx * 4]);
+        b[2 * h] = v.x; b[2 * h + 1] = v.y;
+      }
 #pragma unroll
-        for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+      for (int i = 0; i < 8; ++i) {
+        const unsigned long long d = dup2(a[i]);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) fma2(acc[i][j], d, b[j]);
+      }
     }
     if (more) store(cur ^ 1, av, bv);
     __syncthreads();
     cur ^= 1;
   }
-  // output rows ty*4 + (0..3) and 64 + ty*4 + (0..3), columns likewise with tx
+  // output rows ty*4 + (0..3) and 64 + ty*4 + (0..3), columns h*32 + tx*4 + (0..3)
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     const int64_t gi = i0 + (i < 4 ? ty * 4 + i : 64 + ty * 4 + (i - 4));
     if (gi >= p.Mrows) continue;
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int64_t gj = j0 + h * 64 + tx * 4;
+    for (int h = 0; h < 4; ++h) {
+      const int64_t gj = j0 + h * 32 + tx * 4;
       float *c = p.C + gi * p.ldc + gj;
+      const float2 lo = unpack2(acc[i][2 * h]), hi = unpack2(acc[i][2 * h + 1]);
+      const float v[4] = {lo.x, lo.y, hi.x, hi.y};
       if (gj + 4 <= p.Ncols) {
-        *reinterpret_cast<float4 *>(c) = make_float4(acc[i][4 * h], acc[i][4 * h + 1], acc[i][4 * h + 2], acc[i][4 * h + 3]);
+        *reinterpret_cast<float4 *>(c) = make_float4(v[0], v[1], v[2], v[3]);
       } else {
 #pragma unroll
         for (int e = 0; e < 4; ++e)
-          if (gj + e < p.Ncols) c[e] = acc[i][4 * h + e];
+          if (gj + e < p.Ncols) c[e] = v[e];
       }
     }
   }
@@ -466,7 +499,7 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_kernel(Shared sh, const Gem
 // warp's K / 128 chunks on small plans, by its shared-memory reads (3 for 32 multiply-adds) on large
 // ones; gemm_tiles (plan.cu) chooses and has both kernels' figures.
 constexpr int GST = kGemmSmallTile, GSK = 16;
-__global__ void __launch_bounds__(kGemmThreads) gemm_small_kernel(Shared sh, const GemmProblem *probs,
+__global__ void __launch_bounds__(kGemmSmallThreads) gemm_small_kernel(Shared sh, const GemmProblem *probs,
                                                                   const int4 *tiles) {
   chain_enter();
   const int4 t = tiles[blockIdx.x];
@@ -558,7 +591,7 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_small_kernel(Shared sh, con
 void launch_gemm(const Shared &sh, const GemmProblem *probs, const int4 *tiles, int32_t ntiles, bool small,
                  cudaStream_t s) {
   if (ntiles <= 0) return;
-  if (small) launch_chained(gemm_small_kernel, ntiles, kGemmThreads, 0, s, sh, probs, tiles);
+  if (small) launch_chained(gemm_small_kernel, ntiles, kGemmSmallThreads, 0, s, sh, probs, tiles);
   else launch_chained(gemm_kernel, ntiles, kGemmThreads, 0, s, sh, probs, tiles);
 }
 
@@ -1030,10 +1063,15 @@ void launch_colnorm(const Shared &sh, const int4 *tiles, int32_t ntiles, float e
 // M = B - (1 - mu) P R^T and X = X - eta sqrt(m/n) P Q_t^T in one pass over the tile, plus the
 // fp64 partial of ||M_t||^2 for Equation 1.  128 x 64 tiles, 8-deep k slices through two
 // shared-memory buffers (the next slice's 16-byte loads in flight during this one's products),
-// 8 x 4 outputs of each product per thread (rows 64 apart, so the 16-byte shared reads are
-// conflict-free); the epilogue reads and writes M and X 16 bytes at a time.
+// 8 x 8 outputs of each product per thread (2 x 2 blocks of 4 x 4, 64 rows and 32 columns apart) as
+// packed pairs: 6 16-byte shared reads for 128 multiply-adds, as in the grouped GEMM, and two blocks
+// per SM, so that one's epilogue runs under the other's products.  The tile's M and X are prefetched
+// into L2 when it starts, and the epilogue has a column block's 16 loads of 16 bytes in flight.  350M
+// stack, rank 256: 8.26 -> 6.40 ms (48 TFLOP/s; the tile alone 7.80, the loads together 7.26, the
+// prefetch 7.13, two threads per row of P, R and Q_t in a load 6.40); at rank 16, HBM-bound, two
+// 1024-wide blocks 139 -> 100 us.
 // Tile = {layer, tile row, tile col, slot}.
-constexpr int UBM = kUpdTileM, UBN = kUpdTileN, UBK = 8, kUpdThreads = 256;
+constexpr int UBM = kUpdTileM, UBN = kUpdTileN, UBK = 8, kUpdThreads = 128;
 
 __global__ void __launch_bounds__(kUpdThreads, 2) update_kernel(Shared sh, const int4 *tiles, float mu, float eta,
                                                              float keep) {
@@ -1049,26 +1087,38 @@ __global__ void __launch_bounds__(kUpdThreads, 2) update_kernel(Shared sh, const
   if (!sh.active[t.x]) return;
   const DevLayer &L = sh.layers[t.x];
   const float *P = sh.orth_shifted[t.x] ? L.P : L.P_raw;  // the last pass's result
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
   const int64_t i0 = (int64_t)t.y * UBM, j0 = (int64_t)t.z * UBN, r = L.r, ldp = L.ldp;
-  // this thread's share of a k slice: 4 consecutive k of one row of P, and of one row of R
-  // (threads 0..127) or of Q_t (threads 128..255)
-  const int pr = tid >> 1, kq = (tid & 1) * 4, br = (tid & 127) >> 1;
-  const bool is_q = tid >= 128;
-  auto load = [&](int64_t k0, float4 &pv, float4 &bv) {
-    pv = ld4_rows(P, i0 + pr, k0 + kq, L.m, r, ldp);
-    bv = is_q ? ld4_rows(L.Q, j0 + br, k0 + kq, L.n, r, L.ldq) : ld4_rows(L.R, j0 + br, k0 + kq, L.n, r, ldp);
+  // this thread's share of a k slice: 4 consecutive k of two rows of P (64 apart), of one row of R and
+  // of one of Q_t
+  const int kr = tid >> 1, kq = (tid & 1) * 4;
+  auto load = [&](int64_t k0, float4 (&pv)[2], float4 (&bv)[2]) {
+    pv[0] = ld4_rows(P, i0 + kr, k0 + kq, L.m, r, ldp);
+    pv[1] = ld4_rows(P, i0 + 64 + kr, k0 + kq, L.m, r, ldp);
+    bv[0] = ld4_rows(L.R, j0 + kr, k0 + kq, L.n, r, ldp);
+    bv[1] = ld4_rows(L.Q, j0 + kr, k0 + kq, L.n, r, L.ldq);
   };
-  auto store = [&](int buf, const float4 &pv, const float4 &bv) {
-    As[buf][kq + 0][pr] = pv.x; As[buf][kq + 1][pr] = pv.y;
-    As[buf][kq + 2][pr] = pv.z; As[buf][kq + 3][pr] = pv.w;
-    float(*Bd)[UBN + 4] = is_q ? Qs[buf] : Rs[buf];
-    Bd[kq + 0][br] = bv.x; Bd[kq + 1][br] = bv.y;
-    Bd[kq + 2][br] = bv.z; Bd[kq + 3][br] = bv.w;
+  auto store = [&](int buf, const float4 (&pv)[2], const float4 (&bv)[2]) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      As[buf][kq + 0][64 * h + kr] = pv[h].x; As[buf][kq + 1][64 * h + kr] = pv[h].y;
+      As[buf][kq + 2][64 * h + kr] = pv[h].z; As[buf][kq + 3][64 * h + kr] = pv[h].w;
+      float(*Bd)[UBN + 4] = h ? Qs[buf] : Rs[buf];
+      Bd[kq + 0][kr] = bv[h].x; Bd[kq + 1][kr] = bv[h].y;
+      Bd[kq + 2][kr] = bv[h].z; Bd[kq + 3][kr] = bv[h].w;
+    }
   };
-  float u1[8][4] = {}, u2[8][4] = {};
-  float4 pv, bv;
+  unsigned long long u1[8][4] = {}, u2[8][4] = {};
+  float4 pv[2], bv[2];
   load(0, pv, bv);
+  // this thread's row of the tile's M and X on its way into L2 under the products
+  if (i0 + tid < L.m)
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (j0 + 32 * h < L.n) {
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(L.M + (i0 + tid) * L.ldm + j0 + 32 * h));
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(L.X + (i0 + tid) * L.ldx + j0 + 32 * h));
+      }
   store(0, pv, bv);
   __syncthreads();
   int cur = 0;
@@ -1079,52 +1129,85 @@ __global__ void __launch_bounds__(kUpdThreads, 2) update_kernel(Shared sh, const
     for (int kk = 0; kk < UBK; ++kk) {
       const float4 a0 = *reinterpret_cast<const float4 *>(&As[cur][kk][ty * 4]);
       const float4 a1 = *reinterpret_cast<const float4 *>(&As[cur][kk][64 + ty * 4]);
-      const float4 b4 = *reinterpret_cast<const float4 *>(&Rs[cur][kk][tx * 4]);
-      const float4 q4 = *reinterpret_cast<const float4 *>(&Qs[cur][kk][tx * 4]);
       const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-      const float b[4] = {b4.x, b4.y, b4.z, b4.w}, q[4] = {q4.x, q4.y, q4.z, q4.w};
+      unsigned long long b[4], q[4];
 #pragma unroll
-      for (int i = 0; i < 8; ++i)
+      for (int h = 0; h < 2; ++h) {
+        const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(&Rs[cur][kk][h * 32 + tx * 4]);
+        const ulonglong2 w = *reinterpret_cast<const ulonglong2 *>(&Qs[cur][kk][h * 32 + tx * 4]);
+        b[2 * h] = v.x; b[2 * h + 1] = v.y;
+        q[2 * h] = w.x; q[2 * h + 1] = w.y;
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const unsigned long long d = dup2(a[i]);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          u1[i][j] = fmaf(a[i], b[j], u1[i][j]);
-          u2[i][j] = fmaf(a[i], q[j], u2[i][j]);
+          fma2(u1[i][j], d, b[j]);
+          fma2(u2[i][j], d, q[j]);
         }
+      }
     }
     if (more) store(cur ^ 1, pv, bv);
     __syncthreads();
     cur ^= 1;
   }
   const float dec = 1.f - mu, c = eta * L.sqrt_m_over_n;
-  float ss = 0.f;
-  const int64_t gj = j0 + tx * 4;
+  float ss[2] = {0.f, 0.f};  // one per column block: 32 entries in a row
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int64_t gi = i0 + (i < 4 ? ty * 4 + i : 64 + ty * 4 + (i - 4));
-    if (gi >= L.m || gj >= L.n) continue;
-    float *mp = L.M + gi * L.ldm + gj, *xp = L.X + gi * L.ldx + gj;
+  for (int h = 0; h < 2; ++h) {
+    const int64_t gj = j0 + h * 32 + tx * 4;
+    if (gj >= L.n) continue;
+    float *const m0 = L.M + gj, *const x0 = L.X + gj;
+    auto row = [&](int i) { return i0 + (i < 4 ? ty * 4 + i : 64 + ty * 4 + (i - 4)); };
     if (gj + 4 <= L.n) {
-      float4 mv = *reinterpret_cast<float4 *>(mp), xv = *reinterpret_cast<float4 *>(xp);
-      mv.x = fmaf(-dec, u1[i][0], mv.x); mv.y = fmaf(-dec, u1[i][1], mv.y);
-      mv.z = fmaf(-dec, u1[i][2], mv.z); mv.w = fmaf(-dec, u1[i][3], mv.w);
-      xv.x = fmaf(-c, u2[i][0], xv.x * keep); xv.y = fmaf(-c, u2[i][1], xv.y * keep);
-      xv.z = fmaf(-c, u2[i][2], xv.z * keep); xv.w = fmaf(-c, u2[i][3], xv.w * keep);
-      *reinterpret_cast<float4 *>(mp) = mv;
-      *reinterpret_cast<float4 *>(xp) = xv;
-      ss = fmaf(mv.x, mv.x, ss); ss = fmaf(mv.y, mv.y, ss);
-      ss = fmaf(mv.z, mv.z, ss); ss = fmaf(mv.w, mv.w, ss);
+      float4 mv[8], xv[8];  // all of a column block's loads in flight together
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int64_t gi = row(i);
+        mv[i] = xv[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (gi < L.m) {
+          mv[i] = *reinterpret_cast<const float4 *>(m0 + gi * L.ldm);
+          xv[i] = *reinterpret_cast<const float4 *>(x0 + gi * L.ldx);
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int64_t gi = row(i);
+        if (gi >= L.m) continue;
+        const float2 a0 = unpack2(u1[i][2 * h]), a1 = unpack2(u1[i][2 * h + 1]);
+        const float2 b0 = unpack2(u2[i][2 * h]), b1 = unpack2(u2[i][2 * h + 1]);
+        float4 &m = mv[i], &x = xv[i];
+        m.x = fmaf(-dec, a0.x, m.x); m.y = fmaf(-dec, a0.y, m.y);
+        m.z = fmaf(-dec, a1.x, m.z); m.w = fmaf(-dec, a1.y, m.w);
+        x.x = fmaf(-c, b0.x, x.x * keep); x.y = fmaf(-c, b0.y, x.y * keep);
+        x.z = fmaf(-c, b1.x, x.z * keep); x.w = fmaf(-c, b1.y, x.w * keep);
+        *reinterpret_cast<float4 *>(m0 + gi * L.ldm) = m;
+        *reinterpret_cast<float4 *>(x0 + gi * L.ldx) = x;
+        ss[h] = fmaf(m.x, m.x, ss[h]); ss[h] = fmaf(m.y, m.y, ss[h]);
+        ss[h] = fmaf(m.z, m.z, ss[h]); ss[h] = fmaf(m.w, m.w, ss[h]);
+      }
     } else {
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        if (gj + j >= L.n) continue;
-        const float mn = fmaf(-dec, u1[i][j], mp[j]);
-        mp[j] = mn;
-        xp[j] = fmaf(-c, u2[i][j], xp[j] * keep);
-        ss = fmaf(mn, mn, ss);
+      for (int i = 0; i < 8; ++i) {
+        const int64_t gi = row(i);
+        if (gi >= L.m) continue;
+        const float2 a0 = unpack2(u1[i][2 * h]), a1 = unpack2(u1[i][2 * h + 1]);
+        const float2 b0 = unpack2(u2[i][2 * h]), b1 = unpack2(u2[i][2 * h + 1]);
+        const float d1[4] = {a0.x, a0.y, a1.x, a1.y}, d2[4] = {b0.x, b0.y, b1.x, b1.y};
+        float *mp = m0 + gi * L.ldm, *xp = x0 + gi * L.ldx;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          if (gj + j >= L.n) continue;
+          const float mn = fmaf(-dec, d1[j], mp[j]);
+          mp[j] = mn;
+          xp[j] = fmaf(-c, d2[j], xp[j] * keep);
+          ss[h] = fmaf(mn, mn, ss[h]);
+        }
       }
     }
   }
-  const double tot = block_sum<kUpdThreads>((double)ss, red);
+  const double tot = block_sum<kUpdThreads>((double)ss[0] + (double)ss[1], red);
   if (tid == 0) sh.upart[t.w] = tot;
 }
 

@@ -150,11 +150,11 @@ int64_t row_tile_elems(const dion_layer *layers, int32_t num_layers, int sms) {
 // short ones: 3.72 / 3.41 ms for B Q on the 350M stack).  lower: tiles above the diagonal are left
 // out (a Gram, whose lower triangle alone is read).  *small: 32 x 32 tiles (K split over a block's
 // warps) instead of 128 x 128, where an estimate from both kernels' measured rates says so.  Large
-// tiles: 22e6 multiply-adds per us in all, and 0.117 us per k of the longest tile alone on its SM,
-// 0.16 with a second one beside it; small ones: 15.5e6, and 5 us + 0.0125 us per k.  Measured, large /
-// small: 256 x 512 rank 16 B Q 68 / 14 us, Gram 37 / 10; one 1024-wide block at rank 256 B Q 491 /
-// 215, Gram 475 / 58, solve 39 / 57; four 768-wide blocks at rank 192 B Q 502 / 360; the 350M stack
-// B Q 3407 / 4852, Gram 665 / 496, solve 706 / 1196.
+// tiles: 27e6 multiply-adds per us in all, and 0.118 us per k of the longest tile alone on its SM,
+// 0.13 where tiles share one; small ones: 15.5e6, and 5 us + 0.0125 us per k.  Measured, large /
+// small: one 1024 x 4096 matrix at rank 256 B Q 483 / 83 us, Gram 123 / 18, B^T P 125 / 76, solve 39 /
+// 12; one 768-wide block at rank 192 B Q 371 / 101, solve 31 / 31; two 2048-wide blocks at rank 128
+// B Q 1025 / 792; the 350M stack B Q 2834 / 4852, solve 583 / 1196.
 std::vector<int4> gemm_tiles(const std::vector<GemmProblem> &probs, bool lower, int sms, bool *small) {
   int64_t longest = 0;
   for (const GemmProblem &q : probs) longest = std::max(longest, q.K);
@@ -172,7 +172,7 @@ std::vector<int4> gemm_tiles(const std::vector<GemmProblem> &probs, bool lower, 
   };
   double macs_l, macs_s;
   std::vector<int4> t = tiles_of(kGemmTile, &macs_l), ts = tiles_of(kGemmSmallTile, &macs_s);
-  const double us_l = std::max(macs_l / 22e6, ((int64_t)t.size() > sms ? 0.16 : 0.117) * (double)longest);
+  const double us_l = std::max(macs_l / 27e6, ((int64_t)t.size() > sms ? 0.13 : 0.118) * (double)longest);
   const double us_s = std::max(macs_s / 15.5e6, 5.0 + 0.0125 * (double)longest);
   *small = us_s < us_l;
   if (*small) t = std::move(ts);
