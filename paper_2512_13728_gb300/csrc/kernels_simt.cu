@@ -973,10 +973,13 @@ void launch_chol_inv(const Shared &sh, size_t smem, int32_t pass, float near_ide
 
 // ===================================================================== ColumnNormalize ===
 // Q_t[:, j] = R[:, j] / (||R[:, j]||_2 + eps_col).  Tile = {layer, 32-column group}.  A thread
-// owns 4 adjacent columns of every 32nd row (8 threads span the group's 128 bytes of a row, so a
+// owns 4 adjacent columns of every 64th row (8 threads span the group's 128 bytes of a row, so a
 // warp reads 4 full row segments per instruction) and keeps 4 rows' 16-byte loads in flight;
-// fp32 sums of 16 rows folded into fp64, the 32 row-group partials added in a fixed order.
-constexpr int kColThreads = 256, kColRowGroups = kColThreads / 8, kColUnroll = 4;
+// fp32 sums of 16 rows folded into fp64, the 64 row-group partials added in a fixed order.  Bound by
+// the loads of one block's rows in turn where a plan has few groups, by HBM where it has many.  With
+// 256 / 512 / 1024 threads: one 768-wide block at rank 192 34 / 26 / 24 us, four 1024-wide at rank 64
+// 51 / 35 / 31, the 160M stack at rank 192 50 / 46 / 55, the 350M stack at rank 256 137 / 124 / 131.
+constexpr int kColThreads = 512, kColRowGroups = kColThreads / 8, kColUnroll = 4;
 
 __global__ void __launch_bounds__(kColThreads) colnorm_kernel(Shared sh, const int4 *tiles, float eps_col) {
   chain_enter();
@@ -1024,10 +1027,17 @@ __global__ void __launch_bounds__(kColThreads) colnorm_kernel(Shared sh, const i
   part[rg][4 * quad + 2] = a2 + f2;
   part[rg][4 * quad + 3] = a3 + f3;
   __syncthreads();
-  if (threadIdx.x < 32) {
+  const int col = threadIdx.x & 31, seg = threadIdx.x >> 5;  // a warp adds 32 row groups
+  if (seg < kColRowGroups / 32) {
     double s = 0.0;
-    for (int g = 0; g < kColRowGroups; ++g) s += part[g][threadIdx.x];
-    inv[threadIdx.x] = (float)(1.0 / (sqrt(s) + (double)eps_col));
+    for (int g = 0; g < 32; ++g) s += part[seg * 32 + g][col];
+    part[seg * 32][col] = s;
+  }
+  __syncthreads();
+  if (seg == 0) {
+    double s = 0.0;
+    for (int g = 0; g < kColRowGroups / 32; ++g) s += part[g * 32][col];
+    inv[col] = (float)(1.0 / (sqrt(s) + (double)eps_col));
   }
   __syncthreads();
   if (nc == 0) return;
