@@ -141,8 +141,7 @@ def _kernel_work(name: str, w, prec: str, gate: str = "always", wt=None):
         # buffer pass fused into B Q (bf16 G): read M (and G unless B is already in M); write Bh,
         # P and P^T fp32
         "tc_form_bq": ("hbm", mn * (4 + (0 if b_in_m else gsz) + 2) + mr * 8, "B"),
-        # gated modes: the norms pass reads M, G and writes B into M on every layer (and runs
-        # the gate in its last block)
+        # gated modes: the norms pass reads M, G and writes B into M on every layer
         "norms_gate": ("hbm", mn_all * (4 + gsz + 4), "B"),
         "tc_btp": ("hbm", mn * bh + mr * 2 * hl + nr * (4 + 2 * hl), "B"),  # Bh (Bl), bf16 P; R fp32, bf16
         "tc_update": ("hbm", mn * (16 + (gsz if deferred else 0)), "B"),

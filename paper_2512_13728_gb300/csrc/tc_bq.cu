@@ -3,12 +3,14 @@
 //
 //   P = B Q_{t-1} (PowerIter)  and  R = B^T P (after Orthogonalize)
 //
-// run as one persistent TMA-fed GEMM kernel template: warp 0 issues TMA loads of both bf16
-// operands into a shared-memory ring, warp 1 issues 128 x N x 16 tcgen05.mma (N <= 256 per
-// instruction) into a 128 x r fp32 TMEM accumulator, warps 2..5 drain TMEM through swizzled
-// shared boxes into TMA stores.  Bh serves both GEMMs (K-major rows for B Q, MN-major boxes for
-// B^T P), the bf16 copy of Q is read MN-major and the bf16 copy of P MN-major, so no transposed
-// copy of a large matrix is made.
+// run as one persistent TMA-fed GEMM kernel template over CTA pairs (256 rows a pair, half of the
+// second operand in each CTA): warp 0 issues TMA loads of both bf16 operands into a shared-memory
+// ring, the even CTA's warp 1 issues the pair MMAs (N <= 256 per instruction) into a fp32 TMEM
+// accumulator of 128 rows a CTA (two, alternating between tiles, where a tile's columns fit 256),
+// warps 2..5 drain TMEM through swizzled shared boxes into TMA stores.  Bh serves both GEMMs (K-major
+// rows for B Q, MN-major boxes for B^T P), the bf16 copy of Q is read MN-major and the bf16 copy of
+// P MN-major, so no transposed copy of a large matrix is made.  With bf16 gradients the buffer pass
+// and B Q are one kernel, tc_form_bq below.
 //   qn_refresh   the bf16 copy of the caller's Q (plan creation, dion_plan_refresh).
 #include "tc.cuh"
 #include "tc_common.cuh"
