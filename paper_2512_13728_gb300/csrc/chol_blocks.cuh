@@ -106,6 +106,7 @@ __device__ __forceinline__ void diag_factor_segment(float (&v)[CB], DiagState &d
       v[4 * q + 1] = fmaf(-t, b.z, v[4 * q + 2]);
       v[4 * q + 2] = fmaf(-t, b.w, v[4 * q + 3]);
     }
+    __syncwarp();  // every lane has read this column: the next iteration writes its buffer
   }
 }
 // v: this lane's row of the block (entries right of the diagonal are not used).  Returns whether
