@@ -311,7 +311,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(R_THREADS, 1)
         const uint32_t id0 = idesc_bf16(256, 2u * half_cols(np, 0), KIND == GEMM_BTP, true);
         const uint32_t id1 = nparts > 1u ? idesc_bf16(256, 2u * half_cols(np, 1), KIND == GEMM_BTP, true) : 0u;
         const uint32_t slot = acc.s;
-        if (!ab.wait(&acc_empty[slot], acc.ph ^ 1u, sh.status)) break;
+        if (!ab.wait<true>(&acc_empty[slot], acc.ph ^ 1u, sh.status)) break;
         tc_fence_after();
         for (int kc = 0; kc < kch; ++kc) {
           if (!ab.wait(&full[rp.s], rp.ph, sh.status)) { ok = false; break; }
@@ -400,7 +400,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(R_THREADS, 1)
 // HBM-bound on stacks (1.3B, rank 512: 1.85 ms for 11.5 GB; 160M, rank 48: 124 us for 0.72 GB).  M
 // came through 16-byte cp.async copies of four warps before, which kept about 16 KB in flight per SM
 // (4100 cycles per chunk), and each chunk's arrival in CTA 0 took 2700 cycles more (see
-// mbar_arrive_cluster): 2417 us on the 1.3B stack, 174 / 207 us on the 160M stack at ranks 48 / 192
+// mbar_publish_cluster): 2417 us on the 1.3B stack, 174 / 207 us on the 160M stack at ranks 48 / 192
 // (now 124 / 152), 119 us on the 160M block (now 56).
 constexpr int FB_MSTAGES = 3;  // M ring (2 x 16 KB per slot)
 constexpr int FB_ASTAGES = 4;  // G / A ring (16 KB per slot)
@@ -595,10 +595,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(FB_THREADS, 1)
         const uint32_t np = rpad16(L.r), nparts = (np + 255) / 256;
         const uint32_t id0 = idesc_bf16(256, 2u * half_cols(np, 0), false, true);
         const uint32_t id1 = nparts > 1u ? idesc_bf16(256, 2u * half_cols(np, 1), false, true) : 0u;
-        if (!ab.wait(acc_empty, (tcount & 1u) ^ 1u, sh.status)) break;
+        if (!ab.wait<true>(acc_empty, (tcount & 1u) ^ 1u, sh.status)) break;
         tc_fence_after();
         for (int kc = 0; kc < kch; ++kc) {
-          if (!ab.wait(&qfull[rq.s], rq.ph, sh.status) || !ab.wait(&afull[ra.s], ra.ph, sh.status)) { ok = false; break; }
+          if (!ab.wait(&qfull[rq.s], rq.ph, sh.status) || !ab.wait<true>(&afull[ra.s], ra.ph, sh.status)) {
+            ok = false;
+            break;
+          }
+          acquire_pair_smem();  // the converted A boxes of both CTAs
           tc_fence_after();
           const uint64_t ads = desc_at(ad0, ra.s * FB_GBOX), bds = desc_at(bd0, rq.s * qstage_bytes);
 #pragma unroll
@@ -699,7 +703,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(FB_THREADS, 1)
         if (!named_and(2, FB_CT, in)) { ok = false; break; }
         if (ct == 0) {
           mbar_arrive(&mempty[sm]);
-          mbar_arrive_cluster(cluster_addr(&afull[sg], 0));
+          mbar_publish_cluster(cluster_addr(&afull[sg], 0));
           mbar_arrive(&cvt[sg]);
         }
       }

@@ -41,13 +41,24 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
                : "memory");
 }
+// PAIR: the arrivals may come from the other CTA of the cluster (mbar_arrive_cluster and
+// mbar_publish_cluster); what they order is named there.
+template <bool PAIR = false>
 __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
   uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
+  if constexpr (PAIR)
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.relaxed.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, "
+        "0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+  else
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
   return ok != 0;
 }
 // Bounded wait for the phase with the given parity to complete.  Returns false on timeout
@@ -180,13 +191,27 @@ __device__ __forceinline__ void tma_load_2d_pair(void *dst, const CUtensorMap *m
       "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1)
       : "memory");
 }
-// Arrival on a barrier of either CTA (`bar` is a shared::cluster address), with the instruction's
-// default release at CTA scope: what it publishes are shared-memory writes that each writer has
-// fenced to the async proxy (fence_async_smem) before a barrier among them, and TMEM reads ordered
-// by tcgen05.fence.  With .release.cluster the arriving thread waited ~2700 cycles here, per
-// 64-column chunk in the fused buffer kernel.
+// Arrivals on a barrier of either CTA of the pair (`bar` is a shared::cluster address).  The waiting
+// thread may be in the other CTA, so both sides name the cluster scope; it waits with
+// mbar_try_wait<true> (Abort::wait<true>).
+//   mbar_arrive_cluster   frees a TMEM accumulator.  What has to be over are TMEM reads, which
+//     tcgen05.wait::ld and tcgen05.fence::before_thread_sync order before the arrival and the waiter's
+//     tcgen05.fence::after_thread_sync before its MMAs; no memory is handed over, so it is relaxed.
+//   mbar_publish_cluster  hands over shared memory of this CTA that a pair MMA issued in the other
+//     one reads.  Each writer has fenced its writes to the async proxy (fence_async_smem) and they
+//     meet at a barrier before this thread; its release fence and the waiter's acquire_pair_smem are
+//     at cluster scope, limited to shared memory.
+// mbarrier.arrive.release.cluster orders every kind of memory instead and held the arriving thread for
+// ~2700 cycles per 64-column chunk of the fused buffer kernel.
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void mbar_publish_cluster(uint32_t bar) {
+  asm volatile("fence.release.sync_restrict::shared::cta.cluster;" ::: "memory");
+  mbar_arrive_cluster(bar);
+}
+__device__ __forceinline__ void acquire_pair_smem() {
+  asm volatile("fence.acquire.sync_restrict::shared::cluster.cluster;" ::: "memory");
 }
 
 // ------------------------------------------------------------------------ cluster ---
@@ -343,14 +368,15 @@ bool encode_f32_2d(CUtensorMap *map, const void *base, uint64_t inner, uint64_t 
 struct Abort {
   int *flag;
   uint64_t limit_ns = kWaitLimitNs;
+  template <bool PAIR = false>
   __device__ bool wait(uint64_t *bar, uint32_t parity, int32_t *status) const {
-    if (mbar_try_wait(bar, parity)) return true;
+    if (mbar_try_wait<PAIR>(bar, parity)) return true;
     const uint64_t t0 = globaltimer_ns();
     // the clock is read every 256 tries at the default limit (each try may suspend the thread
     // for a while), and on every try under a shortened one
     const uint32_t every = limit_ns < kWaitLimitNs ? 0u : 255u;
     for (uint32_t i = 1;; ++i) {
-      if (mbar_try_wait(bar, parity)) return true;
+      if (mbar_try_wait<PAIR>(bar, parity)) return true;
       if ((i & every) == 0) {
         if (*(volatile int *)flag) return false;
         if (globaltimer_ns() - t0 > limit_ns) {

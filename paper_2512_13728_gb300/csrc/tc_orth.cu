@@ -270,7 +270,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(X3 ? O_THREADS_X3 : 
     auto report = [&](uint32_t s) {
       fence_async_smem();  // the converted boxes are visible to the tensor cores' reads
       named_sync(2, 128);
-      if (ct == 0) mbar_arrive_cluster(cluster_addr(&conv[s], 0));
+      if (ct == 0) mbar_publish_cluster(cluster_addr(&conv[s], 0));
     };
     uint32_t it = 0;
     bool ok = true;
@@ -328,12 +328,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(X3 ? O_THREADS_X3 : 
         if constexpr (KIND == ORTH_TRSM) {
           for (uint32_t q = 0; q < nparts && ok; ++q) {
             const uint32_t slot = tcount & 1u;  // tcount counts sub-tiles here
-            if (!ab.wait(&acc_empty[slot], ((tcount >> 1) & 1u) ^ 1u, sh.status)) { ok = false; break; }
+            if (!ab.wait<true>(&acc_empty[slot], ((tcount >> 1) & 1u) ^ 1u, sh.status)) { ok = false; break; }
             tc_fence_after();
             const int kq = min(kch, (int)(8u * (q + 1u)));
             const uint32_t idesc = idesc_tf32(256, 2u * half_rows(N, q), false, false), d = tmem + slot * 256u;
             for (int kc = 0; kc < kq; ++kc) {
-              if (!ab.wait(&ready[rp.s], rp.ph, sh.status)) { ok = false; break; }
+              if (!ab.wait<X3>(&ready[rp.s], rp.ph, sh.status)) { ok = false; break; }
+              if (X3) acquire_pair_smem();  // the split boxes of both CTAs
               tc_fence_after();
               const uint64_t as = desc_at(sd0, rp.s * stage_bytes);
 #pragma unroll
@@ -357,7 +358,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(X3 ? O_THREADS_X3 : 
         const GramTile g = gram_tile(L.r, t.y & 0xff);
         const uint32_t slot = slots == 2u ? (tcount & 1u) : 0u;
         const uint32_t aph = slots == 2u ? ((tcount >> 1) & 1u) : (tcount & 1u);
-        if (!ab.wait(&acc_empty[slot], aph ^ 1u, sh.status)) break;
+        if (!ab.wait<true>(&acc_empty[slot], aph ^ 1u, sh.status)) break;
         tc_fence_after();
         const uint32_t d0 = tmem + slot * 256u;
         // per part: its instruction and its A box (in place in a B box, or the stage's own)
@@ -365,7 +366,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(X3 ? O_THREADS_X3 : 
         const uint32_t ao[2] = {g.a_box[0] >= 0 ? (uint32_t)(1 + g.a_box[0]) * O_BOX : 0u,
                                 g.a_box[1] >= 0 ? (uint32_t)(1 + g.a_box[1]) * O_BOX : 0u};
         for (int kc = 0; kc < t.w; ++kc) {
-          if (!ab.wait(&ready[rp.s], rp.ph, sh.status)) { ok = false; break; }
+          if (!ab.wait<X3>(&ready[rp.s], rp.ph, sh.status)) { ok = false; break; }
+          if (X3) acquire_pair_smem();  // the split boxes of both CTAs
           tc_fence_after();
           const uint64_t as = desc_at(sd0, rp.s * stage_bytes);
 #pragma unroll

@@ -172,7 +172,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(U_THREADS, 1)
         if (!sh.active[t.x]) continue;
         const int kch = (int)((sh.layers[t.x].r + KW - 1) / KW);
         const uint32_t b = tcount & 1u, aph = (tcount >> 1) & 1u;
-        if (!ab.wait(&acc_empty[b], aph ^ 1u, sh.status)) break;
+        if (!ab.wait<true>(&acc_empty[b], aph ^ 1u, sh.status)) break;
         tc_fence_after();
         const uint32_t d1 = tmem + b * 256u, d2 = d1 + 128u;
         for (int kc = 0; kc < kch; ++kc, ++it) {

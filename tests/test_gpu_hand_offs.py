@@ -56,3 +56,14 @@ def test_cholesky_blocks_repeat_bitwise(prec, rank):
     """The three Cholesky kernels, whose two warps per diagonal block pass columns through shared memory."""
     w = wl.scaled(wl.WORKLOADS["gpt160m_block_r192"], "lanes", [(520, 300), (300, 520)] * 8, rank=rank)
     repeat(w, prec, 24)
+
+
+@pytest.mark.parametrize("prec,rank,g_dtype", [("bf16", 48, "bf16"), ("bf16", 300, "bf16"), ("bf16x3", 64, "bf16"),
+                                               ("bf16x3", 256, "fp32")])
+def test_pair_hand_offs_repeat_bitwise(prec, rank, g_dtype):
+    """Converted operand boxes that the pair's other CTA has multiplied: the fused buffer kernel (bf16,
+    bf16 gradients) and the Gram and solve with split operands, over many chunks and tiles per pair,
+    with an empty second row tile and partial chunks."""
+    w = wl.scaled(wl.WORKLOADS["gpt160m_block_r192"], "pairs", [(1160, 1100), (640, 2056), (2056, 640)] * 12, rank=rank,
+                  g_dtype=g_dtype)
+    repeat(w, prec, 24)
