@@ -748,11 +748,13 @@ __device__ bool chol_inverse(const float *S, float *__restrict__ W, int r, int64
   return true;
 }
 
-// ||S - I||_2 estimated by 8 power iterations.  S - I is symmetric, so each product reads only
-// the 32 x 32 tiles on and below the diagonal (half of S, which stays in L2 across the
-// iterations): warp w takes tiles w, w + 16, ... and adds each tile's row sums (a
-// reduce-scatter over the lanes) and, off the diagonal, its column sums into its own partial
-// vector; the partials are then summed in warp order, so the estimate is deterministic.
+// ||S - I||_2 estimated by 8 power iterations.  S - I is symmetric and S holds its lower triangle
+// (above the diagonal a split Gram has the first row range's partial sum alone), so each product
+// reads only the entries on and below the diagonal (half of S, which stays in L2 across the
+// iterations): warp w takes the 32 x 32 tiles w, w + 16, ... and adds each tile's row sums (a
+// reduce-scatter over the lanes) and, for the mirrored entries, the column sums of what lies
+// below the diagonal into its own partial vector; the partials are then summed in warp order, so
+// the estimate is deterministic.
 // Shared memory: Y (at least 18 rows of ldy floats).  Called by the whole block.
 __device__ __noinline__ float power_norm_sym(const float *S, int r, int64_t ls, float *Y, int ldy) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -777,9 +779,9 @@ __device__ __noinline__ float power_norm_sym(const float *S, int r, int64_t ls, 
       for (int y = 0; y < 32; ++y) {
         const int row = bi * 32 + y;
         float e = 0.f;
-        if (row < r && c < r) e = S[(int64_t)row * ls + c] - (row == c ? 1.f : 0.f);
+        if (row < r && c <= row) e = S[(int64_t)row * ls + c] - (row == c ? 1.f : 0.f);
         a[y] = e * vc;
-        if (bi != bj) colsum = fmaf(e, (row < r) ? pv[row] : 0.f, colsum);
+        if (c != row) colsum = fmaf(e, (row < r) ? pv[row] : 0.f, colsum);
       }
       // reduce-scatter: lane y ends with sum over the lanes of a[y] (row y of the tile)
 #pragma unroll
@@ -794,7 +796,7 @@ __device__ __noinline__ float power_norm_sym(const float *S, int r, int64_t ls, 
       }
       if (bi * 32 + lane < r) mine[bi * 32 + lane] += a[0];
       __syncwarp();
-      if (bi != bj && c < r) mine[c] += colsum;
+      if (c < r) mine[c] += colsum;
       __syncwarp();
     }
     __syncthreads();
