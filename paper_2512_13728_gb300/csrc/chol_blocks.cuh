@@ -79,7 +79,7 @@ __device__ __forceinline__ void diag_column(DiagScratch &sc, DiagState &ds, int 
   ds.next = col[CB];
 }
 // Columns 32 - N .. 39 - N: v[0 .. N) hold this lane's row from column 32 - N on.  Every lane also
-// works out the next pivot (the arithmetic of the lane that holds it), and the next column is on its
+// works out the next pivot (the lane that holds it does not use its own), and the next column is on its
 // way through shared memory before this one's multiply-adds, which run under both latencies.
 template <int N>
 __device__ __forceinline__ void diag_factor_segment(float (&v)[CB], DiagState &ds, DiagScratch &sc, int lane) {
@@ -87,11 +87,11 @@ __device__ __forceinline__ void diag_factor_segment(float (&v)[CB], DiagState &d
   for (int J = CB - N; J < CB - N + 8; ++J) {
     const float *col = sc.col[J & 1];
     const float4 a = ds.a;
-    const float inv = ds.rs * ds.rs;
-    const float t = lane > J ? v[0] * inv : 0.f;
+    // scaled twice by 1 / sqrt(pivot): 1 / pivot itself overflows for a subnormal pivot
+    const float t = lane > J ? (v[0] * ds.rs) * ds.rs : 0.f, l1 = a.y * ds.rs;
     const float v0 = fmaf(-t, a.y, v[1]), v1 = fmaf(-t, a.z, v[2]), v2 = fmaf(-t, a.w, v[3]);
     sc.rs[J] = ds.rs;
-    ds.piv = fmaf(-(a.y * inv), a.y, ds.next);
+    ds.piv = fmaf(-l1, l1, ds.next);
     ds.rs = rsqrtf(ds.piv);
     diag_column(sc, ds, J + 1, lane, v0, v1);
     sc.t[J][(lane - J) & 31] = t;

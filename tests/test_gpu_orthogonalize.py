@@ -92,3 +92,19 @@ def test_hard_p_with_a_split_gram(m, n, r, power, zero_rows, prec):
             assert apart <= DEFECT[prec] + ORDER * cond
     print("defect", worst)
     assert worst <= DEFECT[prec]
+
+
+@pytest.mark.parametrize("r", [16, 40])
+@pytest.mark.parametrize("gram", [2e38, 1.0, 1e-39, 1e-41])
+def test_gram_at_the_ends_of_fp32(gram, r):
+    """Pivots at the largest fp32 values and among the subnormal ones (whose reciprocals overflow), in FP32
+    mode.  A Gram of 1e-41 keeps 13 bits, which pass 1 makes up for: 3 (1e-3 / 1.5)^2 = 1.3e-6 is the most
+    that the first-order factor leaves, and the fp32 solve adds about r 2^-24."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(2)
+    B = torch.randn((256, 320), generator=g, device="cuda") * math.sqrt(gram / 256)
+    Q = torch.linalg.qr(torch.randn((320, r), generator=g, device="cuda"))[0].contiguous()
+    P = orthonormal_p(B, Q, "fp32", 1)
+    defect = torch.linalg.matrix_norm(P.T @ P - torch.eye(r, device="cuda", dtype=torch.float64), 2).item()
+    print("defect", defect)
+    assert defect <= 1e-5
