@@ -234,7 +234,9 @@ int32_t dion_step_launch_count(const dion_plan *plan);
  * dion_timing_read(plan, cap, ms_out, names_out, count_out): synchronizes on the recorded
  * events, writes the average duration in milliseconds of each launch position over the
  * recorded steps (ms_out[i], names_out[i] = static kernel name) for i < min(cap, launches),
- * sets *count_out to the number of launches per step and to 0 steps recorded afterwards.
+ * sets *count_out to the number of launches per recorded step and to 0 steps recorded afterwards.
+ * Recorded steps have one launch sequence: a step with another one (a gated mode after
+ * DION_GATE_ALWAYS, or the reverse) drops what is recorded so far, until max_steps are.
  * Errors: INVALID_ARG (NULL plan/outputs), CUDA. */
 dion_status dion_timing_enable(dion_plan *plan, int32_t max_steps);
 dion_status dion_timing_read(dion_plan *plan, int32_t cap, float *ms_out, const char **names_out,

@@ -48,6 +48,7 @@ struct dion_plan {
   std::vector<cudaEvent_t> ev;  // [max_steps][launches + 1]
   std::vector<const char *> names;
   int32_t timing_steps = 0, recorded = 0, cursor = 0;
+  int32_t timed_launches = 0;  // of the recorded steps
   // host gradients (dion_step_host): two device gradient buffers per layer, filled in turn
   std::vector<DevLayer> dl_host;  // the layer records as uploaded at creation
   struct HostGrad {
@@ -81,10 +82,12 @@ void tick_begin(dion_plan *p, cudaStream_t s) {
   cudaEventRecord(p->ev[(size_t)p->recorded * (kMaxLaunches + 1)], s);
 }
 void tick_end(dion_plan *p) {
-  // steps are averaged launch by launch: a gate mode with another sequence starts again
-  if (p->cursor != p->launches_per_step && p->recorded > 0) p->recorded = -1;
   p->launches_per_step = p->cursor;
-  if (p->timing_steps > 0 && p->recorded < p->timing_steps) ++p->recorded;
+  if (p->timing_steps <= 0 || p->recorded >= p->timing_steps) return;  // a finished recording stays
+  // steps are averaged launch by launch: a gate mode with another sequence starts again
+  if (p->recorded > 0 && p->cursor != p->timed_launches) p->recorded = 0;
+  else ++p->recorded;
+  p->timed_launches = p->cursor;
 }
 }  // namespace cd
 
@@ -819,7 +822,8 @@ dion_status dion_timing_read(dion_plan *p, int32_t cap, float *ms_out, const cha
                              int32_t *steps_out) {
   if (!p || !count_out || !steps_out || (cap > 0 && (!ms_out || !names_out))) return DION_ERR_INVALID_ARG;
   const int32_t per = kMaxLaunches + 1;
-  const int32_t n = std::min(std::min(cap, p->launches_per_step), kMaxLaunches);
+  const int32_t launches = p->recorded > 0 ? p->timed_launches : p->launches_per_step;
+  const int32_t n = std::min(std::min(cap, launches), kMaxLaunches);
   for (int32_t i = 0; i < n; ++i) {
     double tot = 0.0;
     for (int32_t st = 0; st < p->recorded; ++st) {
@@ -832,7 +836,7 @@ dion_status dion_timing_read(dion_plan *p, int32_t cap, float *ms_out, const cha
     ms_out[i] = p->recorded ? (float)(tot / p->recorded) : 0.f;
     names_out[i] = i < (int32_t)p->names.size() ? p->names[i] : "";
   }
-  *count_out = p->launches_per_step;
+  *count_out = launches;
   *steps_out = p->recorded;
   p->recorded = 0;
   return DION_OK;
