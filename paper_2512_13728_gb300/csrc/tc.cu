@@ -378,7 +378,8 @@ cudaError_t init(const TcLayout &lo, char *base, const DevLayer *dl, int32_t L, 
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   tp->num_sms = sms;
-  tp->launches = tp->fuse_buffer ? 16 : x3 ? 18 : 17;  // of an ALWAYS step; BF16X3: the split of B
+  // of an ALWAYS step; BF16X3: the split of B; ranks on both sides of 256: two first-pass Cholesky kernels
+  tp->launches = (tp->fuse_buffer ? 16 : x3 ? 18 : 17) + (tp->min_r <= kCholTmemRank && tp->max_r > kCholTmemRank);
   return e;
 }
 

@@ -57,3 +57,23 @@ def test_finished_timing_outlives_a_step_of_another_mode(prec):
         assert recorded == 2 and len(launches) == gated and "local" in [name for name, _ in launches]
     finally:
         plan.close()
+
+
+@pytest.mark.parametrize("prec,shapes,rank", [("fp32", [(200, 136)], 16), ("bf16", [(200, 136)], 16),
+                                              ("bf16", [(400, 500)], 300), ("bf16x3", [(200, 136)], 16),
+                                              ("bf16", [(520, 300), (300, 200), (400, 700), (200, 64)], 300)])
+@pytest.mark.parametrize("g_dtype", ["bf16", "fp32"])
+def test_launch_count_before_the_first_step(prec, shapes, rank, g_dtype):
+    """Before the first step the count is that of an ALWAYS step, also where the first pass's Cholesky takes
+    two launches (ranks on both sides of 256)."""
+    import paper_2512_13728_gb300 as cd
+
+    plan = make_plan(shapes, rank, prec, g_dtype)
+    try:
+        before = plan.launches_per_step()
+        plan.step(cd.hparams(step=1))
+        torch.cuda.synchronize()
+        assert plan.device_status() == 0
+        assert plan.launches_per_step() == before
+    finally:
+        plan.close()
