@@ -336,8 +336,7 @@ size_t chol_tc_smem(int32_t max_r) {
 
 cudaError_t prepare_chol_inv_tc(int32_t max_r, size_t *smem_out) {
   *smem_out = chol_tc_smem(max_r);
-  if (*smem_out > 227u * 1024u) return cudaErrorInvalidValue;
-  return cudaFuncSetAttribute(chol_inv_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem_out);
+  return allow_dynamic_smem(chol_inv_tc_kernel, *smem_out);
 }
 
 void launch_chol_inv_tc(const Shared &sh, const tc::LayerMaps *maps, size_t smem, cudaStream_t s) {

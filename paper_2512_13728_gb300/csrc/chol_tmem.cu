@@ -326,7 +326,7 @@ __global__ void __launch_bounds__(kThreads, 1) chol_inv_tmem_kernel(Shared sh) {
 
 cudaError_t prepare_chol_inv_tmem(size_t *smem_out) {
   *smem_out = 1024 + 2 * (size_t)yt_rows(kCholTmemRank) * 128 + sizeof(float) * (CB * kUld + CB * kDild) + sizeof(DiagScratch);
-  return cudaFuncSetAttribute(chol_inv_tmem_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem_out);
+  return allow_dynamic_smem(chol_inv_tmem_kernel, *smem_out);
 }
 
 void launch_chol_inv_tmem(const Shared &sh, size_t smem, cudaStream_t s) {

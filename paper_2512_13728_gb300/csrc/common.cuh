@@ -182,6 +182,22 @@ inline void launch_chained(void (*kernel)(P...), int grid, int block, size_t sme
   cudaLaunchKernelEx(&cfg, kernel, P(args)...);
 }
 
+// Lets `kernel` be launched with `smem` bytes of dynamic shared memory.  The attribute belongs to the
+// kernel and not to a plan: it is always set to all that fits beside the kernel's static shared
+// memory, as a plan of a smaller rank would otherwise take a larger one's launches away.
+template <class... P>
+inline cudaError_t allow_dynamic_smem(void (*kernel)(P...), size_t smem) {
+  cudaFuncAttributes fa{};
+  int dev = 0, most = 0;
+  cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
+  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e != cudaSuccess) return e;
+  most -= (int)fa.sharedSizeBytes;
+  if (smem > (size_t)most) return cudaErrorInvalidValue;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+}
+
 __device__ __forceinline__ void set_status(int32_t *st, int32_t code) { atomicCAS(st, 0, code); }
 
 __device__ __forceinline__ float bf16_bits_to_float(uint32_t bits16) {

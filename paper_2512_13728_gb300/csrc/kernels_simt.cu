@@ -966,7 +966,7 @@ cudaError_t prepare_chol_inv(int32_t max_r, size_t *smem_out) {
   const int ldy = (max_r + 7) / 8 * 8;
   const size_t smem = sizeof(DiagScratch) + sizeof(float) * (CB * CB + (size_t)CB * std::max(ldy, 8));
   *smem_out = smem;
-  return cudaFuncSetAttribute(chol_inv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  return allow_dynamic_smem(chol_inv_kernel, smem);
 }
 
 void launch_chol_inv(const Shared &sh, size_t smem, int32_t pass, float near_identity, cudaStream_t s) {

@@ -764,20 +764,14 @@ uint32_t fused_bq_qring(uint32_t bq_boxes) { return std::max(fb_qstages(bq_boxes
 uint32_t fused_bq_smem(uint32_t bq_boxes) { return 1024u + FB_Q_OFF + fused_bq_qring(bq_boxes) + 512u; }
 
 cudaError_t setup_bq_kernels(uint32_t f_smem, uint32_t r_smem, bool x3) {
-  cudaError_t e = x3 ? cudaFuncSetAttribute(tc_tma_gemm_kernel<GEMM_BQ, true>,
-                                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f_smem)
-                     : cudaFuncSetAttribute(tc_tma_gemm_kernel<GEMM_BQ, false>,
-                                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f_smem);
+  cudaError_t e = allow_dynamic_smem(x3 ? tc_tma_gemm_kernel<GEMM_BQ, true> : tc_tma_gemm_kernel<GEMM_BQ, false>, f_smem);
   if (e == cudaSuccess)
-    e = x3 ? cudaFuncSetAttribute(tc_tma_gemm_kernel<GEMM_BTP, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)r_smem)
-           : cudaFuncSetAttribute(tc_tma_gemm_kernel<GEMM_BTP, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)r_smem);
+    e = allow_dynamic_smem(x3 ? tc_tma_gemm_kernel<GEMM_BTP, true> : tc_tma_gemm_kernel<GEMM_BTP, false>, r_smem);
   return e;
 }
 
 cudaError_t setup_fused_bq_kernel(uint32_t smem) {
-  return cudaFuncSetAttribute(tc_form_bq_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  return allow_dynamic_smem(tc_form_bq_kernel, smem);
 }
 
 void launch_fused_bq(const Shared &sh, const TcPlan &tp, bool gated, cudaStream_t s) {

@@ -541,13 +541,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(X3 ? O_THREADS_X3 : 
 uint32_t orth_smem(int nstages, uint32_t stage_bytes) { return 1024u + nstages * stage_bytes + 4u * O_BOX + 512u; }
 
 cudaError_t setup_orth_kernels(uint32_t smem, bool x3) {
-  const int sm = (int)smem;
-  const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  cudaError_t e = x3 ? cudaFuncSetAttribute(tc_orth_kernel<ORTH_GRAM, true>, at, sm)
-                     : cudaFuncSetAttribute(tc_orth_kernel<ORTH_GRAM, false>, at, sm);
-  if (e == cudaSuccess)
-    e = x3 ? cudaFuncSetAttribute(tc_orth_kernel<ORTH_TRSM, true>, at, sm)
-           : cudaFuncSetAttribute(tc_orth_kernel<ORTH_TRSM, false>, at, sm);
+  cudaError_t e = allow_dynamic_smem(x3 ? tc_orth_kernel<ORTH_GRAM, true> : tc_orth_kernel<ORTH_GRAM, false>, smem);
+  if (e == cudaSuccess) e = allow_dynamic_smem(x3 ? tc_orth_kernel<ORTH_TRSM, true> : tc_orth_kernel<ORTH_TRSM, false>, smem);
   return e;
 }
 

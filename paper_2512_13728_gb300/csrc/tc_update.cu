@@ -349,8 +349,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(U_THREADS, 1)
 // ========================================================================= launch ===
 template <bool X3, bool GIN, bool DEEP>
 cudaError_t setup() {
-  return cudaFuncSetAttribute(tc_update_kernel<X3, GIN, DEEP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)UpdCfg<X3, GIN, DEEP>::SMEM);
+  return allow_dynamic_smem(tc_update_kernel<X3, GIN, DEEP>, UpdCfg<X3, GIN, DEEP>::SMEM);
 }
 cudaError_t setup_update_kernel(bool x3) {
   if (x3) return setup<true, false, false>();

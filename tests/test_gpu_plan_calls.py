@@ -77,3 +77,21 @@ def test_launch_count_before_the_first_step(prec, shapes, rank, g_dtype):
         assert plan.launches_per_step() == before
     finally:
         plan.close()
+
+
+@pytest.mark.parametrize("prec,rank", [("fp32", 500), ("bf16", 500), ("bf16", 256), ("bf16x3", 256)])
+def test_a_plan_of_smaller_rank_leaves_others_usable(prec, rank):
+    """Two plans in one process: creating the second, of a smaller rank, takes nothing from the first."""
+    import paper_2512_13728_gb300 as cd
+
+    shapes = [(600, 520), (520, 600)]
+    a = make_plan(shapes, rank, prec)
+    b = make_plan(shapes, 8, prec)
+    try:
+        for plan in (a, b, a):
+            plan.step(cd.hparams(step=1))
+            torch.cuda.synchronize()
+            assert plan.device_status() == 0
+    finally:
+        a.close()
+        b.close()
