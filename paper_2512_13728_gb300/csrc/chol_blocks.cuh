@@ -1,5 +1,5 @@
 // 32 x 32 diagonal-block building blocks of the Cholesky + L^{-1} kernels (kernels_simt.cu:
-// FFMA sweep; chol_tc.cu: sweep with the trailing update on tensor cores).
+// FFMA sweep; chol_tmem.cu and chol_tc.cu: sweeps with the trailing update on tensor cores).
 #pragma once
 
 #include <cstdint>

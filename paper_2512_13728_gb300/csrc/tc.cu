@@ -1,6 +1,6 @@
 // Tensor-core path of the CurvaDion step (DION_PREC_BF16, DION_PREC_BF16X3): plan layout, tensor
 // maps and the step's launch sequence.  The kernels are in tc_update.cu (error feedback +
-// parameter update), tc_bq.cu, tc_orth.cu and chol_tc.cu.
+// parameter update), tc_bq.cu, tc_orth.cu, chol_tmem.cu and chol_tc.cu.
 #include "tc.cuh"
 #include "tc_common.cuh"
 #include "tc_kernels.cuh"
@@ -191,14 +191,12 @@ dion_status layout(const dion_layer *layers, int32_t L, int32_t precision, int n
     sc->o_off = take(sizeof(int) * sc->off.size());
   }
   lo.o_maps = take(sizeof(LayerMaps) * std::max(L, 1), 128);
-  lo.o_utiles = take(sizeof(int4) * std::max<size_t>(lo.utiles.size(), 1));
   lo.o_rtiles = take(sizeof(int4) * std::max<size_t>(lo.rtiles.size(), 1));
   lo.o_qtiles = take(sizeof(int4) * std::max<size_t>(lo.qtiles.size(), 1));
   lo.o_ttiles = take(sizeof(int4) * std::max<size_t>(lo.trsm_tiles.size(), 1));
   lo.fuse_buffer = L > 0 && !x3;  // BF16X3 forms B and its two bf16 halves in the buffer pass
   for (int32_t l = 0; l < L; ++l) lo.fuse_buffer = lo.fuse_buffer && layers[l].g_dtype == DION_DTYPE_BF16;
   lo.end = off;
-  (void)num_sms;
   return DION_OK;
 }
 
@@ -246,8 +244,6 @@ void bind(const TcLayout &lo, char *base, DevLayer *dl, int32_t L, TcPlan *tp) {
     ++dl[l].upart_cnt;
   }
   tp->maps = reinterpret_cast<LayerMaps *>(base + lo.o_maps);
-  tp->utiles = reinterpret_cast<int4 *>(base + lo.o_utiles);
-  tp->n_utiles = (int32_t)lo.utiles.size();
   tp->rtiles = reinterpret_cast<int4 *>(base + lo.o_rtiles);
   tp->n_rtiles = (int32_t)lo.rtiles.size();
   tp->qtiles = reinterpret_cast<int4 *>(base + lo.o_qtiles);
@@ -319,7 +315,6 @@ cudaError_t init(const TcLayout &lo, char *base, const DevLayer *dl, int32_t L, 
   auto up = [&](int4 *dst, const std::vector<int4> &v) {
     return v.empty() ? cudaSuccess : cudaMemcpy(dst, v.data(), sizeof(int4) * v.size(), cudaMemcpyHostToDevice);
   };
-  if (e == cudaSuccess) e = up(tp->utiles, lo.utiles);
   if (e == cudaSuccess) e = up(tp->rtiles, lo.rtiles);
   if (e == cudaSuccess) e = up(tp->qtiles, lo.qtiles);
   if (e == cudaSuccess) e = up(tp->trsm_tiles, lo.trsm_tiles);
@@ -333,13 +328,11 @@ cudaError_t init(const TcLayout &lo, char *base, const DevLayer *dl, int32_t L, 
   // and 1 KB of column partials
   const uint32_t budget = 227u * 1024u - 1024u - 4u * 128u * 32u * 4u - 1024u - 512u - 256u;
   const bool x3 = lo.precision == DION_PREC_BF16X3;
-  const uint32_t nb64 = (uint32_t)std::max(1, (lo.max_r + 63) / 64);
   // B Q / B^T P (CTA pairs): A tile + per 256-column part of N, this CTA's half (two 64-column boxes)
   const uint32_t bq_boxes = 2u * (uint32_t)std::max(1, ((lo.max_r + 15) / 16 * 16 + 255) / 256);
   // BF16X3: the high and low halves of both operands
   const uint32_t stage = (x3 ? 2u : 1u) * (128u * 64u * 2u + bq_boxes * 64u * 64u * 2u);
   const int stages = (int)std::min<uint32_t>(4u, budget / stage);
-  const uint32_t nb128 = (uint32_t)std::max(1, (lo.max_r + 127) / 128);
   // Gram / TRSM (CTA pairs): A box + per 256-column part of N, this CTA's half (one 128-row box)
   const uint32_t o_parts = (uint32_t)std::max(1, ((lo.max_r + 15) / 16 * 16 + 255) / 256);
   // BF16X3: every stage also holds the lo boxes its converters write
@@ -351,9 +344,7 @@ cudaError_t init(const TcLayout &lo, char *base, const DevLayer *dl, int32_t L, 
   const uint32_t tstage = (x3 ? 2u : 1u) * 128u * 32u * 4u * 2u;
   const int tstages = (int)std::min<uint32_t>(5u, budget / tstage);
   if (stages < 2 || ostages < 2 || tstages < 2) return cudaErrorInvalidValue;
-  tp->nb64 = nb64;
   tp->bq_boxes = bq_boxes;
-  tp->nb128 = nb128;
   tp->o_parts = o_parts;
   tp->f_stages = tp->r_stages = stages;
   tp->o_stages = ostages;
@@ -374,10 +365,6 @@ cudaError_t init(const TcLayout &lo, char *base, const DevLayer *dl, int32_t L, 
   for (int32_t l = 0; l < L; ++l) tp->min_r = std::min<int32_t>(tp->min_r, (int32_t)dl[l].r);
   if (e == cudaSuccess) e = prepare_chol_inv_tc(lo.max_r, &tp->chol_tc_smem);
   if (e == cudaSuccess) e = prepare_chol_inv_tmem(&tp->chol_tmem_smem);
-  int dev = 0, sms = 0;
-  if (e == cudaSuccess) e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  tp->num_sms = sms;
   // of an ALWAYS step; BF16X3: the split of B; ranks on both sides of 256: two first-pass Cholesky kernels
   tp->launches = (tp->fuse_buffer ? 16 : x3 ? 18 : 17) + (tp->min_r <= kCholTmemRank && tp->max_r > kCholTmemRank);
   return e;
@@ -439,7 +426,7 @@ void step(dion_plan *p, const TcPlan &tp, const Shared &sh_in, const StepArgs &a
     launch_orth(sh, tp, true, pass, s);  // S = X^T X
     tick(p, s, kGram[pass]);
     if (pass == 0) {
-      launch_chol_first(p, sh, tp, s);  // trailing update on tensor cores (3xTF32)
+      launch_chol_first(p, sh, tp, s);  // L, L^{-1}: the update on tensor cores (3xTF32)
     } else {
       launch_chol_inv(sh, chol_smem, pass, x3 ? 1e-3f : 6e-2f, s);  // usually the first-order factor
       tick(p, s, kChol[pass]);

@@ -57,13 +57,14 @@ struct TcLayout {
   Schedule s_update, s_bq, s_btp, s_gram, s_trsm;
   size_t end = 0;
   size_t o_maps = 0;
-  size_t o_utiles = 0, o_rtiles = 0, o_qtiles = 0, o_ttiles = 0;
+  size_t o_rtiles = 0, o_qtiles = 0, o_ttiles = 0;
   std::vector<size_t> o_phi, o_rhi, o_qnhi, o_bh, o_ptraw, o_pt, o_colsq, o_colinv;
   std::vector<size_t> o_bl, o_plo, o_rlo, o_qnlo;  // BF16X3 low halves
   std::vector<uint64_t> guards;  // offsets of the guard words after each region
   std::vector<int4> gram_tiles, trsm_tiles;
-  // update tiles {layer, m-block, n-block, slot}; P-convert tiles {layer, row0, rows, 0};
-  // B Q tiles {layer, m-block, 0, slot}; B^T P tiles {layer, n-block, 0, 0}; Q-copy tiles
+  // update tiles {layer, m-block, n-block, slot} (host only: the schedule's pairs and the norm slots
+  // come from them); B Q tiles {layer, m-block, 0, 0}; B^T P tiles {layer, n-block, 0, 0}; Q-copy
+  // tiles {layer, first row, rows, 0}
   std::vector<int4> utiles, ftiles, rtiles, qtiles;
   int32_t precision = 0;
   int32_t max_r = 0;
@@ -80,8 +81,6 @@ struct DevSchedule {
 struct TcPlan {
   DevSchedule d_update, d_bq, d_btp, d_gram, d_trsm;
   LayerMaps *maps = nullptr;
-  int4 *utiles = nullptr;
-  int32_t n_utiles = 0;
   int4 *rtiles = nullptr;
   int32_t n_rtiles = 0;
   int4 *qtiles = nullptr;
@@ -90,8 +89,7 @@ struct TcPlan {
   int32_t n_trsm_tiles = 0;
   int32_t max_r = 0;
   int32_t f_stages = 0, r_stages = 0, o_stages = 0, t_stages = 0;  // t: the TRSM's (A + one B box per stage)
-  uint32_t f_smem = 0, r_smem = 0, o_smem = 0, nb64 = 0, nb128 = 0, bq_boxes = 0, o_parts = 0, tmem_cols = 0;
-  int32_t num_sms = 0;
+  uint32_t f_smem = 0, r_smem = 0, o_smem = 0, bq_boxes = 0, o_parts = 0, tmem_cols = 0;
   int32_t precision = 0;
   int32_t launches = 0;
   bool fuse_buffer = false;
@@ -123,7 +121,5 @@ void destroy(TcPlan *tp);
 // Re-derives the bf16 copy of every layer's Q from the caller's fp32 Q (plan creation and
 // dion_plan_refresh).
 void refresh(const TcPlan &tp, const Shared &sh, cudaStream_t s);
-// Number of B Q tiles (one norm-partial slot each) the layout needs for these layers.
-
 }  // namespace tc
 }  // namespace cd
