@@ -656,15 +656,16 @@ def test_gram_row_ranges(rank, prec, tol):
 @pytest.mark.parametrize("shapes,rank", [([(31, 33), (33, 31)], 5), ([(64, 520), (520, 64)], 33), ([(1030, 40)], 40),
                                          ([(700, 650), (650, 700)], 129)])
 def test_fp32_small_gemm_tiles(shapes, rank):
-    """The 32 x 32-tile fp32 GEMM (small plans): partial tiles both ways, K shorter than the warps'
-    chunks, not a multiple of them, and long, ranks past one and several tiles."""
+    """The 32 x 32-tile fp32 GEMM (small plans; the smallest here, and some solves, are so short that the
+    128 x 128 one is taken): partial tiles both ways, K shorter than the warps' chunks, not a multiple
+    of them, and long, ranks past one and several tiles."""
     w = wl.scaled(wl.WORKLOADS["gpt160m_block_r192"], "smallgemm", shapes, rank=rank, steps=2)
     run_per_step(w, PRECS["fp32"], dict(gate_mode=oc.GATE_ALWAYS), w.steps, TOL_FP32)
 
 
 def test_fp32_large_gemm_tiles():
-    """A plan whose B Q, B^T P and solves take the 128 x 128-tile fp32 GEMM (the small plans of the
-    other tests take the 32 x 32 one), with partial tiles."""
+    """A plan whose B Q, B^T P and solves take the 128 x 128-tile fp32 GEMM over several waves of tiles
+    (most plans of the other tests take the 32 x 32 one), with partial tiles."""
     w = wl.scaled(wl.WORKLOADS["gpt160m_block_r192"], "largegemm", [(1100, 1030)] * 14, rank=250, steps=1)
     run_per_step(w, PRECS["fp32"], dict(gate_mode=oc.GATE_ALWAYS), w.steps, TOL_FP32)
 
