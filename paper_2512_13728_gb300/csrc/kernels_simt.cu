@@ -777,11 +777,12 @@ __device__ __noinline__ float power_norm_sym(const float *S, int r, int64_t ls, 
       float a[32], colsum = 0.f;
 #pragma unroll
       for (int y = 0; y < 32; ++y) {
-        const int row = bi * 32 + y;
-        float e = 0.f;
-        if (row < r && c <= row) e = S[(int64_t)row * ls + c] - (row == c ? 1.f : 0.f);
+        // every lane loads (an entry of the triangle), so that the 32 loads go out together
+        const int row = bi * 32 + y, lr = min(row, r - 1);
+        const float s = S[(int64_t)lr * ls + min(c, lr)];
+        const float e = (row < r && c <= row) ? s - (row == c ? 1.f : 0.f) : 0.f;
         a[y] = e * vc;
-        if (c != row) colsum = fmaf(e, (row < r) ? pv[row] : 0.f, colsum);
+        colsum = fmaf(row == c ? 0.f : e, pv[lr], colsum);
       }
       // reduce-scatter: lane y ends with sum over the lanes of a[y] (row y of the tile)
 #pragma unroll
